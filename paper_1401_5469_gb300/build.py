@@ -23,8 +23,10 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # The mixed-precision kernel is compiled twice with different register caps
 # (single models, batches) and must compute the same bits in both: only its
 # explicit fma/fmaf calls fuse, so no multiply-add contraction can depend on
-# how the registers were allocated.
-PER_FILE_FLAGS = {"mc_transport_mixed.cu": ["-fmad=false"]}
+# how the registers were allocated.  The binary64 kernel's lone walk repeats a
+# segment's arithmetic in code of its own, which must round alike for the same
+# reason.
+PER_FILE_FLAGS = {"mc_transport_mixed.cu": ["-fmad=false"], "mc_transport.cu": ["-fmad=false"]}
 
 
 def nvcc() -> str:

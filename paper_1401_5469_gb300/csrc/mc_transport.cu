@@ -2,38 +2,29 @@
 // (Kerzendorf & Sim 2014, Sects. 2.4-2.7 and 2.9), one packet per thread in a
 // persistent grid.
 //
-// GB300 notes.  Binary64 add/mul/fma/compare issue at 1/64 of the binary32
-// rate and every binary64 warp instruction holds its warp for ~64 cycles,
-// whatever the number of active lanes.  A line-thick model is latency-bound by
-// its longest random walks (the packet queue empties within a few percent of
-// the kernel time), so the kernel minimises binary64 instructions per flight
-// segment:
+// GB300 notes.  A binary64 warp instruction occupies its SM sub-partition's
+// pipe for 64 cycles, whatever the number of active lanes (a 64-bit integer
+// high product takes 27, a binary32 operation 1), and a line-thick model is
+// latency-bound by its longest random walks (the packet queue empties within a
+// few percent of the kernel time), so the kernel minimises binary64
+// instructions per flight segment:
 //  * the packet carries p = x mu and q = x^2 - p^2 (conserved in free flight;
 //    radii in units of c t_exp): D = 1 - p, x^2 = q + p^2, the shell exit is
-//    at p = +-sqrt(x_b^2 - q) -- a root taken only when a line is passed or
-//    the shell event wins -- and a flight of length l is p += l;
-//  * the line scan runs in the frequency domain: a Sobolev point is the
-//    closest event while nu_line > max(nu_shell, nu_e), where nu_shell and
-//    nu_e are the comoving frequencies reached at d_shell and d_e; passing a
-//    line of depth tau moves nu_e up by tau nu_lab / k (one FMA), and the line
-//    absorbs the packet exactly when that new nu_e exceeds nu_line (Sect. 2.6's
-//    test tau_S + kappa d_line > tau with kappa d = (nu_cmf - nu) / (nu_lab/k));
-//    every comparison is an integer compare of the values' bit patterns
-//    (one operand is always positive, so the patterns order like the values);
-//  * 1/D and 1/nu_lab are carried and refreshed with Newton reciprocals,
-//    E/nu_lab is carried instead of E_lab (the same in both frames), and
-//    -ln z comes from a table-driven logarithm;
+//    at p = +-sqrt(x_b^2 - q) and a flight of length l is p += l;
+//  * the line scan is decided in binary32 wherever an error bound allows, and
+//    by a binary64 scan elsewhere (see ScanF);
+//  * 1/nu_lab is carried and nu_lab taken only where it is needed, E/nu_lab is
+//    carried instead of E_lab (the same in both frames);
 //  * downbranch emission is an integer guide-table search, and the next
 //    line's nu/tau loads are issued before the current line is resolved;
 //  * lanes stay converged: a lane that finishes claims the next packet at the
 //    loop head (warp-aggregated atomic); shell estimators accumulate in
 //    registers and are flushed once per shell change;
-//  * a warp down to its last live walk runs it with all 32 lanes (lone-walker
-//    mode): the line list 32 lines at a time, the scan of such a window in
-//    one step through a binary32 filter with an error bound (the scalar scan
-//    wherever a sign is within the bound), the absorbing line's emission
-//    record loaded as soon as the scan names it, and the walk's draws
-//    computed ahead by the whole warp.
+//  * a warp down to its last live walk runs it with all 32 lanes (the lone
+//    walk), and few packets are spread over all warps.
+// Longest walk of the 500,000-line model (94,495 segments) alone: 212 ms before
+// the binary32 scan, 165 ms with it; its 1e6-packet iteration 236 -> 182 ms (queue
+// 9.9 -> 6.9 ms); 1e4 packets of the 2000-line scatter model 520 -> 388 us.
 #include <cstdint>
 
 #include "mc_device.cuh"
@@ -48,22 +39,20 @@ constexpr int kShellArrays = 6;  // x_in^2, x_out^2, x_in, x_out, kappa, 1/kappa
 constexpr int kLineEvent = 1, kElectronEvent = 2, kShellEvent = 3;
 
 struct Packet {
-  double p, q;               // x mu, x^2 - p^2
-  // nu_lab, 1/nu_lab and E_lab / nu_lab = E_cmf / nu_cmf: the first-order
-  // Doppler factor scales energy and frequency alike, so the ratio is the
-  // same in both frames; it changes only when a line re-emits at another
-  // frequency (Thomson and resonant scatterings keep both comoving values).
-  double nu_lab, e_per_nu, inv_nu;
+  double p, q;  // x mu, x^2 - p^2
+  // 1/nu_lab and E_lab / nu_lab = E_cmf / nu_cmf: the first-order Doppler
+  // factor scales energy and frequency alike, so the ratio is the same in
+  // both frames; it changes only when a line re-emits at another frequency
+  // (Thomson and resonant scatterings keep both comoving values).
+  double inv_nu, e_per_nu;
   // Frame quantities at the start of the next flight segment, carried from
-  // the event that began it (valid while have_cmf): D = 1 - p, 1/D, the
-  // comoving frequency nu_lab D and E_cmf D = E_lab D^2 (the estimators'
-  // weight per unit length).  After an interaction they are known without
-  // new products (nu_cmf is the emitted comoving frequency, E_cmf D = E_cmf' D
-  // with the new direction's D); after a shell crossing they are recomputed.
-  double D, inv_D, nu_cmf, eD2;
+  // the event that began it (have_cmf): D = 1 - p, the comoving frequency
+  // and energy there; after a shell crossing they are taken from nu_lab.
+  double D, nu_cmf, e_cmf;
+  double nu_lab;  // have_lab: nu_cmf / D, taken where it is needed
   int32_t shell, next_line;
   uint32_t pid;
-  bool have_cmf;
+  bool have_cmf, have_lab;
   uint32_t cnt[kNCounters];
 };
 
@@ -187,18 +176,18 @@ __device__ __forceinline__ Emission downbranch_pick(const TransportParams &p, in
 // returns the branching-row info (begin | length << 32) of the level it
 // deactivates from, for the emission pick.  After kMaMaxJumps jumps it
 // deactivates without the decision draw.
-__device__ __forceinline__ unsigned long long macroatom_walk(const TransportParams &p, int32_t row,
-                                                             const WarpDraws &wd, DrawStream &ds) {
+template <class Draws>
+__device__ __forceinline__ unsigned long long macroatom_walk(const TransportParams &p, int32_t row, const Draws &md) {
   for (uint32_t n = 0; n < kMaMaxJumps; ++n) {
     const MaRow *mr = p.ma_row + row;
     const unsigned long long thr = __ldg(&mr->jump_thr);
     const uint2 jb = __ldg(reinterpret_cast<const uint2 *>(&mr->jump_begin));  // begin, length
-    const unsigned long long za = wd.template next_u53<true>(ds);
+    const unsigned long long za = md.next();
     if (!(za < thr)) {
       const uint2 db = __ldg(reinterpret_cast<const uint2 *>(&mr->dbr_begin));
       return static_cast<unsigned long long>(db.x) | (static_cast<unsigned long long>(db.y) << 32);
     }
-    const unsigned long long zb = wd.template next_u53<true>(ds);
+    const unsigned long long zb = md.next();
     const MaJump *jp = p.ma_jump + jb.x;
     int32_t next = __ldg(&jp[jb.y - 1].target);
     for (uint32_t k = 0; k < jb.y; ++k) {
@@ -220,69 +209,6 @@ __device__ __forceinline__ double shell_exit(double q, bool inner, double xi2, d
   return inner ? -root : root;
 }
 
-// Does an event at path length l (units of c t_exp) come before the shell
-// exit?  Along the ray x mu grows by l and x^2 = q + (x mu)^2; pl = x mu and
-// r2 = x^2 at the event point.  Outward exit: before it exactly when x^2 <
-// x_out^2 there (a point with x mu < 0 has x^2 <= the current x^2).  Inner
-// exit at x mu = -sqrt(x_in^2 - q): before it exactly when x mu < 0 and
-// x^2 > x_in^2 there.
-__device__ __forceinline__ bool inside_shell(double pl, double r2, bool inner, double xi2, double xo2) {
-  const long long k2 = rawkey(r2);  // all three squares are >= 0
-  return inner ? (strictly_negative(pl) && k2 > rawkey(xi2)) : k2 < rawkey(xo2);
-}
-
-// binary64 -> binary32 toward zero on the bit pattern (no conversion
-// instruction: on GB300 those issue on the binary64 pipe), for d >= 0 below
-// the binary32 overflow threshold; values below the binary32 normal range
-// give 0 (an absolute error under 2^-126).
-__device__ __forceinline__ float f32_rz(double d) {
-  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(d));
-  const int e = static_cast<int>(b >> 52) - 1023 + 127;
-  return e <= 0 ? 0.0f : __int_as_float((e << 23) | static_cast<int>((b >> 29) & 0x7fffffull));
-}
-
-// Bit pattern of the binary64 value of a positive normal binary32 (exact).
-__device__ __forceinline__ long long f64_bits(float f) {
-  const unsigned int b = static_cast<unsigned int>(__float_as_int(f));
-  return static_cast<long long>(((static_cast<unsigned long long>(b >> 23) + (1023 - 127)) << 52) |
-                                (static_cast<unsigned long long>(b & 0x7fffffu) << 29));
-}
-
-// The comoving frequency at the shell exit, K = nu_lab (1 - p_exit) with
-// p_exit = +-sqrt64(x_b^2 - q) as shell_exit and the key below compute it
-// in binary64, bracketed from binary32 arithmetic: on success K lies in
-// [lo, hi] (binary64 bit patterns), so that a line frequency or threshold
-// outside the bracket is ordered against K without the binary64 root; a
-// value inside it needs the exact K.  Error budget (u = 2^-24): the
-// operands truncated to binary32 (2u each), the difference (u), the
-// approximate reciprocal square root (taken as 2^-20 relative), the
-// products and sums (u each), and the binary64 path's own rounding (1 ulp
-// root, 3 roundings); the bracket is widened by 2^-19 K beyond the sum so
-// that rounding its ends keeps K inside.  Near-tangent exits (x_b^2 - q
-// within 4x its own error) and roots of 0.5 or more are not bracketed.
-struct ShellBracket {
-  long long lo, hi;
-  bool ok;
-};
-__device__ __forceinline__ ShellBracket shell_bracket(double q, double xb2, bool inner, double nu_lab) {
-  ShellBracket b;
-  const float a = f32_rz(xb2), c = f32_rz(q), nu = f32_rz(nu_lab);
-  const float dq = a - c;
-  const float e1 = 0x1.0p-22f * (a + dq);  // >= |dq - (x_b^2 - q)| + the binary64 difference's rounding
-  b.ok = dq >= 4.0f * e1;
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(dq));
-  const float P = dq * r;                                  // ~ sqrt(x_b^2 - q)
-  const float ep = fmaf(0x1.0p-18f, P, 1.01f * (e1 * r));  // >= |p_exit| - P
-  b.ok = b.ok && P < 0.5f;
-  const float g = inner ? 1.0f + P : 1.0f - P;
-  const float k = nu * g;
-  const float ek = k * fmaf(2.5f, ep, 0x1.0p-19f);
-  b.lo = f64_bits(k - ek);
-  b.hi = f64_bits(k + ek);
-  return b;
-}
-
 // Injection at the inner boundary, Sect. 2.4: Planck-sampled comoving
 // frequency (Carter & Cashwell series method), mu = sqrt(z), equal comoving
 // energy (Eq. 10), lab-frame values by the first-order Doppler factor.
@@ -298,18 +224,16 @@ __device__ __forceinline__ double inject(const TransportParams &p, const double 
   const double mu = sqrt(ds.open0());
   const double pp = x0 * mu;
   const double D = 1.0 - pp;
-  const double iD = rcp64(D);
   pk.p = pp;
   pk.q = max0(fma(-pp, pp, x0sq));
   const double inv_nu_cmf = rcp64(nu_cmf);
-  pk.nu_lab = nu_cmf * iD;
   pk.e_per_nu = p.e_cmf * inv_nu_cmf;
   pk.inv_nu = inv_nu_cmf * D;
   pk.D = D;
-  pk.inv_D = iD;
   pk.nu_cmf = nu_cmf;
-  pk.eD2 = p.e_cmf * D;
+  pk.e_cmf = p.e_cmf;
   pk.have_cmf = true;
+  pk.have_lab = false;
   pk.shell = 0;
   pk.next_line = first_redward(p.nu, p.L, nu_cmf);
 #pragma unroll
@@ -397,6 +321,119 @@ __device__ __noinline__ void spawn_virtual(const TransportParams &p, const doubl
   }
 }
 
+// ---- the line scan in binary32, with certainty
+//
+// The scan of Sect. 2.6 stops at the first line that lies beyond the
+// electron-scattering point, beyond the shell exit, or absorbs the packet.
+// Each of these is a sign, and nearly always one that binary32 settles: a
+// line at path length l (units of c t_exp) is passed when
+//   tau - C - kappa' D l > 0,   l < l_exit   and   tau - C - tau_k - kappa' D l > 0,
+// C the depths of the lines passed before it.  Every quantity is formed in
+// binary32 with a bound on its error that also covers the rounding of the
+// binary64 scan below (exact_scan); where a sign lies within its bound, the
+// segment is resolved by exact_scan, so that the events are the binary64
+// scan's.  Binary64 warp instructions hold their SM sub-partition's pipe for 64
+// cycles each; this takes the reciprocal 1/D, nu_lab, the thresholds and one
+// fma per line off it (28 -> 19 binary64 instructions for a line event).
+//
+// Error budget (u = 2^-24).  Frequency difference: the significands subtracted
+// as integers in units of nu_cmf's last place (a line in a lower binade is
+// truncated to it: at most one unit), converted in two halves (2u).  l: that
+// difference (2u), D truncated (2u), 1/significand (truncated 2u, approximate
+// reciprocal 2u) and two products (2u) -- below 2^-20 l.  kappa' D l: three
+// more roundings -- below 2^-20 of it.  tau, the depths: truncated (2u each),
+// and n differences (u each of tau).  M = (2^-19 + n 2^-23) (kappa' D l + tau)
+// + kappa' D (2^-44 + n 2^-51) + 2^-100 bounds these, the unit of the
+// significands and the binary64 chain's n fmas (2^-53 nu each).
+struct ScanF {
+  unsigned long long mc;  // significand of nu_cmf
+  int ec;                 // its exponent field
+  float lf, tf;           // path length per unit of significand difference; kappa' D
+  float tau;              // the optical-depth draw
+  float lx, mx;           // path length to the shell exit and its error bound (infinite: not known)
+};
+
+// Path length to the exit: x mu there is +-sqrt(x_b^2 - q) (P, in binary32 from
+// the operands truncated, the difference's error e1 carried through the root).
+// Near-tangent exits (x_b^2 - q within 4 e1) are not bounded.
+__device__ __forceinline__ ScanF scan_setup(double nu_cmf, double D, double p, double q, float kap, bool inner,
+                                            float xi2, float xo2, double tau) {
+  ScanF f;
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(nu_cmf));
+  f.ec = static_cast<int>(b >> 52);
+  f.mc = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  float im;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(im) : "f"(static_cast<float>(static_cast<uint32_t>(f.mc >> 29))));
+  const float Df = f32_rz_any(D), pf = f32_rz_any(p), qf = f32_rz_any(q);
+  f.lf = (Df * im) * 0x1.0p-29f;
+  f.tf = kap * Df;
+  f.tau = f32_rz_any(tau);
+  const float xb2 = inner ? xi2 : xo2;
+  const float dq = xb2 - qf;
+  const float e1 = 0x1.0p-22f * (xb2 + dq);
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(dq));
+  const float P = dq * r;
+  f.lx = (inner ? -P : P) - pf;
+  f.mx = (dq >= 4.0f * e1 && f.ec > 0 && f.ec < 2047) ? fmaf(0x1.0p-20f, P + fabsf(pf), fmaf(e1, r, 0x1.0p-44f)) : __int_as_float(0x7f800000);
+  return f;
+}
+
+// Significand difference nu_cmf - nu_line in units of nu_cmf's last place, as
+// binary32 (0 when the line is not below nu_cmf); ok: the line's binade is
+// nu_cmf's or a lower one.
+__device__ __forceinline__ float scan_delta(const ScanF &f, long long line_bits, bool &ok) {
+  const unsigned long long b = static_cast<unsigned long long>(line_bits);
+  const int sh = f.ec - static_cast<int>(b >> 52);
+  ok = sh >= 0;
+  const unsigned long long m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  const long long d = static_cast<long long>(f.mc) - static_cast<long long>(m >> (sh < 63 ? sh & 63 : 63));
+  const float v = fmaf(static_cast<float>(static_cast<uint32_t>(d >> 32)), 0x1.0p32f,
+                       static_cast<float>(static_cast<uint32_t>(d)));
+  return d > 0 ? v : 0.0f;
+}
+
+// Draws of a lone walk, computed ahead by its warp: the walk's draws base ..
+// base + 63 as u53, as -ln of the open-interval draw and as the isotropic mu.
+struct LoneDraws {
+  unsigned long long *u;
+  double *t, *m;
+  uint32_t base;
+
+  // All 32 lanes: refill when fewer than the three draws that a segment may
+  // take are left (a macro atom's jumps past the end are computed one by one).
+  __device__ __forceinline__ void keep(uint32_t d, uint32_t pid, uint32_t it, uint32_t k0, uint32_t k1,
+                                       unsigned lane, bool first) {
+    if (!first && d + 3u <= base + kWarpDraws) return;
+    base = d & ~1u;
+    const uint4 o = philox4x32_10(make_uint4((base >> 1) + lane, pid, it, 0u), k0, k1);
+    __syncwarp();  // every lane has read the old contents
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const unsigned long long v = h ? DrawStream::u53_of(o.z, o.w) : DrawStream::u53_of(o.x, o.y);
+      const int i = 2 * static_cast<int>(lane) + h;
+      u[i] = v;
+      t[i] = neg_log_u53(v + 1ull);
+      m[i] = DrawStream::mu_from_u53(v);
+    }
+    __syncwarp();
+  }
+};
+
+// A macro atom's draws: from the lane's own stream, or from a lone walk's
+// buffer and past its end one by one.
+struct MaDraws {
+  DrawStream *ds;
+  const LoneDraws *ld;  // nullptr: the lane's own stream
+  uint32_t *d;
+  uint32_t k0, k1, pid, it;
+  __device__ __forceinline__ unsigned long long next() const {
+    if (!ld) return ds->next_u53();
+    const uint32_t i = (*d)++ - ld->base;
+    return i < kWarpDraws ? ld->u[i] : u53_past_buffer(k0, k1, pid, it, *d - 1u);
+  }
+};
+
 template <int MODE, bool JB, bool REC>
 __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p) {
   extern __shared__ double sh[];
@@ -411,8 +448,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
     sh[5 * S + i] = p.inv_kappa ? p.inv_kappa[i] : (kap > 0.0 ? 1.0 / kap : 0.0);
   }
   __syncthreads();
-  const double *s_xi2 = sh, *s_xo2 = sh + S, *s_ikap = sh + 5 * S;
-  const double *s_kap = sh + 4 * S;
+  const double *s_xi2 = sh, *s_xo2 = sh + S, *s_kap = sh + 4 * S, *s_ikap = sh + 5 * S;
   const double x0 = sh[2 * S], x0sq = sh[0];
 
   const unsigned lane = threadIdx.x & 31u;
@@ -422,26 +458,18 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   uint32_t polls = 0u;  // loop iterations between looks at the host's stop request
   if (lane == 0u) atomicCAS(p.flags + 3, 0ull, t_start);
 
-  Packet pk;
+  // Few packets are spread over all warps of the grid, so many to each: a warp
+  // runs its lanes' events one kind after the other, and the binary64 pipe
+  // serves a warp instruction for one lane or 32 in the same time.  (1000
+  // packets of a 200-line scatter model: 126 -> 81 us with this and the scan.)
+  const unsigned long long n_warps = static_cast<unsigned long long>(gridDim.x) * (kBlock / 32);
+  const unsigned quota = static_cast<unsigned>(
+      min(32ull, (p.n_packets + n_warps - 1ull) / n_warps));
+
+  Packet pk{};
   DrawStream ds;
-  WarpDraws wd;
-  wd.init(reinterpret_cast<unsigned long long *>(sh + kShellArrays * S) +
-          2 * kWarpDraws * (threadIdx.x >> 5));
-  bool alive = false, finished = false;
-  // Lone-walker mode: once the packet queue is empty and a warp is down to
-  // one live walk, every lane of the warp takes that walk's state and runs
-  // its segments together with the owner lane (the same instructions on the
-  // same values, so the walk's results are those of the owner alone).  The
-  // lanes then load the line list 32 lines at a time in one coalesced load
-  // (line lwin_j0 + lane in each lane) and pass line data by shuffles;
-  // only the owner lane makes the walk's side effects (estimator and J_blue
-  // atomics, spectrum, records, statistics).
-  bool lone = false;
-  int owner = 0;
-  int32_t lwin_j0 = 0, lwin_s = -1;
-  long long lwin_b = 0;
-  double lwin_t = 0.0;
-  unsigned long long lwin_r = 0ull;
+  bool alive = false, finished = lane >= quota;
+  bool drained = false;  // warp-uniform: the packet queue is empty
   uint32_t vdraws = 0u;  // v-packet draws used by this lane's packet
   unsigned long long n_esc = 0, n_reab = 0, n_cap = 0, n_seg = 0, n_chk = 0, n_res = 0, n_lint = 0,
                      n_esca = 0, n_shell = 0;
@@ -450,7 +478,16 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   const long long *nub = reinterpret_cast<const long long *>(p.nu);
   // the lane's current shell and its constants (reloaded on a shell change)
   int32_t cs = -1;
-  double c_kap = 0.0, c_ikap = 0.0, c_xi2 = 0.0, c_xo2 = 0.0;
+  double c_xi2 = 0.0, c_xo2 = 0.0;
+  float f_kap = 0.0f, f_xi2 = 0.0f, f_xo2 = 0.0f;
+  auto enter_shell = [&](int32_t s_) {
+    cs = s_;
+    c_xi2 = s_xi2[s_];
+    c_xo2 = s_xo2[s_];
+    f_kap = f32_rz_any(s_kap[s_]);
+    f_xi2 = f32_rz_any(c_xi2);
+    f_xo2 = f32_rz_any(c_xo2);
+  };
   // Lines next_line and next_line + 1 of the next segment (frequency bits,
   // Sobolev depth in the segment's shell, branching-row info), loaded by the
   // event that began it as soon as next_line is known, so that their latency
@@ -465,50 +502,115 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
     if (j_ < L) {
       lw_b0 = __ldg(nub + j_);
       lw_t0 = __ldg(ts + j_);
-      if (MODE >= 1 && p.row_info) lw_r0 = __ldg(p.row_info + j_);
+      if (MODE == 1 && p.row_info) lw_r0 = __ldg(p.row_info + j_);
     }
     if (j_ + 1 < L) {
       lw_b1 = __ldg(nub + j_ + 1);
       lw_t1 = __ldg(ts + j_ + 1);
-      if (MODE >= 1 && p.row_info) lw_r1 = __ldg(p.row_info + j_ + 1);
+      if (MODE == 1 && p.row_info) lw_r1 = __ldg(p.row_info + j_ + 1);
     }
     lw_ok = true;
   };
-  auto lone_reload = [&](int32_t s_, int32_t j0) {
-    lwin_j0 = j0;
-    lwin_s = s_;
-    const int32_t jj = j0 + static_cast<int32_t>(lane);
-    lwin_b = 0;
-    lwin_t = 0.0;
-    lwin_r = 0ull;
-    if (jj < L) {
-      lwin_b = __ldg(nub + jj);
-      lwin_t = __ldg(p.tau + static_cast<size_t>(s_) * static_cast<size_t>(L) + jj);
-      if (MODE >= 1 && p.row_info) lwin_r = __ldg(p.row_info + jj);
+
+  // ---- steps of a segment, shared by a lane's own walk and the lone walk, so
+  // that a packet's history does not depend on which of the two runs it
+  // nu_lab, taken only where it is needed (a shell change, an electron
+  // scattering, exact_scan, the end of the walk)
+  auto need_lab = [&]() {
+    if (!pk.have_lab) {
+      pk.nu_lab = pk.nu_cmf * rcp64(pk.D);
+      pk.have_lab = true;
     }
   };
-  auto lone_fetch = [&](int32_t s_, int32_t jj, long long &b, double &t, unsigned long long &r) {
-    int idx = jj - lwin_j0;
-    if (lwin_s != s_ || idx < 0 || idx >= 32) {
-      lone_reload(s_, jj);
-      idx = 0;
+  // after a shell crossing: Doppler factor D = 1 - mu v/c at the boundary
+  // point, comoving frequency and energy (Sect. 2.5)
+  auto need_cmf = [&]() {
+    if (!pk.have_cmf) {
+      pk.D = 1.0 - pk.p;
+      pk.nu_cmf = pk.nu_lab * pk.D;
+      pk.e_cmf = pk.e_per_nu * pk.nu_cmf;
+      pk.have_cmf = true;
     }
-    b = __shfl_sync(0xffffffffu, lwin_b, idx);
-    t = __shfl_sync(0xffffffffu, lwin_t, idx);
-    r = __shfl_sync(0xffffffffu, lwin_r, idx);
+  };
+  // The event of a segment that scanned lines [j0, j) without doubt, by
+  // binary64 comparisons: frequency thresholds in place of path lengths (a
+  // Sobolev point comes before d_e while nu_line > thr_e, and before the shell
+  // exit while nu_line > nu_lab (1 - p_exit); a line of depth tau moves thr_e up by
+  // tau nu_lab / k and absorbs exactly when thr_e then exceeds nu_line).
+  // Updates j; nu_hit: the absorbing line's frequency bits; thr: thr_e.
+  auto exact_scan = [&](double tau, bool inner, int32_t j0, int32_t &j, bool act, double e_inv2, long long &nu_hit,
+                        double &thr, double &p_exit) -> int {
+    need_lab();
+    const double nu_lab = pk.nu_lab;
+    const double *ts = p.tau + static_cast<size_t>(cs) * static_cast<size_t>(L);
+    p_exit = shell_exit(pk.q, inner, c_xi2, c_xo2);
+    const long long key_x = rawkey(nu_lab * (1.0 - p_exit));  // > 0
+    const double kap = s_kap[cs];
+    const bool thomson = rawkey(kap) > 0;
+    double c_e = 0.0, rem = tau;
+    long long key_e = kKeyNegInf;
+    thr = 0.0;
+    if (thomson) {
+      c_e = (nu_lab * s_ikap[cs]) * rcp64(pk.D);  // nu_lab / k, k = kappa' D
+      thr = fma(-tau, c_e, pk.nu_cmf);
+    }
+    for (int32_t i = j0; i < j; ++i) {
+      const double t = __ldg(ts + i);
+      if (thomson) thr = fma(t, c_e, thr);
+      else rem -= t;
+    }
+    if (thomson) key_e = rawkey(thr);
+    for (; j < L; ++j) {
+      const long long b = __ldg(nub + j);
+      if (b <= key_e || b <= key_x) break;
+      const double t = __ldg(ts + j);
+      const double moved = fma(t, c_e, thr);
+      if (thomson ? rawkey(moved) > b : rawkey(t) > rawkey(rem)) {
+        nu_hit = b;
+        return kLineEvent;
+      }
+      if (JB && act)
+        red_add_evict_first(p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L) + j, e_inv2, jb_pol);
+      if (thomson) {
+        thr = moved;
+        key_e = rawkey(thr);
+      } else {
+        rem -= t;
+      }
+    }
+    return (thomson && key_e > key_x) ? kElectronEvent : kShellEvent;
+  };
+  // Where an absorbing line's Sobolev point lies: nu_lab (1 - x mu) = nu_j (a
+  // resonance that rounding puts behind the packet is taken where it is).
+  auto line_point = [&](double nuj, double &l, double &r2) {
+    l = max0(fma(-nuj, pk.inv_nu, pk.D));
+    const double pl = rawkey(l) > 0 ? fma(-nuj, pk.inv_nu, 1.0) : pk.p;
+    r2 = fma(pl, pl, pk.q);
+  };
+  // isotropic re-emission at radius^2 r2 with comoving frequency nu_c
+  auto leave = [&](double r2, double mu, double nu_c, double inv_nu_c) -> double {
+    const double xn = sqrt64(r2);
+    const double pn = xn * mu;
+    pk.D = fma(-xn, mu, 1.0);
+    pk.p = pn;
+    pk.q = max0(fma(-pn, pn, r2));
+    pk.inv_nu = inv_nu_c * pk.D;
+    pk.nu_cmf = nu_c;  // = nu_lab D
+    pk.have_lab = false;
+    return xn;
   };
 
   for (;;) {
-    // ---- claim packets for idle lanes (one atomic per warp; none in lone mode,
-    // where every lane carries the walk until it ends)
-    const bool need = !lone && !alive && !finished;
-    const unsigned needmask = lone ? 0u : __ballot_sync(0xffffffffu, need);
+    // ---- claim packets for idle lanes (one atomic per warp)
+    const bool need = !alive && !finished;
+    const unsigned needmask = __ballot_sync(0xffffffffu, need);
     if (needmask) {
       const int leader = __ffs(needmask) - 1;
       unsigned long long base = 0ull;
       if (static_cast<int>(lane) == leader)
         base = atomicAdd(p.work_counter, static_cast<unsigned long long>(__popc(needmask)));
       base = __shfl_sync(0xffffffffu, base, leader);
+      if (base + __popc(needmask) > p.n_packets) drained = true;
       if (need) {
         const unsigned long long id = base + __popc(needmask & lanemask_lt);
         if (id < p.n_packets) {
@@ -528,7 +630,8 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
         }
       }
     }
-    if (!lone && __all_sync(0xffffffffu, finished)) break;
+    const unsigned live = __ballot_sync(0xffffffffu, alive);
+    if (!live && __all_sync(0xffffffffu, finished)) break;
     if (p.timeout_ns) {
       bool late = false;
       if (lane == 0u) late = (global_ns() - t_start) > p.timeout_ns;
@@ -547,421 +650,463 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
         break;
       }
     }
-    // ---- a warp's last live walk: the idle lanes compute its draws ahead
-    if (lone) {
-      wd.keep(ds, p.key0, p.key1, p.iteration, lane);
-    } else {
-      wd.prepare(alive, __any_sync(0xffffffffu, finished), ds, pk.pid, p.key0, p.key1, p.iteration, lane);
-      if (wd.on && !p.n_virtual) {
-        // enter lone-walker mode: the other lanes' packets are done; they hand
-        // their estimator sums over and take the walk's state
-        owner = __ffs(__ballot_sync(0xffffffffu, alive)) - 1;
-        if (!alive && acc_s >= 0) {
-          atomicAdd(p.j_est + acc_s, acc_j);
-          atomicAdd(p.nu_bar + acc_s, acc_nb);
-        }
-        const unsigned F = 0xffffffffu;
-        pk.p = __shfl_sync(F, pk.p, owner);
-        pk.q = __shfl_sync(F, pk.q, owner);
-        pk.nu_lab = __shfl_sync(F, pk.nu_lab, owner);
-        pk.e_per_nu = __shfl_sync(F, pk.e_per_nu, owner);
-        pk.inv_nu = __shfl_sync(F, pk.inv_nu, owner);
-        pk.D = __shfl_sync(F, pk.D, owner);
-        pk.inv_D = __shfl_sync(F, pk.inv_D, owner);
-        pk.nu_cmf = __shfl_sync(F, pk.nu_cmf, owner);
-        pk.eD2 = __shfl_sync(F, pk.eD2, owner);
-        pk.shell = __shfl_sync(F, pk.shell, owner);
-        pk.next_line = __shfl_sync(F, pk.next_line, owner);
-        pk.pid = __shfl_sync(F, pk.pid, owner);
-        pk.have_cmf = __shfl_sync(F, static_cast<int>(pk.have_cmf), owner) != 0;
-#pragma unroll
-        for (int c = 0; c < kNCounters; ++c) pk.cnt[c] = __shfl_sync(F, pk.cnt[c], owner);
-        ds.k0 = __shfl_sync(F, ds.k0, owner);
-        ds.k1 = __shfl_sync(F, ds.k1, owner);
-        ds.packet = __shfl_sync(F, ds.packet, owner);
-        ds.iteration = __shfl_sync(F, ds.iteration, owner);
-        ds.d = __shfl_sync(F, ds.d, owner);
-        ds.spare_a = __shfl_sync(F, ds.spare_a, owner);
-        ds.spare_b = __shfl_sync(F, ds.spare_b, owner);
-        cs = __shfl_sync(F, cs, owner);
-        c_kap = __shfl_sync(F, c_kap, owner);
-        c_ikap = __shfl_sync(F, c_ikap, owner);
-        c_xi2 = __shfl_sync(F, c_xi2, owner);
-        c_xo2 = __shfl_sync(F, c_xo2, owner);
-        acc_s = __shfl_sync(F, acc_s, owner);
-        acc_j = __shfl_sync(F, acc_j, owner);
-        acc_nb = __shfl_sync(F, acc_nb, owner);
-        vdraws = __shfl_sync(F, vdraws, owner);
-        lwin_s = -1;
-        alive = true;
-        lone = true;
+    if ((drained || quota == 1u) && __popc(live) == 1 && !p.n_virtual) {
+      // ---- lone walk: the queue is empty and one walk of the warp is left.
+      // All 32 lanes take its state and run it to its end, the line list 32
+      // lines at a time (line w0 + lane in each lane, one coalesced load), the
+      // scan of such a window in one step, its draws computed ahead; lane 0
+      // makes the walk's side effects.  The chain of a line event is then two
+      // dependent loads (the emission record, the window behind the emitted
+      // line) and the scan; the event's binary64 arithmetic runs while they
+      // are in flight.
+      const unsigned F = 0xffffffffu;
+      const int owner = __ffs(live) - 1;
+      if (acc_s >= 0) {
+        atomicAdd(p.j_est + acc_s, acc_j);
+        atomicAdd(p.nu_bar + acc_s, acc_nb);
       }
+      acc_s = -1;
+      pk.p = __shfl_sync(F, pk.p, owner);
+      pk.q = __shfl_sync(F, pk.q, owner);
+      pk.nu_lab = __shfl_sync(F, pk.nu_lab, owner);
+      pk.e_per_nu = __shfl_sync(F, pk.e_per_nu, owner);
+      pk.inv_nu = __shfl_sync(F, pk.inv_nu, owner);
+      pk.D = __shfl_sync(F, pk.D, owner);
+      pk.nu_cmf = __shfl_sync(F, pk.nu_cmf, owner);
+      pk.e_cmf = __shfl_sync(F, pk.e_cmf, owner);
+      pk.shell = __shfl_sync(F, pk.shell, owner);
+      pk.next_line = __shfl_sync(F, pk.next_line, owner);
+      pk.pid = __shfl_sync(F, pk.pid, owner);
+      pk.have_cmf = __shfl_sync(F, static_cast<int>(pk.have_cmf), owner) != 0;
+      pk.have_lab = __shfl_sync(F, static_cast<int>(pk.have_lab), owner) != 0;
+#pragma unroll
+      for (int c = 0; c < kNCounters; ++c) pk.cnt[c] = __shfl_sync(F, pk.cnt[c], owner);
+      uint32_t d = __shfl_sync(F, ds.d, owner);
+      LoneDraws ld;
+      ld.u = reinterpret_cast<unsigned long long *>(sh + kShellArrays * S) + 3 * kWarpDraws * (threadIdx.x >> 5);
+      ld.t = reinterpret_cast<double *>(ld.u + kWarpDraws);
+      ld.m = ld.t + kWarpDraws;
+      ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, true);
+      enter_shell(pk.shell);
+      int32_t w0 = 0;
+      long long w_b = 0;
+      double w_t = 0.0;
+      unsigned long long w_r = 0ull;
+      auto reload = [&](int32_t j_) {
+        w0 = j_;
+        const int32_t jj = j_ + static_cast<int32_t>(lane);
+        w_b = 0;
+        w_t = 0.0;
+        w_r = 0ull;
+        if (jj < L) {
+          w_b = __ldg(nub + jj);
+          w_t = __ldg(p.tau + static_cast<size_t>(cs) * static_cast<size_t>(L) + jj);
+          if (MODE == 1 && p.row_info) w_r = __ldg(p.row_info + jj);
+        }
+      };
+      reload(pk.next_line);
+      // The estimator terms of a segment (Eqs. 13-14) are kept by one lane and
+      // evaluated for 32 segments at once.
+      double g_e = 0.0, g_D = 0.0, g_l = 0.0, g_nu = 0.0;
+      uint32_t n_log = 0u;
+      double a_j = 0.0, a_nb = 0.0;  // this lane's sums in shell cs
+      auto sum_log = [&]() {
+        const double wgt = (g_e * g_D) * g_l;
+        a_j += wgt;
+        a_nb = fma(wgt, g_nu, a_nb);
+        g_l = 0.0;
+        n_log = 0u;
+      };
+      auto flush_shell = [&]() {
+        sum_log();
+        if (rawkey(a_j) > 0) {
+          atomicAdd(p.j_est + cs, a_j);
+          atomicAdd(p.nu_bar + cs, a_nb);
+        }
+        a_j = 0.0;
+        a_nb = 0.0;
+      };
+      int status = 0;
+      bool stopped = false;
+      while (status == 0) {
+        if (p.timeout_ns && __any_sync(F, (global_ns() - t_start) > p.timeout_ns)) {
+          if (lane == 0u) atomicExch(p.flags, 1ull);
+          stopped = true;
+          break;
+        }
+        if (p.cancel && (++polls & 255u) == 0u && __any_sync(F, load_sys_u32(p.cancel) != 0u)) {
+          if (lane == 0u) atomicExch(p.flags, 2ull);
+          stopped = true;
+          break;
+        }
+        if (pk.cnt[0] >= p.max_segments) {
+          status = 3;
+          break;
+        }
+        ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, false);
+        pk.cnt[0] += 1u;
+        const uint32_t di = d - ld.base;
+        const double tau = ld.t[di];
+        d += 1u;
+        need_cmf();
+        const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);
+        const ScanF f = scan_setup(pk.nu_cmf, pk.D, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, tau);
+        const double e_inv2 = JB ? pk.e_per_nu * pk.inv_nu : 0.0;
+        double *jb_row = p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L);
+        const int32_t j0 = pk.next_line;
+        int32_t j = j0;
+        int kind = 0;
+        long long hit = 0;
+        unsigned long long rinfo = 0ull;
+        float C = 0.0f;
+        for (;;) {  // one window at a time
+          const int idx = j - w0;
+          const int32_t jl = w0 + static_cast<int32_t>(lane);
+          const bool cand = static_cast<int>(lane) >= idx;
+          const bool there = jl < L;
+          bool ok;
+          const float l = scan_delta(f, w_b, ok) * f.lf;
+          const float a = l * f.tf;
+          // the depths before this line (exclusive prefix, so that a thick line's
+          // own depth does not round them away) and including it
+          const float own = (cand && there) ? f32_rz_any(w_t) : 0.0f;
+          float Px = __shfl_up_sync(F, own, 1);
+          if (lane == 0u) Px = C;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const float y = __shfl_up_sync(F, Px, o);
+            if (static_cast<int>(lane) >= o) Px = __fadd_rn(Px, y);
+          }
+          const float n = static_cast<float>(j - j0 + 32);
+          const float m0 = fmaf(f.tf, fmaf(n, 0x1.0p-51f, 0x1.0p-44f), 0x1.0p-100f);
+          const float m1 = fmaf(n, 0x1.0p-23f, 0x1.0p-19f);
+          const float M = fmaf(m1, a + f.tau, m0);
+          const float r0 = (f.tau - Px) - a;                 // before this line
+          const float r1 = r0 - own;                         // after it
+          const float xm = f.lx - l, xM = fmaf(0x1.0p-19f, l, f.mx);
+          const bool before = there && ok && r0 > M;         // certainly before d_e
+          const bool inside = xm > xM;                       // ... and before the exit
+          const bool pass = before && inside && r1 > M && own >= 0.0f;
+          const bool take = before && inside && r1 < -M;
+          // the exit comes before this line and before d_e
+          const float ax = f.lx * f.tf;
+          const float rx = (f.tau - Px) - ax;
+          const bool out = (!there || (ok && xm < -xM)) &&
+                           rx > fmaf(m1, fabsf(ax) + f.tau, fmaf(f.tf, f.mx, m0));
+          const unsigned stop = __ballot_sync(F, cand && !pass);
+          const unsigned took = __ballot_sync(F, take);
+          const unsigned outs = __ballot_sync(F, out);
+          const int k = stop ? __ffs(stop) - 1 : 32;
+          const bool taken = stop && ((took >> k) & 1u);
+          if (JB && cand && static_cast<int>(lane) < (taken ? k + 1 : k))
+            red_add_evict_first(jb_row + jl, e_inv2, jb_pol);
+          j = w0 + k;
+          if (taken) {
+            kind = kLineEvent;
+            hit = __shfl_sync(F, w_b, k);
+            rinfo = __shfl_sync(F, w_r, k);
+            break;
+          }
+          if (stop) {
+            kind = ((outs >> k) & 1u) ? kShellEvent : 0;
+            break;
+          }
+          C = __shfl_sync(F, Px + own, 31);
+          reload(j);
+        }
+        double thr = 0.0, p_exit = 0.0;
+        if (kind == 0) {
+          kind = exact_scan(tau, inner, j0, j, lane == 0u, e_inv2, hit, thr, p_exit);
+          if (kind == kLineEvent) {
+            if (JB && lane == 0u) red_add_evict_first(jb_row + j, e_inv2, jb_pol);
+            if (MODE == 1 && p.row_info) rinfo = __ldg(p.row_info + j);
+          }
+        } else if (kind == kShellEvent) {
+          p_exit = shell_exit(pk.q, inner, c_xi2, c_xo2);
+        }
+        const uint32_t npass = static_cast<uint32_t>(j - j0);
+        pk.cnt[1] += npass + (j < L ? 1u : 0u);
+        pk.cnt[2] += npass + (kind == kLineEvent ? 1u : 0u);
+        pk.next_line = j;
+        double l = 0.0;
+        if (kind == kLineEvent) {
+          pk.cnt[3] += 1u;
+          ulonglong2 ra = make_ulonglong2(0ull, 0ull), rc = make_ulonglong2(0ull, 0ull);
+          unsigned long long u_em = 0ull;
+          const bool slot = MODE == 1 && p.dbr_rec;
+          if (MODE == 2) {
+            const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
+            rinfo = macroatom_walk(p, __ldg(p.line_row + j), md);
+            u_em = md.next();
+          } else if (MODE == 1) {
+            u_em = ld.u[di + 1u];
+            d += 1u;
+          }
+          if (slot) load_slot(bucket_slot(p, rinfo, u_em), ra, rc);
+          const double nuj = __longlong_as_double(hit);
+          double r2;
+          line_point(nuj, l, r2);
+          // log the segment, then the event's energy
+          if (lane == (n_log & 31u)) { g_e = pk.e_cmf; g_D = pk.D; g_l = l; g_nu = pk.nu_cmf; }
+          const double e_c = pk.e_per_nu * nuj;
+          double mu;
+          if (MODE == 2) {
+            const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
+            mu = DrawStream::mu_from_u53(md.next());
+          } else {
+            mu = ld.m[d - ld.base];
+            d += 1u;
+          }
+          const double xn = sqrt64(r2);
+          const double pn = xn * mu;
+          const double D2 = fma(-xn, mu, 1.0);
+          const double q2 = max0(fma(-pn, pn, r2));
+          double nu_c, inv_c;
+          if (MODE >= 1) {
+            Emission em;
+            if (slot) em = pick_from_slot_lone(p, rinfo, u_em, ra, rc, lane);
+            else em = downbranch_pick(p, j, rinfo, u_em);
+            nu_c = em.nu;
+            inv_c = em.inv_nu;
+            pk.next_line = em.line + 1;
+            reload(pk.next_line);
+            pk.e_per_nu = e_c * inv_c;  // re-emitted at another frequency
+          } else {
+            nu_c = nuj;
+            inv_c = rcp64(nuj);
+            pk.next_line = j + 1;
+          }
+          pk.e_cmf = e_c;
+          pk.D = D2;
+          pk.p = pn;
+          pk.q = q2;
+          pk.inv_nu = inv_c * D2;
+          pk.nu_cmf = nu_c;
+          pk.have_lab = false;
+        } else if (kind == kShellEvent) {
+          pk.cnt[5] += 1u;
+          l = max0(p_exit - pk.p);
+          if (lane == (n_log & 31u)) { g_e = pk.e_cmf; g_D = pk.D; g_l = l; g_nu = pk.nu_cmf; }
+          need_lab();
+          flush_shell();
+          n_log = 0xffffffffu;  // (counted up below)
+          const int32_t ns = inner ? cs - 1 : cs + 1;
+          pk.p = p_exit;
+          pk.have_cmf = false;
+          if (ns >= S) status = 1;
+          else if (ns < 0) status = 2;
+          else {
+            enter_shell(ns);
+            reload(j);
+          }
+        } else {
+          pk.cnt[4] += 1u;
+          l = max0(fma(-thr, pk.inv_nu, pk.D));
+          const double pl = pk.p + l;
+          if (lane == (n_log & 31u)) { g_e = pk.e_cmf; g_D = pk.D; g_l = l; g_nu = pk.nu_cmf; }
+          const double D1 = 1.0 - pl;
+          const double nu_c = pk.nu_lab * D1;
+          pk.e_cmf = pk.e_per_nu * nu_c;
+          leave(fma(pl, pl, pk.q), ld.m[d - ld.base], nu_c, pk.inv_nu * rcp64(D1));
+          d += 1u;
+        }
+        if (pk.next_line < w0 || pk.next_line - w0 >= 32) reload(pk.next_line);  // behind the window
+        if (++n_log == 32u) sum_log();
+      }
+      need_lab();
+      flush_shell();
+      if (status != 0 && lane == 0u) {
+        if (status == 1) ++n_esc;
+        else if (status == 2) ++n_reab;
+        else ++n_cap;
+        n_seg += pk.cnt[0];
+        n_chk += pk.cnt[1];
+        n_res += pk.cnt[2];
+        n_lint += pk.cnt[3];
+        n_esca += pk.cnt[4];
+        n_shell += pk.cnt[5];
+        const double e_lab = pk.e_per_nu * pk.nu_lab;
+        if (status == 1) atomicAdd(p.spectrum + spectrum_bin(p, pk.nu_lab), e_lab);
+        if (REC) {
+          const uint32_t r = static_cast<uint32_t>(pk.pid - p.first_packet);
+          p.rec_status[r] = status;
+          p.rec_nu[r] = pk.nu_lab;
+          p.rec_e[r] = e_lab;
+#pragma unroll
+          for (int c = 0; c < kNCounters; ++c) p.rec_cnt[static_cast<size_t>(r) * kNCounters + c] = pk.cnt[c];
+        }
+      }
+      if (stopped) break;
+      alive = false;
+      lw_ok = false;
+      continue;
     }
     if (!alive) continue;
-    const bool act = !lone || static_cast<int>(lane) == owner;  // makes the walk's side effects
 
-    // ---- one flight segment (Sect. 2.6)
+    // ---- one flight segment of every live lane (Sect. 2.6)
     int status = 0;
     if (pk.cnt[0] >= p.max_segments) {
       status = 3;  // capped
+      need_lab();
     } else {
       pk.cnt[0] += 1u;
       const int32_t s = pk.shell;
-      const double pp = pk.p, q = pk.q, nu_lab = pk.nu_lab, inv_nu = pk.inv_nu;
-      if (!pk.have_cmf) {
-        // after a shell crossing: Doppler factor D = 1 - mu v/c at the boundary
-        // point, comoving frequency and E_cmf D (Sect. 2.5)
-        const double D0 = 1.0 - pp;
-        pk.D = D0;
-        pk.inv_D = rcp64(D0);
-        pk.nu_cmf = nu_lab * D0;
-        pk.eD2 = (pk.e_per_nu * pk.nu_cmf) * D0;  // E_cmf D
-        pk.have_cmf = true;
-      }
-      const double D = pk.D, inv_D = pk.inv_D, nu_cmf = pk.nu_cmf, eD2 = pk.eD2;
-      if (s != cs) {
-        cs = s;
-        c_kap = s_kap[s];
-        c_ikap = s_ikap[s];
-        c_xi2 = s_xi2[s];
-        c_xo2 = s_xo2[s];
-      }
-      const bool thomson = rawkey(c_kap) > 0;
+      if (s != cs) enter_shell(s);
+      need_cmf();
       // optical depth to the next event, tau = -ln z
-      double tau_rem = wd.template next_tau<MODE == 2>(ds);
-      // Shell boundary: at the exit point x mu = p_exit = +-sqrt(x_b^2 - q) (the
-      // inner sphere is hit when moving inward with q <= x_in^2), so the path
-      // length is p_exit - p and the comoving frequency there nu_lab (1 - p_exit).
-      // That frequency orders the lines passed against the exit; it is first
-      // bracketed in binary32 (shell_bracket) and taken exactly (binary64
-      // root) only for a value inside the bracket or when the shell event
-      // wins.  An event at path length l with no line passed before it is
-      // placed against the exit through x^2 = q + (p+l)^2 at the event point,
-      // the same p + l and x^2 the move to the event computes.
-      const double xi2 = c_xi2, xo2 = c_xo2;
-      const bool inner = strictly_negative(pp) && rawkey(q) <= rawkey(xi2);  // q, x_in^2 >= 0
-      int shell_state = 0;  // 0 nothing known, 1 bracket [klo, khi], 2 exact (klo = khi = key)
-      long long klo = 0, khi = 0;
-      double p_exit = 0.0;
-      auto exact_exit = [&]() {
-        p_exit = shell_exit(q, inner, xi2, xo2);
-        klo = khi = rawkey(nu_lab * (1.0 - p_exit));  // > 0
-        shell_state = 2;
-      };
-      // is a Sobolev point or threshold at comoving frequency key beyond the exit?
-      auto beyond_exit = [&](long long key) -> bool {
-        if (key > khi) return false;
-        if (key > klo) exact_exit();
-        return key <= klo;
-      };
-      double c_e = 0.0, thr_e = 0.0;
-      long long key_e = kKeyNegInf;
-      if (thomson) {
-        c_e = (nu_lab * c_ikap) * inv_D;  // nu_lab / k, k = kappa' D
-        thr_e = fma(-tau_rem, c_e, nu_cmf);
-        key_e = rawkey(thr_e);
-      }
+      const double tau = neg_log_u53(ds.next_u53() + 1ull);
+      const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);  // q, x_in^2 >= 0
+      const ScanF f = scan_setup(pk.nu_cmf, pk.D, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, tau);
       // J_blue weight of this segment, E_lab / nu_lab^2 (Eq. 17 without its
       // line factor nu_j, applied per cell after the launch)
-      const double e_inv2 = JB ? pk.e_per_nu * inv_nu : 0.0;
+      const double e_inv2 = JB ? pk.e_per_nu * pk.inv_nu : 0.0;
       const size_t row = static_cast<size_t>(s) * static_cast<size_t>(L);
       const double *tau_s = p.tau + row;
-      int32_t j = pk.next_line;
+      const int32_t j0 = pk.next_line;
+      int32_t j = j0;
       int kind = 0;
-      double l = 0.0, nu_hit = 0.0;
-      double pl_ev = 0.0, r2_ev = 0.0;  // x mu and x^2 at the event, when the exit test made them
-      bool have_ev = false;
-      double D1_ev = 0.0;  // Doppler factor at an electron-scattering point
-      unsigned long long rinfo_hit = 0ull;
+      if (!lw_ok) load_window(s, j);
       // two lines ahead are always in flight while line j is resolved
-      long long bj = 0, bj_n = 0;
-      double taul = 0.0, tau_n = 0.0;
-      unsigned long long rinfo = 0ull, rinfo_n = 0ull;
-      // An absorbing line (Sect. 2.6): the Sobolev point nu_lab (1 - x mu) =
-      // nu_j, so x mu = 1 - nu_j / nu_lab and D = nu_j / nu_lab there (a
-      // resonance that rounding puts behind the packet is taken where the
-      // packet is).  With no line passed yet the event point is also placed
-      // against the shell exit; if the exit comes first the scan ends with no
-      // event (kind stays 0).
-      auto absorb = [&](long long b_, unsigned long long r_) {
-        const double nuj = __longlong_as_double(b_);
-        const double lj = max0(fma(-nuj, inv_nu, D));
-        const bool ahead = rawkey(lj) > 0;
-        pl_ev = ahead ? fma(-nuj, inv_nu, 1.0) : pp;
-        r2_ev = fma(pl_ev, pl_ev, q);
-        have_ev = true;
-        if (shell_state == 0 && !inside_shell(pl_ev, r2_ev, inner, xi2, xo2)) return;  // exit comes first
-        pk.cnt[2] += 1u;
-        if (JB && act) red_add_evict_first(p.j_blue + row + j, e_inv2, jb_pol);
-        kind = kLineEvent;
-        l = lj;
-        nu_hit = nuj;
-        rinfo_hit = r_;
-      };
-      bool fast = false;  // the lone scan below settled the segment's line event
-      // downbranch: the absorbing line's emission record, loaded as soon as the
-      // lone scan names the line (the emission draw is the next in the buffer)
-      bool have_slot = false;
-      ulonglong2 slot_a = make_ulonglong2(0ull, 0ull), slot_c = make_ulonglong2(0ull, 0ull);
-      if (lone) {
-        int idx = j - lwin_j0;
-        if (lwin_s != s || idx < 0 || idx >= 32) {
-          lone_reload(s, j);
-          idx = 0;
-        }
-        if (thomson) {
-          // The scan of lines j0 + idx .. j0 + 31 of the window in one step, lane
-          // k taking line j0 + k.  In exact arithmetic the scan below stops at
-          // line k when nu_k <= T_{k-1} (beyond d_e), when nu_k lies beyond the
-          // shell exit, or when T_k > nu_k (absorbed), with T_k = thr_e + c_e
-          // (tau_idx + ... + tau_k).  Each lane forms A = nu_k - T_{k-1} and B =
-          // nu_k - T_k in binary32 from the exact binary64 difference nu_k - thr_e
-          // (one binary64 instruction for the whole window) and a prefix sum of
-          // the depths, with a bound M on |error| that also covers the rounding
-          // of the scan's own chain of fmas (at most 32 of them).  Where every
-          // sign up to the first line that stops the scan is certain and that
-          // line absorbs, the result is the scan's; otherwise (a sign within
-          // the bound, the exit, d_e or the end of the window reached) the scan
-          // below runs as usual.  Error budget (u = 2^-24): the difference
-          // truncated to binary32 (2u), the depths truncated (2u) and summed in
-          // five levels (5u), c_e truncated (2u), the product and the final
-          // difference (u each), so |A|, |B| error <= 3u |d| + 11u C; the fma
-          // chain adds at most 2^-48 (|thr_e| + C); depths below the binary32
-          // normal range add at most 32 c_e 2^-126.  M = 2^-20 (|d| + C) +
-          // 2^-44 |thr_e| + c_e 2^-119 + 2^-124 bounds all of it.
-          const ShellBracket sb = shell_bracket(q, inner ? xi2 : xo2, inner, nu_lab);
-          const int32_t jl = lwin_j0 + static_cast<int32_t>(lane);
-          const bool cand = static_cast<int>(lane) >= idx;
-          const bool valid = cand && jl < L;
-          const float dk = f32_rz_any(__longlong_as_double(lwin_b) - thr_e);
-          float P = valid ? f32_rz_any(lwin_t) : 0.0f;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const float y = __shfl_up_sync(0xffffffffu, P, o);
-            if (static_cast<int>(lane) >= o) P = __fadd_rn(P, y);
-          }
-          float Px = __shfl_up_sync(0xffffffffu, P, 1);
-          if (lane == 0u) Px = 0.0f;
-          const float ce = f32_rz_any(c_e);
-          const float C = __fmul_rn(ce, P);
-          const float A = __fsub_rn(dk, __fmul_rn(ce, Px)), B = __fsub_rn(dk, C);
-          const float M = __fadd_rn(__fmul_rn(0x1.0p-20f, __fadd_rn(fabsf(dk), C)),
-                                    __fadd_rn(__fmul_rn(0x1.0p-44f, fabsf(f32_rz_any(thr_e))),
-                                              __fmaf_rn(ce, 0x1.0p-119f, 0x1.0p-124f)));
-          const bool e_no = A > M;                               // certainly before d_e
-          const bool a_yes = B < -M, a_no = B > M;               // certainly absorbed / passed
-          const bool x_no = sb.ok && lwin_b > sb.hi;             // certainly before the exit
-          const bool pass = valid && e_no && a_no && x_no;
-          const bool take = valid && e_no && a_yes && (static_cast<int>(lane) == idx || x_no);
-          const unsigned stop = __ballot_sync(0xffffffffu, cand && !pass);
-          const unsigned took = __ballot_sync(0xffffffffu, take);
-          const int kstar = __ffs(stop) - 1;
-          if (kstar >= 0 && ((took >> kstar) & 1u)) {
-            fast = true;
-            const int npass = kstar - idx;
-            pk.cnt[1] += static_cast<uint32_t>(npass + 1);
-            pk.cnt[2] += static_cast<uint32_t>(npass);
-            if (JB && cand && static_cast<int>(lane) < kstar)  // the lines passed, one lane each
-              red_add_evict_first(p.j_blue + row + jl, e_inv2, jb_pol);
-            if (npass > 0) {  // as the scan leaves it after its first pass
-              klo = sb.lo;
-              khi = sb.hi;
-              shell_state = 1;
-            }
-            j = lwin_j0 + kstar;
-            bj = __shfl_sync(0xffffffffu, lwin_b, kstar);
-            rinfo = __shfl_sync(0xffffffffu, lwin_r, kstar);
-            if (MODE == 1 && p.dbr_rec) {
-              load_slot(bucket_slot(p, rinfo, wd.peek_u53(ds)), slot_a, slot_c);
-              have_slot = true;
-            }
-          }
-        }
-        if (!fast) {
-          lone_fetch(s, j, bj, taul, rinfo);
-          lone_fetch(s, j + 1, bj_n, tau_n, rinfo_n);
-        }
-      } else {
-        if (!lw_ok) load_window(s, j);
-        bj = lw_b0; taul = lw_t0; rinfo = lw_r0;
-        bj_n = lw_b1; tau_n = lw_t1; rinfo_n = lw_r1;
-      }
+      long long bj = lw_b0, bj_n = lw_b1, bj_nn = 0;
+      double taul = lw_t0, tau_n = lw_t1, tau_nn = 0.0;
+      unsigned long long rinfo = lw_r0, rinfo_n = lw_r1, rinfo_nn = 0ull;
       lw_ok = false;
-      long long bj_nn = 0;
-      double tau_nn = 0.0;
-      unsigned long long rinfo_nn = 0ull;
-      if (fast) absorb(bj, rinfo);
-      else while (j < L) {
-        pk.cnt[1] += 1u;
-        bj_nn = 0;
-        tau_nn = 0.0;
-        rinfo_nn = 0ull;
-        if (lone) {
-          lone_fetch(s, j + 2, bj_nn, tau_nn, rinfo_nn);
-        } else if (j + 2 < L) {
-          bj_nn = __ldg(nub + j + 2);
-          tau_nn = __ldg(tau_s + j + 2);
-          if (MODE >= 1 && p.row_info) rinfo_nn = __ldg(p.row_info + j + 2);
+      float rem = f.tau, m1 = 0x1.0p-19f, m0 = fmaf(f.tf, 0x1.0p-44f, 0x1.0p-100f);
+      const float m0_step = f.tf * 0x1.0p-51f;
+      for (;;) {
+        bool at_exit = j >= L;
+        if (!at_exit) {
+          bj_nn = 0;
+          tau_nn = 0.0;
+          rinfo_nn = 0ull;
+          if (j + 2 < L) {
+            bj_nn = __ldg(nub + j + 2);
+            tau_nn = __ldg(tau_s + j + 2);
+            if (MODE == 1 && p.row_info) rinfo_nn = __ldg(p.row_info + j + 2);
+          }
+          bool ok;
+          const float l = scan_delta(f, bj, ok) * f.lf;
+          const float a = l * f.tf;
+          const float M = fmaf(m1, a + f.tau, m0);
+          const float r0 = rem - a;
+          if (!ok || !(r0 > M)) break;  // beyond d_e, or in doubt
+          const float xm = f.lx - l, xM = fmaf(0x1.0p-19f, l, f.mx);
+          if (!(xm > xM)) {
+            if (!(xm < -xM)) break;  // in doubt
+            at_exit = true;
+          } else {
+            const float tf = f32_rz_any(taul);
+            const float r1 = r0 - tf;
+            if (r1 < -M) {
+              kind = kLineEvent;
+              break;
+            }
+            if (!(r1 > M) || tf < 0.0f) break;  // in doubt
+            rem -= tf;
+          }
         }
-        if (bj <= key_e) break;                             // the Sobolev point lies beyond d_e
-        if (shell_state != 0 && beyond_exit(bj)) break;     // ... or beyond the shell exit
-        bool absorbed;
-        double t = 0.0;
-        if (thomson) {
-          t = fma(taul, c_e, thr_e);
-          absorbed = rawkey(t) > bj;  // nu_j > 0
-        } else {
-          absorbed = rawkey(taul) > rawkey(tau_rem);  // both >= 0
-        }
-        if (absorbed) {
-          absorb(bj, rinfo);
+        if (at_exit) {  // no line before the exit; certainly before d_e?
+          const float ax = f.lx * f.tf;
+          if (rem - ax > fmaf(m1, fabsf(ax) + f.tau, fmaf(f.tf, f.mx, m0))) kind = kShellEvent;
           break;
         }
-        if (shell_state == 0) {  // a line is passed: the scan needs the exit frequency
-          const ShellBracket sb = shell_bracket(q, inner ? xi2 : xo2, inner, nu_lab);
-          if (sb.ok) {
-            klo = sb.lo;
-            khi = sb.hi;
-            shell_state = 1;
-          } else {
-            exact_exit();
-          }
-          if (beyond_exit(bj)) break;  // this line lies beyond the exit
-        }
-        pk.cnt[2] += 1u;
-        if (JB && act) red_add_evict_first(p.j_blue + row + j, e_inv2, jb_pol);
-        if (thomson) {
-          thr_e = t;
-          key_e = rawkey(t);
-        } else {
-          tau_rem -= taul;
-        }
+        m1 += 0x1.0p-23f;
+        m0 += m0_step;
+        if (JB) red_add_evict_first(p.j_blue + row + j, e_inv2, jb_pol);
         ++j;
         bj = bj_n; taul = tau_n; rinfo = rinfo_n;
         bj_n = bj_nn; tau_n = tau_nn; rinfo_n = rinfo_nn;
       }
+      double thr = 0.0, p_exit = 0.0;
+      long long hit = bj;
+      bool exact = false;
       if (kind == 0) {
-        bool electron;
-        double le = 0.0;
-        have_ev = false;  // an absorbed line that lay beyond the exit left its point here
-        if (shell_state != 0) {
-          electron = thomson && !beyond_exit(key_e);
-          if (electron) le = max0(fma(-thr_e, inv_nu, D));
-        } else {
-          le = thomson ? max0(fma(-thr_e, inv_nu, D)) : 0.0;
-          if (thomson) {
-            pl_ev = pp + le;
-            r2_ev = fma(pl_ev, pl_ev, q);
-            have_ev = true;
-          }
-          electron = thomson && inside_shell(pl_ev, r2_ev, inner, xi2, xo2);
-        }
-        if (electron) {
-          kind = kElectronEvent;
-          l = le;
-          if (!have_ev) {
-            pl_ev = pp + le;
-            r2_ev = fma(pl_ev, pl_ev, q);
-            have_ev = true;
-          }
-          D1_ev = 1.0 - pl_ev;
-        } else {
-          if (shell_state != 2) exact_exit();
-          kind = kShellEvent;
-          l = max0(p_exit - pp);
-          have_ev = false;
-        }
+        exact = true;
+        kind = exact_scan(tau, inner, j0, j, true, e_inv2, hit, thr, p_exit);
+        if (MODE == 1 && p.row_info && kind == kLineEvent) rinfo = __ldg(p.row_info + j);
+      } else if (kind == kShellEvent) {
+        p_exit = shell_exit(pk.q, inner, c_xi2, c_xo2);
+      }
+      const uint32_t npass = static_cast<uint32_t>(j - j0);
+      pk.cnt[1] += npass + (j < L ? 1u : 0u);
+      pk.cnt[2] += npass + (kind == kLineEvent ? 1u : 0u);
+      pk.next_line = j;
+      double l, r2 = 0.0;
+      const double nuj = __longlong_as_double(hit);
+      if (kind == kLineEvent) {
+        if (JB) red_add_evict_first(p.j_blue + row + j, e_inv2, jb_pol);
+        line_point(nuj, l, r2);
+      } else if (kind == kShellEvent) {
+        l = max0(p_exit - pk.p);
+      } else {
+        l = max0(fma(-thr, pk.inv_nu, pk.D));
       }
       // estimators, Eqs. 13-14 (segment-start comoving values)
-      const double wgt = eD2 * l;
+      const double wgt = (pk.e_cmf * pk.D) * l;
       if (s != acc_s) {
-        if (acc_s >= 0 && act) {
+        if (acc_s >= 0) {
           atomicAdd(p.j_est + acc_s, acc_j);
           atomicAdd(p.nu_bar + acc_s, acc_nb);
         }
         acc_s = s; acc_j = 0.0; acc_nb = 0.0;
       }
       acc_j += wgt;
-      acc_nb = fma(wgt, nu_cmf, acc_nb);
-      pk.next_line = j;
+      acc_nb = fma(wgt, pk.nu_cmf, acc_nb);
       if (kind == kShellEvent) {
         // move to the boundary; free flight keeps q, nu_lab and E_lab
         pk.cnt[5] += 1u;
+        need_lab();
         const int32_t ns = inner ? s - 1 : s + 1;
         pk.p = p_exit;
         pk.shell = ns;
         pk.have_cmf = false;
-        lw_ok = false;
         if (ns >= S) status = 1;
         else if (ns < 0) status = 2;
       } else {
-        // move to the event point (x mu, x^2 and D there from the scan)
-        const double r2n = r2_ev;
-        const double xn = sqrt64(r2n);
-        // comoving energy at the event: E / nu times the comoving frequency
-        // there (the line's own frequency at a Sobolev point)
-        double nu_c, inv_nu_c, e_c;
+        double nu_c, inv_c;
         if (kind == kLineEvent) {
           pk.cnt[3] += 1u;
-          e_c = pk.e_per_nu * nu_hit;
+          pk.e_cmf = pk.e_per_nu * nuj;  // E / nu times the line's own frequency
           if (MODE >= 1) {
             // MODE 2: macro atom, internal jumps before the emission pick
-            const unsigned long long rinfo_em =
-                MODE == 2 ? macroatom_walk(p, __ldg(p.line_row + j), wd, ds) : rinfo_hit;
-            const unsigned long long u_em = wd.template next_u53<MODE == 2>(ds);
-            const Emission em = have_slot ? pick_from_slot_lone(p, rinfo_em, u_em, slot_a, slot_c, lane)
-                                          : downbranch_pick(p, j, rinfo_em, u_em);
+            unsigned long long rinfo_em = rinfo;
+            if (MODE == 2) {
+              const MaDraws md{&ds, nullptr, nullptr, 0u, 0u, 0u, 0u};
+              rinfo_em = macroatom_walk(p, __ldg(p.line_row + j), md);
+            }
+            const Emission em = downbranch_pick(p, j, rinfo_em, ds.next_u53());
             nu_c = em.nu;
-            inv_nu_c = em.inv_nu;
-            pk.e_per_nu = e_c * inv_nu_c;  // re-emitted at another frequency
+            inv_c = em.inv_nu;
+            pk.e_per_nu = pk.e_cmf * inv_c;  // re-emitted at another frequency
             pk.next_line = em.line + 1;
-            if (lone) lone_reload(s, pk.next_line);
-            else load_window(s, pk.next_line);
+            load_window(s, pk.next_line);
           } else {
-            nu_c = nu_hit;
-            inv_nu_c = rcp64(nu_hit);
+            nu_c = nuj;
+            inv_c = rcp64(nuj);
             pk.next_line = j + 1;
-            lw_ok = true;  // lines j + 1, j + 2 are in the scan's registers
-            lw_b0 = bj_n; lw_t0 = tau_n; lw_r0 = rinfo_n;
-            lw_b1 = bj_nn; lw_t1 = tau_nn; lw_r1 = rinfo_nn;
+            if (!exact) {
+              lw_ok = true;  // lines j + 1, j + 2 are in the scan's registers
+              lw_b0 = bj_n; lw_t0 = tau_n; lw_r0 = rinfo_n;
+              lw_b1 = bj_nn; lw_t1 = tau_nn; lw_r1 = rinfo_nn;
+            }
           }
         } else {
           pk.cnt[4] += 1u;
-          nu_c = nu_lab * D1_ev;
-          inv_nu_c = inv_nu * rcp64(D1_ev);
-          e_c = pk.e_per_nu * nu_c;
-          lw_ok = true;  // the next segment starts at line j again
-          lw_b0 = bj; lw_t0 = taul; lw_r0 = rinfo;
-          lw_b1 = bj_n; lw_t1 = tau_n; lw_r1 = rinfo_n;
+          const double pl = pk.p + l;
+          r2 = fma(pl, pl, pk.q);
+          const double D1 = 1.0 - pl;
+          nu_c = pk.nu_lab * D1;
+          inv_c = pk.inv_nu * rcp64(D1);
+          pk.e_cmf = pk.e_per_nu * nu_c;
         }
-        // isotropic re-emission: new direction, lab values from the comoving ones
-        const double mu2 = DrawStream::mu_from_u53(wd.template next_u53<MODE == 2>(ds));
-        const double pn = xn * mu2;
-        const double D2 = 1.0 - pn;
-        const double iD2 = rcp64(D2);
-        pk.p = pn;
-        pk.q = max0(fma(-pn, pn, r2n));
-        pk.nu_lab = nu_c * iD2;
-        pk.inv_nu = inv_nu_c * D2;
-        pk.D = D2;
-        pk.inv_D = iD2;
-        pk.nu_cmf = nu_c;       // = nu_lab D2
-        pk.eD2 = e_c * D2;      // = E_lab D2^2
-        pk.have_cmf = true;
-        if (p.n_virtual && act) {
-          spawn_virtual(p, sh, VirtualLaunch{xn, r2n, nu_c, e_c, s, pk.next_line, pk.pid, vdraws, false});
+        const double xn = leave(r2, DrawStream::mu_from_u53(ds.next_u53()), nu_c, inv_c);
+        if (p.n_virtual) {
+          spawn_virtual(p, sh, VirtualLaunch{xn, r2, nu_c, pk.e_cmf, s, pk.next_line, pk.pid, vdraws, false});
           vdraws += static_cast<uint32_t>(p.n_virtual);
         }
       }
     }
-    if (status != 0 && !act) {  // lone mode, not the owner lane: drop the adopted walk
-      alive = false;
-      lone = false;
-      acc_s = -1;
-      acc_j = 0.0;
-      acc_nb = 0.0;
-    } else if (status != 0) {
-      lone = false;
+    if (status != 0) {
       if (status == 1) ++n_esc;
       else if (status == 2) ++n_reab;
       else ++n_cap;
@@ -974,17 +1119,17 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       const double e_lab = pk.e_per_nu * pk.nu_lab;
       if (status == 1) atomicAdd(p.spectrum + spectrum_bin(p, pk.nu_lab), e_lab);
       if (REC) {
-        p.rec_status[pk.pid - p.first_packet] = status;
-        p.rec_nu[pk.pid - p.first_packet] = pk.nu_lab;
-        p.rec_e[pk.pid - p.first_packet] = e_lab;
+        const uint32_t r = static_cast<uint32_t>(pk.pid - p.first_packet);
+        p.rec_status[r] = status;
+        p.rec_nu[r] = pk.nu_lab;
+        p.rec_e[r] = e_lab;
 #pragma unroll
-        for (int c = 0; c < kNCounters; ++c)
-          p.rec_cnt[static_cast<size_t>(pk.pid - p.first_packet) * kNCounters + c] = pk.cnt[c];
+        for (int c = 0; c < kNCounters; ++c) p.rec_cnt[static_cast<size_t>(r) * kNCounters + c] = pk.cnt[c];
       }
       alive = false;
     }
   }
-  if (acc_s >= 0 && (!lone || static_cast<int>(lane) == owner)) {  // (a launch stopped in lone mode)
+  if (acc_s >= 0) {
     atomicAdd(p.j_est + acc_s, acc_j);
     atomicAdd(p.nu_bar + acc_s, acc_nb);
   }
@@ -1019,10 +1164,10 @@ const void *select_kernel(int line_mode, int precision, bool jb, bool rec) {
 }
 
 size_t smem_bytes(int S, int precision) {
-  // binary64: shell tables, then one WarpDraws buffer (u53 + -ln z) per warp
+  // binary64: shell tables, then one LoneDraws buffer (u53, -ln z, mu) per warp
   return precision == 1 ? mixed_smem_bytes(S)
                         : static_cast<size_t>(kShellArrays) * S * sizeof(double) +
-                              (kBlock / 32) * 2 * kWarpDraws * sizeof(double);
+                              (kBlock / 32) * 3 * kWarpDraws * sizeof(double);
 }
 
 }  // namespace
