@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "mc_internal.h"
+
 namespace mcgpu {
 
 // Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of two
@@ -92,6 +94,15 @@ __device__ __forceinline__ float f32_rz_any(double d) {
   return __int_as_float(static_cast<int>(mag | (static_cast<unsigned int>(b >> 63) << 31)));
 }
 
+// The same for |d| < 2^127 (fewer instructions): below the binary32 normal
+// range (signed) 0.
+__device__ __forceinline__ float f32_rz_small(double d) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(d)), lo = static_cast<uint32_t>(__double2loint(d));
+  const uint32_t a = hi & 0x7fffffffu;
+  const uint32_t m = __funnelshift_l(lo, a - 0x38000000u, 3);  // the exponent rebiased, 23 fraction bits
+  return __uint_as_float((a >= 0x38100000u ? m : 0u) | (hi & 0x80000000u));
+}
+
 // v < 0, excluding -0 (its pattern is the most negative integer).
 __device__ __forceinline__ bool strictly_negative(double v) {
   const long long b = __double_as_longlong(v);
@@ -124,6 +135,25 @@ __device__ __forceinline__ void red_add_evict_first(unsigned long long *a, unsig
   asm volatile("red.global.add.L2::cache_hint.u64 [%0], %1, %2;" ::"l"(a), "l"(v), "l"(pol) : "memory");
 }
 
+// Read-only loads that are issued where they stand: the compiler may move a
+// plain load down to its first use, and on a lone walk the instructions
+// between the two are what its latency hides behind.
+__device__ __forceinline__ unsigned long long load_here(const void *a) {
+  unsigned long long v;
+  asm volatile("ld.global.nc.b64 %0, [%1];" : "=l"(v) : "l"(a));
+  return v;
+}
+__device__ __forceinline__ float load_here_f(const float *a) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 load_here4(const void *a) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
+  return v;
+}
+
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -138,11 +168,21 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // ch. 2).  Three binary64 operations instead of the four of two Newton steps.
 // Within 1 ulp of 1/x for normal |x| in [2^-1000, 2^1000] (tested against
 // IEEE division through mc_selftest_math).
+__device__ __forceinline__ double rcp64_from(double x, double r) {
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
 __device__ __forceinline__ double rcp64(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
+  return rcp64_from(x, r);
+}
+// The same value, evaluated only where it stands (the compiler may evaluate
+// the one above ahead of the branch that needs it).
+__device__ __forceinline__ double rcp64_here(double x) {
+  double r;
+  asm volatile("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return rcp64_from(x, r);
 }
 
 // Square root of x >= 0 (0 or a normal number) to within 1 ulp, in five
@@ -154,14 +194,16 @@ __device__ __forceinline__ double rcp64(double x) {
 // 5e^3/16, is below 2^-58 relative.  (CUDA's sqrt rounds correctly but takes
 // about ten binary64 instructions; on GB300 each costs its sub-partition's
 // FP64 pipe ~64 cycles.)
-__device__ __forceinline__ double sqrt64(double x) {
+__device__ __forceinline__ double sqrt64_pos(double x) {  // x > 0
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double t = x * y;
   const double e = fma(-t, y, 1.0);
   const double p = fma(0.375, e, 0.5);
-  const double r = fma(t * e, p, t);
-  return __double_as_longlong(x) == 0ll ? 0.0 : r;
+  return fma(t * e, p, t);
+}
+__device__ __forceinline__ double sqrt64(double x) {
+  return __double_as_longlong(x) == 0ll ? 0.0 : sqrt64_pos(x);
 }
 
 // ln(2) split so that k * kLn2Head is exact for |k| < 2^20.
@@ -230,15 +272,123 @@ __device__ __forceinline__ double neg_log_u53(unsigned long long u) {
   return -((kl.x + ct.y) + fma(p, r, kl.y));
 }
 
-// Draws of a warp's last live packet, computed ahead by the whole warp.
-// Once the packet queue is empty and one lane of a warp is left, the other
-// 31 lanes have nothing to do; a draw's value depends only on (key, packet,
-// iteration, draw index), so lane i computes Philox block base/2 + i and the
-// -ln z of both its draws, and the live lane reads its next 64 draws from
-// shared memory instead of running Philox and the log on its own dependency
-// chain.  Values are identical to DrawStream's.  All state is warp-uniform.
-// (Serving up to four live lanes, with per-lane slots, measured slower: the
-// per-segment bookkeeping then costs more than the draws it saves.)
+// -ln z in binary32 for the draw z = u 2^-53, 1 <= u <= 2^53, to a relative
+// error below 2^-21: z = m 2^e with m in [0.75, 1.5), f = m - 1 from the
+// integer (exact to 2^-23 however near 1 the draw is), ln m = 2 atanh(s) with
+// s = f / (2 + f), |s| <= 1/5, by its series to s^9 (Abramowitz & Stegun
+// 4.1.27; the first omitted term is below 2^-27 of the sum).
+__device__ __forceinline__ float neg_log_u53_f(unsigned long long u) {
+  const int lz = __clzll(static_cast<long long>(u));
+  const unsigned long long m = u << lz;  // [2^63, 2^64)
+  const bool up = m >= 0xc000000000000000ull;
+  const unsigned long long a = up ? 0ull - m : m - 0x8000000000000000ull;  // |f| 2^64 or 2^63
+  const float mag = fmaf(static_cast<float>(static_cast<uint32_t>(a >> 32)), 0x1.0p32f,
+                         static_cast<float>(static_cast<uint32_t>(a)));
+  const float f = up ? mag * -0x1.0p-64f : mag * 0x1.0p-63f;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(2.0f + f));
+  const float s = f * r, s2 = s * s;
+  float q = fmaf(s2, 1.0f / 9.0f, 1.0f / 7.0f);
+  q = fmaf(s2, q, 0.2f);
+  q = fmaf(s2, q, 1.0f / 3.0f);
+  const float lnm = 2.0f * fmaf(s * s2, q, s);
+  return fmaf(static_cast<float>(lz - 10 - (up ? 1 : 0)), 0x1.62e43p-1f, -lnm);
+}
+
+// Downbranch emission (Sect. 2.5): the first entry k of the activated upper
+// level's branching row with z < cdf[k], z = u 2^-53.  z < cdf[k] <=> u <
+// ceil(cdf[k] 2^53) = thr[k] exactly; the search starts at the guide entry of
+// bucket floor(z n), whose slot settles most draws.
+// The bucket slot of draw u in the row of rinfo (begin | length << 32):
+// floor(u n / 2^53) in two 32-bit products.
+__device__ __forceinline__ const DbrSlot *bucket_slot(const DbrSlot *slots, unsigned long long rinfo,
+                                                      unsigned long long u) {
+  const uint32_t b = static_cast<uint32_t>(rinfo), len = static_cast<uint32_t>(rinfo >> 32);
+  const unsigned long long lo = static_cast<unsigned long long>(static_cast<uint32_t>(u)) * len;
+  const unsigned long long s = static_cast<unsigned long long>(static_cast<uint32_t>(u >> 32)) * len + (lo >> 32);
+  return slots + b + static_cast<uint32_t>(s >> 21);
+}
+
+__device__ __forceinline__ void load_slot(const DbrSlot *slot, uint4 &a, uint4 &c) {
+  a = __ldg(reinterpret_cast<const uint4 *>(slot));
+  c = __ldg(reinterpret_cast<const uint4 *>(slot) + 1);
+}
+
+__device__ __forceinline__ void load_slot_here(const DbrSlot *slot, uint4 &a, uint4 &c) {
+  a = load_here4(slot);
+  c = load_here4(reinterpret_cast<const uint4 *>(slot) + 1);
+}
+
+// The emitted line from a loaded slot {thr[3], emit[0]}, {emit[1], emit[2],
+// guide, -}, or -1: u's upper 32 bits equal a threshold's, or u lies behind
+// the slot's entries.
+__device__ __forceinline__ int32_t slot_line(uint4 a, uint4 c, unsigned long long u) {
+  const uint32_t v = static_cast<uint32_t>(u >> 21);
+  uint32_t line = a.w;
+  if (v >= a.x) line = (v > a.x && v < a.y) ? c.x : (v > a.y && v < a.z) ? c.y : 0xffffffffu;
+  return static_cast<int32_t>(line);
+}
+
+// The row's entries one by one from position i (the last has thr = 2^53 > u).
+__device__ __forceinline__ int32_t search_row(const DbrRec *rec, uint32_t i, unsigned long long u) {
+  while (u >= __ldg(&rec[i].thr)) ++i;
+  return static_cast<int32_t>(__ldg(&rec[i].emit));
+}
+
+// Lone walk (all 32 lanes converged): 32 entries of the row per coalesced load
+// (lane i takes entry i), the first with u below its threshold by a vote.
+__device__ __forceinline__ int32_t search_row_lone(const DbrRec *rec, unsigned long long rinfo, uint32_t guide,
+                                                   unsigned long long u, unsigned lane) {
+  const uint32_t end = static_cast<uint32_t>(rinfo) + static_cast<uint32_t>(rinfo >> 32);
+  for (uint32_t i0 = static_cast<uint32_t>(rinfo) + guide;; i0 += 32u) {
+    const uint32_t i = i0 + lane;
+    ulonglong2 r = make_ulonglong2(~0ull, 0ull);  // lanes past the row's end vote yes
+    if (i < end) r = __ldg(reinterpret_cast<const ulonglong2 *>(rec + i));
+    const unsigned m = __ballot_sync(0xffffffffu, u < r.x);
+    if (m != 0u)
+      return __shfl_sync(0xffffffffu, static_cast<int32_t>(static_cast<uint32_t>(r.y)), __ffs(m) - 1);
+  }
+}
+
+// Constants of a segment's line scan in binary32 (the error budget stands at
+// the binary64 kernel's scan).
+struct ScanF {
+  unsigned long long mc;  // significand of nu_cmf
+  int ec;                 // its exponent field
+  float lf, tf;           // path length per unit of significand difference; kappa' D
+  float tau;              // the optical-depth draw
+  float lx, mx;           // path length to the shell exit and its error bound (infinite: not known)
+};
+
+// The frequency's part of it; Df = D in binary32.
+__device__ __forceinline__ void scan_frequency(ScanF &f, double nu_cmf, float Df) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(nu_cmf));
+  f.ec = static_cast<int>(b >> 52);
+  f.mc = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  float im;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(im) : "f"(static_cast<float>(static_cast<uint32_t>(f.mc >> 29))));
+  f.lf = (Df * im) * 0x1.0p-29f;
+}
+
+// Significand difference nu_cmf - nu_line in units of nu_cmf's last place, as
+// binary32 (0 when the line is not below nu_cmf); ok: the line's binade is
+// nu_cmf's or a lower one.
+__device__ __forceinline__ float scan_delta(const ScanF &f, long long line_bits, bool &ok) {
+  const unsigned long long b = static_cast<unsigned long long>(line_bits);
+  const int sh = f.ec - static_cast<int>(b >> 52);
+  ok = sh >= 0;
+  const unsigned long long m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  const long long d = static_cast<long long>(f.mc) - static_cast<long long>(m >> (sh < 63 ? sh & 63 : 63));
+  const float v = fmaf(static_cast<float>(static_cast<uint32_t>(d >> 32)), 0x1.0p32f,
+                       static_cast<float>(static_cast<uint32_t>(d)));
+  return d > 0 ? v : 0.0f;
+}
+
+// Draws of a lone walk in the mixed kernel, computed ahead by the whole warp:
+// a draw's value depends only on (key, packet, iteration, draw index), so lane i
+// computes Philox block base/2 + i and the walk reads its next 64 draws from
+// shared memory instead of running Philox on its own dependency chain.  Values
+// are identical to DrawStream's.  All state is warp-uniform.
 constexpr uint32_t kWarpDraws = 64;
 constexpr uint32_t kNoPacket = 0xffffffffu;
 
@@ -250,69 +400,18 @@ static __device__ __noinline__ unsigned long long u53_past_buffer(uint32_t k0, u
   const uint4 o = philox4x32_10(make_uint4(i >> 1, packet, iteration, 0u), k0, k1);
   return (i & 1u) ? DrawStream::u53_of(o.z, o.w) : DrawStream::u53_of(o.x, o.y);
 }
-static __device__ __noinline__ double tau_past_buffer(uint32_t k0, uint32_t k1, uint32_t packet, uint32_t iteration,
-                                               uint32_t i) {
-  return neg_log_u53(u53_past_buffer(k0, k1, packet, iteration, i) + 1ull);
-}
 
 struct WarpDraws {
   unsigned long long *u;  // [64] u53 of draws base .. base + 63 (shared memory, per warp)
-  double *t;              // [64] -ln((u53 + 1) 2^-53) of the same draws
   uint32_t base, pid;     // first draw index held, packet (kNoPacket: none)
-  bool on;                // the warp is down to one live lane, which reads the buffer
 
   __device__ __forceinline__ void init(unsigned long long *warp_buf) {
     u = warp_buf;
-    t = reinterpret_cast<double *>(warp_buf + kWarpDraws);
     base = 0u;
     pid = kNoPacket;
-    on = false;
   }
-
-  // All 32 lanes, converged, after the claim step.  alive: this lane has a
-  // packet; drained: the packet queue is empty.  With one live lane left,
-  // refill the buffer when it holds fewer than the three draws a segment may
-  // take (or belongs to another packet).
-  __device__ __forceinline__ void prepare(bool alive, bool drained, const DrawStream &ds,
-                                          uint32_t packet, uint32_t k0, uint32_t k1,
-                                          uint32_t iteration, unsigned lane) {
-    const unsigned live = __ballot_sync(0xffffffffu, alive);
-    on = drained && __popc(live) == 1;
-    if (!on) return;
-    const int owner = __ffs(live) - 1;
-    const uint32_t d = __shfl_sync(0xffffffffu, ds.d, owner);
-    const uint32_t pk = __shfl_sync(0xffffffffu, packet, owner);
-    if (pk == pid && d + 3u <= base + kWarpDraws) return;
-    const uint32_t b = d & ~1u;
-    const uint4 o = philox4x32_10(make_uint4((b >> 1) + lane, pk, iteration, 0u), k0, k1);
-    const unsigned long long u0 = DrawStream::u53_of(o.x, o.y), u1 = DrawStream::u53_of(o.z, o.w);
-    u[2 * lane] = u0;
-    u[2 * lane + 1] = u1;
-    t[2 * lane] = neg_log_u53(u0 + 1ull);
-    t[2 * lane + 1] = neg_log_u53(u1 + 1ull);
-    __syncwarp();
-    base = b;
-    pid = pk;
-  }
-  // Lone-walker mode (every lane of the warp holds the walker's draw stream):
-  // refill when fewer than the three draws a segment may take are left.
-  __device__ __forceinline__ void keep(const DrawStream &ds, uint32_t k0, uint32_t k1, uint32_t iteration,
-                                       unsigned lane) {
-    if (ds.packet == pid && ds.d + 3u <= base + kWarpDraws) return;
-    const uint32_t b = ds.d & ~1u;
-    const uint4 o = philox4x32_10(make_uint4((b >> 1) + lane, ds.packet, iteration, 0u), k0, k1);
-    const unsigned long long u0 = DrawStream::u53_of(o.x, o.y), u1 = DrawStream::u53_of(o.z, o.w);
-    __syncwarp();  // every lane has read the old contents
-    u[2 * lane] = u0;
-    u[2 * lane + 1] = u1;
-    t[2 * lane] = neg_log_u53(u0 + 1ull);
-    t[2 * lane + 1] = neg_log_u53(u1 + 1ull);
-    __syncwarp();
-    base = b;
-    pid = ds.packet;
-  }
-  // As keep(), for a kernel that takes only the u53 values from the buffer
-  // (the mixed-precision kernel's log is binary32): the -ln z half stays unset.
+  // All 32 lanes hold the walk's draw stream: refill when fewer than the three
+  // draws a segment may take are left.
   __device__ __forceinline__ void keep_u(const DrawStream &ds, uint32_t k0, uint32_t k1, uint32_t iteration,
                                          unsigned lane) {
     if (ds.packet == pid && ds.d + 3u <= base + kWarpDraws) return;
@@ -325,31 +424,10 @@ struct WarpDraws {
     base = b;
     pid = ds.packet;
   }
-  // The lone walker's next draw, from the buffer that keep() or keep_u()
-  // holds filled for the segment.
+  // The walk's next draw, from the buffer that keep_u() holds filled.
   __device__ __forceinline__ unsigned long long take_u53(DrawStream &ds) const { return u[ds.d++ - base]; }
-  // The live lane's next draw (u53, or the -ln z of an open-interval draw).
-  // UNBOUNDED: a segment may take more draws than the buffer holds (a macro
-  // atom's internal jumps), and past its end a draw is computed on its own;
-  // otherwise a segment takes at most three draws and prepare() keeps three
-  // in the buffer.
-  template <bool UNBOUNDED>
-  __device__ __forceinline__ unsigned long long next_u53(DrawStream &ds) const {
-    if (!on) return ds.next_u53();
-    const uint32_t i = ds.d++ - base;
-    if (!UNBOUNDED || i < kWarpDraws) return u[i];
-    return u53_past_buffer(ds.k0, ds.k1, ds.packet, ds.iteration, ds.d - 1u);
-  }
-  // The draw next_u53 returns next, without taking it; only while the buffer
-  // holds it (lone-walker mode, within a segment's three draws).
+  // The draw take_u53 returns next, without taking it.
   __device__ __forceinline__ unsigned long long peek_u53(const DrawStream &ds) const { return u[ds.d - base]; }
-  template <bool UNBOUNDED>
-  __device__ __forceinline__ double next_tau(DrawStream &ds) const {
-    if (!on) return neg_log_u53(ds.next_u53() + 1ull);
-    const uint32_t i = ds.d++ - base;
-    if (!UNBOUNDED || i < kWarpDraws) return t[i];
-    return tau_past_buffer(ds.k0, ds.k1, ds.packet, ds.iteration, ds.d - 1u);
-  }
 };
 
 // ln(x) for a positive normal binary64 x.

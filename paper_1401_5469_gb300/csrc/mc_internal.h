@@ -29,16 +29,22 @@ enum Stat : int {
 constexpr int kNCounters = 6;
 
 // One entry of a downbranch branching row, in the order of the row:
-// thr = ceil(cdf * 2^53) (so that z < cdf <=> u53 < thr for z = u53 2^-53),
-// the emitted line with its frequency and reciprocal, and the guide entry
-// of bucket (this entry's position in the row): the first position whose
-// thr exceeds the smallest u53 of that bucket.
+// thr = ceil(cdf * 2^53) (so that z < cdf <=> u53 < thr for z = u53 2^-53), the
+// emitted line, and the guide entry of bucket (this entry's position in the
+// row): the first position whose thr exceeds the smallest u53 of that bucket.
 struct DbrRec {
   unsigned long long thr;
-  double nu;
-  double inv_nu;
   uint32_t emit;
   uint32_t guide;
+};
+
+// Bucket k of a row: the upper 32 bits of the thresholds of its guide entry
+// and the next two (0 behind the row's end; 2^32 - 1 at most), the lines these
+// emit, and the guide entry's position.  One 32-byte load settles all draws
+// but 2% of those of rows with Dirichlet weights (with the guide entry alone,
+// as a 53-bit threshold, frequency and reciprocal, all but 37%).
+struct DbrSlot {
+  uint32_t thr[3], emit[3], guide, pad;
 };
 
 // Macro-atom level (mode MC_LINE_MACROATOM), one per downbranch row: jump
@@ -74,8 +80,9 @@ struct TransportParams {
   const DbrRec *dbr_rec;             // [nnz] guide-table rows, or nullptr
   const MaRow *ma_row;               // [rows] macro-atom levels, or nullptr (no internal jumps)
   const MaJump *ma_jump;             // [n] macro-atom jump entries
-  const DbrRec *dbr_bucket;          // [nnz] bucket k of a row: copy of its guide entry's
-                                     // record, guide field = that entry's position
+  const DbrSlot *dbr_bucket;         // [nnz] the rows' buckets, or nullptr
+  const double *inv_nu;              // [L] 1 / nu (binary64; with dbr_rec)
+  const float *inv_nu32;             // [L] the same truncated to binary32 (mixed; with dbr_rec)
   double *j_est, *nu_bar;            // [S] raw sums
   double *j_blue;                    // [S*L] raw sums or nullptr
   double *spectrum;                  // [bins + 2]
@@ -169,7 +176,8 @@ struct UpdateParams {
 cudaError_t launch_transport(const TransportParams &p, int line_mode, int precision, bool j_blue,
                              bool record, int grid, int block, cudaStream_t st);
 int transport_block_size();
-cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, int S,
+// tables: the branching rows have bucket slots (a model's; not the caller-owned table's)
+cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, bool tables, int S,
                                 int *blocks_per_sm);
 const void *select_mixed_kernel(int line_mode, bool j_blue, bool record);
 // Batched launches: `block` threads per block (64, 128 or 256).
@@ -198,7 +206,8 @@ cudaError_t launch_zero_large(double *a, size_t n, cudaStream_t st);
 cudaError_t launch_dbr_setup(uint32_t nnz, uint32_t n_rows, uint32_t L, int K,
                              const uint32_t *dbr_offset, const uint32_t *dbr_line,
                              const double *dbr_cdf, const double *nu, const int32_t *line_row,
-                             DbrRec *rec, DbrRec *bucket, unsigned long long *row_info,
+                             DbrRec *rec, DbrSlot *bucket, unsigned long long *row_info,
+                             double *inv_nu, float *inv_nu32,
                              cudaStream_t st);
 cudaError_t launch_line_setup(int L, int K, const double *nu, const double *f, const int32_t *ion,
                               const int32_t *lower, const int32_t *upper, const double *g,

@@ -35,7 +35,10 @@ struct mc_model {
   double *kappa = nullptr, *inv_kappa = nullptr;
   float *shell32 = nullptr;  // [4 S] binary32 x_in^2, x_out^2, kappa', 1/kappa' (mixed precision)
   unsigned long long *est_fix = nullptr;  // [2 S] fixed-point J, nu_bar sums (mixed precision)
-  mcgpu::DbrRec *dbr_rec = nullptr, *dbr_bucket = nullptr;
+  mcgpu::DbrRec *dbr_rec = nullptr;
+  mcgpu::DbrSlot *dbr_bucket = nullptr;
+  double *inv_nu = nullptr;          // with dbr_rec: 1 / nu (binary64 models)
+  float *inv_nu32 = nullptr;         // ... or the same in binary32 (mixed precision)
   mcgpu::MaRow *ma_row = nullptr;    // macro-atom levels (MC_LINE_MACROATOM)
   mcgpu::MaJump *ma_jump = nullptr;
   unsigned long long *row_info = nullptr;

@@ -222,8 +222,7 @@ __global__ void line_setup_kernel(int L, int K, const double *nu, const double *
 // row of length n is the first position whose thr exceeds the smallest u53 of
 // the bucket, ceil(k 2^53 / n).
 __global__ void dbr_rec_kernel(uint32_t nnz, uint32_t n_rows, const uint32_t *off,
-                               const uint32_t *line, const double *cdf, const double *nu,
-                               DbrRec *rec) {
+                               const uint32_t *line, const double *cdf, DbrRec *rec) {
   const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nnz) return;
   uint32_t lo = 0, hi = n_rows;  // row r with off[r] <= e < off[r+1]
@@ -235,8 +234,6 @@ __global__ void dbr_rec_kernel(uint32_t nnz, uint32_t n_rows, const uint32_t *of
   const double scaled = cdf[e] * 0x1.0p53;
   rec[e].thr = static_cast<unsigned long long>(ceil(scaled));
   rec[e].emit = line[e];
-  rec[e].nu = nu[line[e]];
-  rec[e].inv_nu = 1.0 / nu[line[e]];
   const unsigned __int128 num = (static_cast<unsigned __int128>(k) << 53) + (n - 1);
   const unsigned long long u_min = static_cast<unsigned long long>(num / n);
   uint32_t a = 0, z = n - 1;  // first position with thr > u_min (the last has thr = 2^53)
@@ -248,10 +245,9 @@ __global__ void dbr_rec_kernel(uint32_t nnz, uint32_t n_rows, const uint32_t *of
   rec[e].guide = a;
 }
 
-// Bucket slots: slot b + k holds the record of the row's guide entry G[k],
-// with its guide field set to G[k].
+// Bucket slots: slot b + k holds the row's entries from guide entry G[k] on.
 __global__ void dbr_bucket_kernel(uint32_t nnz, uint32_t n_rows, const uint32_t *off,
-                                  const DbrRec *rec, DbrRec *bucket) {
+                                  const DbrRec *rec, DbrSlot *bucket) {
   const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nnz) return;
   uint32_t lo = 0, hi = n_rows;
@@ -259,11 +255,26 @@ __global__ void dbr_bucket_kernel(uint32_t nnz, uint32_t n_rows, const uint32_t 
     const uint32_t mid = (lo + hi) >> 1;
     if (off[mid] <= e) lo = mid; else hi = mid;
   }
-  const uint32_t b = off[lo];
-  const uint32_t g = rec[e].guide;
-  DbrRec r = rec[b + g];
-  r.guide = g;
+  const uint32_t b = off[lo], n = off[lo + 1] - b;
+  DbrSlot r{};
+  r.guide = rec[e].guide;
+  for (uint32_t i = 0; i < 3 && r.guide + i < n; ++i) {
+    const DbrRec q = rec[b + r.guide + i];
+    const unsigned long long t = q.thr >> 21;
+    r.thr[i] = t > 0xffffffffull ? 0xffffffffu : static_cast<uint32_t>(t);
+    r.emit[i] = q.emit;
+  }
   bucket[e] = r;
+}
+
+// 1 / nu of every line, as binary64 or truncated to binary32 (either may be
+// nullptr; binary32 for line frequencies inside its normal range).
+__global__ void inv_nu_kernel(uint32_t L, const double *nu, double *inv, float *inv32) {
+  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= L) return;
+  const double v = 1.0 / nu[j];
+  if (inv) inv[j] = v;
+  if (inv32) inv32[j] = __double2float_rz(v);
 }
 
 __global__ void row_info_kernel(uint32_t L, const int32_t *line_row, const uint32_t *off,
@@ -377,15 +388,16 @@ cudaError_t launch_line_setup(int L, int K, const double *nu, const double *f, c
 cudaError_t launch_dbr_setup(uint32_t nnz, uint32_t n_rows, uint32_t L, int K,
                              const uint32_t *dbr_offset, const uint32_t *dbr_line,
                              const double *dbr_cdf, const double *nu, const int32_t *line_row,
-                             DbrRec *rec, DbrRec *bucket, unsigned long long *row_info,
-                             cudaStream_t st) {
+                             DbrRec *rec, DbrSlot *bucket, unsigned long long *row_info,
+                             double *inv_nu, float *inv_nu32, cudaStream_t st) {
   (void)K;
   if (nnz > 0) {
-    dbr_rec_kernel<<<(nnz + 255) / 256, 256, 0, st>>>(nnz, n_rows, dbr_offset, dbr_line, dbr_cdf, nu, rec);
+    dbr_rec_kernel<<<(nnz + 255) / 256, 256, 0, st>>>(nnz, n_rows, dbr_offset, dbr_line, dbr_cdf, rec);
     dbr_bucket_kernel<<<(nnz + 255) / 256, 256, 0, st>>>(nnz, n_rows, dbr_offset, rec, bucket);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  inv_nu_kernel<<<(L + 255) / 256, 256, 0, st>>>(L, nu, inv_nu, inv_nu32);
   row_info_kernel<<<(L + 255) / 256, 256, 0, st>>>(L, line_row, dbr_offset, row_info);
   return cudaGetLastError();
 }

@@ -22,9 +22,11 @@
 //    registers and are flushed once per shell change;
 //  * a warp down to its last live walk runs it with all 32 lanes (the lone
 //    walk), and few packets are spread over all warps.
-// Longest walk of the 500,000-line model (94,495 segments) alone: 212 ms before
-// the binary32 scan, 165 ms with it; its 1e6-packet iteration 236 -> 182 ms (queue
-// 9.9 -> 6.9 ms); 1e4 packets of the 2000-line scatter model 520 -> 388 us.
+// Longest walk of the 500,000-line model (94,495 segments) alone: 212 ms with a
+// binary64 scan, 165 ms with the scan in binary32, 107 ms with the lone walk's
+// line-event loop (2.25 -> 1.13 us a segment; bound by its binary64 chain, 14
+// instructions of 64 cycles, beside two dependent L2 loads of ~400 cycles);
+// its 1e6-packet iteration 236 -> 155 ms (queue 9.9 -> 5.9 ms).
 #include <cstdint>
 
 #include "mc_device.cuh"
@@ -35,6 +37,7 @@ namespace mcgpu {
 namespace {
 
 constexpr int kBlock = 128;
+constexpr size_t kLoneDrawBytes = kWarpDraws * (2 * sizeof(double) + sizeof(float));
 constexpr int kShellArrays = 6;  // x_in^2, x_out^2, x_in, x_out, kappa, 1/kappa
 constexpr int kLineEvent = 1, kElectronEvent = 2, kShellEvent = 3;
 
@@ -69,92 +72,16 @@ __device__ __forceinline__ int32_t first_redward(const double *nu, int32_t L, do
   return lo;
 }
 
-struct Emission {
-  double nu, inv_nu;
-  int32_t line;
-};
-
-// Downbranch re-emission (Sect. 2.5): the first entry k of the activated
-// upper level's branching row with z < cdf[k], z = u 2^-53.  With the guide
-// table: z < cdf[k] <=> u < ceil(cdf[k] 2^53) = thr[k] exactly; the search
-// starts at the guide entry of bucket floor(z n) and walks forward.
-// The bucket slot of draw u in the branching row of rinfo (begin | length << 32).
-__device__ __forceinline__ const DbrRec *bucket_slot(const TransportParams &p, unsigned long long rinfo,
-                                                     unsigned long long u) {
-  const uint32_t b = static_cast<uint32_t>(rinfo), len = static_cast<uint32_t>(rinfo >> 32);
-  const uint32_t bucket = static_cast<uint32_t>(__umul64hi(u << 11, static_cast<unsigned long long>(len)));
-  return p.dbr_bucket + b + bucket;
-}
-
-// A slot record as two 16-byte halves: {thr, nu} and {inv_nu, emit | guide << 32}.
-__device__ __forceinline__ void load_slot(const DbrRec *slot, ulonglong2 &a, ulonglong2 &c) {
-  a = __ldg(reinterpret_cast<const ulonglong2 *>(slot));
-  c = __ldg(reinterpret_cast<const ulonglong2 *>(slot) + 1);
-}
-
-// The emission from a loaded slot record: the slot itself when u is below its
-// threshold, else the walk forward from its guide entry.
-__device__ __forceinline__ Emission pick_from_slot(const TransportParams &p, unsigned long long rinfo,
-                                                   unsigned long long u, ulonglong2 a, ulonglong2 c) {
-  Emission em;
-  if (u < a.x) {
-    em.nu = __longlong_as_double(static_cast<long long>(a.y));
-    em.inv_nu = __longlong_as_double(static_cast<long long>(c.x));
-    em.line = static_cast<int32_t>(static_cast<uint32_t>(c.y));
-    return em;
-  }
-  const DbrRec *rec = p.dbr_rec;
-  uint32_t i = static_cast<uint32_t>(rinfo) + static_cast<uint32_t>(c.y >> 32) + 1u;
-  unsigned long long thr = __ldg(&rec[i].thr);
-  while (u >= thr) { ++i; thr = __ldg(&rec[i].thr); }
-  em.nu = __ldg(&rec[i].nu);
-  em.inv_nu = __ldg(&rec[i].inv_nu);
-  em.line = static_cast<int32_t>(__ldg(&rec[i].emit));
-  return em;
-}
-
-// Lone-walker mode (all 32 lanes converged on one walk): the pick from the
-// bucket slot's record, and past it the next 32 records of the row in one
-// coalesced load per round (lane i takes entry i), the first with u below
-// its threshold found by a vote.  The row's last threshold is 2^53 > u, so
-// the search ends inside the row.
-__device__ __forceinline__ Emission pick_from_slot_lone(const TransportParams &p, unsigned long long rinfo,
-                                                        unsigned long long u, ulonglong2 a, ulonglong2 c,
-                                                        unsigned lane) {
-  Emission em;
-  if (u < a.x) {
-    em.nu = __longlong_as_double(static_cast<long long>(a.y));
-    em.inv_nu = __longlong_as_double(static_cast<long long>(c.x));
-    em.line = static_cast<int32_t>(static_cast<uint32_t>(c.y));
-    return em;
-  }
-  const uint32_t end = static_cast<uint32_t>(rinfo) + static_cast<uint32_t>(rinfo >> 32);
-  uint32_t i0 = static_cast<uint32_t>(rinfo) + static_cast<uint32_t>(c.y >> 32) + 1u;
-  for (;;) {
-    const uint32_t i = i0 + lane;
-    ulonglong2 ra = make_ulonglong2(~0ull, 0ull), rc = make_ulonglong2(0ull, 0ull);
-    if (i < end) load_slot(p.dbr_rec + i, ra, rc);
-    const unsigned m = __ballot_sync(0xffffffffu, u < ra.x);  // lanes past the row's end vote yes
-    if (m != 0u) {
-      const int k = __ffs(m) - 1;
-      em.nu = __longlong_as_double(__shfl_sync(0xffffffffu, static_cast<long long>(ra.y), k));
-      em.inv_nu = __longlong_as_double(__shfl_sync(0xffffffffu, static_cast<long long>(rc.x), k));
-      em.line = __shfl_sync(0xffffffffu, static_cast<int32_t>(static_cast<uint32_t>(rc.y)), k);
-      return em;
-    }
-    i0 += 32u;
-  }
-}
-
-__device__ __forceinline__ Emission downbranch_pick(const TransportParams &p, int32_t j,
-                                                    unsigned long long rinfo, unsigned long long u) {
-  Emission em;
-  if (p.dbr_rec) {
-    // bucket slot: a copy of the guide entry's record, so that the common case
-    // (the guide entry is the answer) is one 32-byte record load
-    ulonglong2 a, c;
-    load_slot(bucket_slot(p, rinfo, u), a, c);
-    return pick_from_slot(p, rinfo, u, a, c);
+// The emitted line of a downbranch row: through the bucket slots, or without
+// them (caller-owned buffers) by bisection of the row's cdf.
+template <bool SLOTS>
+__device__ __forceinline__ int32_t downbranch_pick(const TransportParams &p, int32_t j,
+                                                   unsigned long long rinfo, unsigned long long u) {
+  if (SLOTS) {
+    uint4 a, c;
+    load_slot(bucket_slot(p.dbr_bucket, rinfo, u), a, c);
+    const int32_t line = slot_line(a, c, u);
+    return line >= 0 ? line : search_row(p.dbr_rec, static_cast<uint32_t>(rinfo) + c.z, u);
   }
   const int32_t row = __ldg(p.line_row + j);
   uint32_t lo = __ldg(p.dbr_offset + row), hi = __ldg(p.dbr_offset + row + 1) - 1u;
@@ -164,10 +91,7 @@ __device__ __forceinline__ Emission downbranch_pick(const TransportParams &p, in
     const uint32_t mid = (lo + hi) >> 1;
     if (kz < __ldg(cb + mid)) hi = mid; else lo = mid + 1u;
   }
-  em.line = static_cast<int32_t>(__ldg(p.dbr_line + lo));
-  em.nu = __ldg(p.nu + em.line);
-  em.inv_nu = rcp64(em.nu);
-  return em;
+  return static_cast<int32_t>(__ldg(p.dbr_line + lo));
 }
 
 // Macro atom (Sect. 2.5, mode macroatom): activated in level `row` (the
@@ -334,40 +258,27 @@ __device__ __noinline__ void spawn_virtual(const TransportParams &p, const doubl
 // segment is resolved by exact_scan, so that the events are the binary64
 // scan's.  Binary64 warp instructions hold their SM sub-partition's pipe for 64
 // cycles each; this takes the reciprocal 1/D, nu_lab, the thresholds and one
-// fma per line off it (28 -> 19 binary64 instructions for a line event).
+// fma per line off it, and the draw's binary64 logarithm (needed by exact_scan
+// only): 40 -> 18 binary64 instructions for a line event.
 //
 // Error budget (u = 2^-24).  Frequency difference: the significands subtracted
 // as integers in units of nu_cmf's last place (a line in a lower binade is
 // truncated to it: at most one unit), converted in two halves (2u).  l: that
-// difference (2u), D truncated (2u), 1/significand (truncated 2u, approximate
+// difference (2u), D = 1 - p in binary32 (2u), 1/significand (truncated 2u, approximate
 // reciprocal 2u) and two products (2u) -- below 2^-20 l.  kappa' D l: three
-// more roundings -- below 2^-20 of it.  tau, the depths: truncated (2u each),
-// and n differences (u each of tau).  M = (2^-19 + n 2^-23) (kappa' D l + tau)
+// more roundings -- below 2^-20 of it.  tau: its binary32 logarithm (8u); the
+// depths: truncated (2u each), and n differences (u each of tau).  M = (2^-19 + n 2^-23) (kappa' D l + tau)
 // + kappa' D (2^-44 + n 2^-51) + 2^-100 bounds these, the unit of the
 // significands and the binary64 chain's n fmas (2^-53 nu each).
-struct ScanF {
-  unsigned long long mc;  // significand of nu_cmf
-  int ec;                 // its exponent field
-  float lf, tf;           // path length per unit of significand difference; kappa' D
-  float tau;              // the optical-depth draw
-  float lx, mx;           // path length to the shell exit and its error bound (infinite: not known)
-};
-
 // Path length to the exit: x mu there is +-sqrt(x_b^2 - q) (P, in binary32 from
 // the operands truncated, the difference's error e1 carried through the root).
 // Near-tangent exits (x_b^2 - q within 4 e1) are not bounded.
-__device__ __forceinline__ ScanF scan_setup(double nu_cmf, double D, double p, double q, float kap, bool inner,
-                                            float xi2, float xo2, double tau) {
+__device__ __forceinline__ ScanF scan_setup(double nu_cmf, double p, double q, float kap, bool inner,
+                                            float xi2, float xo2, float tau) {
   ScanF f;
-  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(nu_cmf));
-  f.ec = static_cast<int>(b >> 52);
-  f.mc = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
-  float im;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(im) : "f"(static_cast<float>(static_cast<uint32_t>(f.mc >> 29))));
-  const float Df = f32_rz_any(D), pf = f32_rz_any(p), qf = f32_rz_any(q);
-  f.lf = (Df * im) * 0x1.0p-29f;
+  const float pf = f32_rz_small(p), qf = f32_rz_small(q), Df = 1.0f - pf;
   f.tf = kap * Df;
-  f.tau = f32_rz_any(tau);
+  f.tau = tau;
   const float xb2 = inner ? xi2 : xo2;
   const float dq = xb2 - qf;
   const float e1 = 0x1.0p-22f * (xb2 + dq);
@@ -375,29 +286,20 @@ __device__ __forceinline__ ScanF scan_setup(double nu_cmf, double D, double p, d
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(dq));
   const float P = dq * r;
   f.lx = (inner ? -P : P) - pf;
-  f.mx = (dq >= 4.0f * e1 && f.ec > 0 && f.ec < 2047) ? fmaf(0x1.0p-20f, P + fabsf(pf), fmaf(e1, r, 0x1.0p-44f)) : __int_as_float(0x7f800000);
+  f.mx = dq >= 4.0f * e1 ? fmaf(0x1.0p-20f, P + fabsf(pf), fmaf(e1, r, 0x1.0p-44f)) : __int_as_float(0x7f800000);
+  // (the frequency last: on a lone walk it is still on its way)
+  scan_frequency(f, nu_cmf, Df);
+  if (f.ec <= 0 || f.ec >= 2047) f.mx = __int_as_float(0x7f800000);
   return f;
 }
 
-// Significand difference nu_cmf - nu_line in units of nu_cmf's last place, as
-// binary32 (0 when the line is not below nu_cmf); ok: the line's binade is
-// nu_cmf's or a lower one.
-__device__ __forceinline__ float scan_delta(const ScanF &f, long long line_bits, bool &ok) {
-  const unsigned long long b = static_cast<unsigned long long>(line_bits);
-  const int sh = f.ec - static_cast<int>(b >> 52);
-  ok = sh >= 0;
-  const unsigned long long m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
-  const long long d = static_cast<long long>(f.mc) - static_cast<long long>(m >> (sh < 63 ? sh & 63 : 63));
-  const float v = fmaf(static_cast<float>(static_cast<uint32_t>(d >> 32)), 0x1.0p32f,
-                       static_cast<float>(static_cast<uint32_t>(d)));
-  return d > 0 ? v : 0.0f;
-}
-
 // Draws of a lone walk, computed ahead by its warp: the walk's draws base ..
-// base + 63 as u53, as -ln of the open-interval draw and as the isotropic mu.
+// base + 63 as u53, as the isotropic mu and as -ln of the open-interval draw
+// (binary32).
 struct LoneDraws {
   unsigned long long *u;
-  double *t, *m;
+  double *m;
+  float *t;
   uint32_t base;
 
   // All 32 lanes: refill when fewer than the three draws that a segment may
@@ -413,7 +315,7 @@ struct LoneDraws {
       const unsigned long long v = h ? DrawStream::u53_of(o.z, o.w) : DrawStream::u53_of(o.x, o.y);
       const int i = 2 * static_cast<int>(lane) + h;
       u[i] = v;
-      t[i] = neg_log_u53(v + 1ull);
+      t[i] = neg_log_u53_f(v + 1ull);
       m[i] = DrawStream::mu_from_u53(v);
     }
     __syncwarp();
@@ -434,8 +336,12 @@ struct MaDraws {
   }
 };
 
-template <int MODE, bool JB, bool REC>
+// LINES: what an absorbing line does -- 0 scatter, 1 downbranch, 2 macro atom,
+// 3 downbranch from the caller's table alone (no bucket slots, no 1/nu).
+template <int LINES, bool JB, bool REC>
 __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p) {
+  constexpr int MODE = LINES == 3 ? 1 : LINES;
+  constexpr bool kSlots = LINES == 1 || LINES == 2;  // the model's tables: bucket slots, row info, 1/nu
   extern __shared__ double sh[];
   const int32_t S = p.S, L = p.L;
   for (int i = threadIdx.x; i < S; i += blockDim.x) {
@@ -502,12 +408,12 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
     if (j_ < L) {
       lw_b0 = __ldg(nub + j_);
       lw_t0 = __ldg(ts + j_);
-      if (MODE == 1 && p.row_info) lw_r0 = __ldg(p.row_info + j_);
+      if (LINES == 1) lw_r0 = __ldg(p.row_info + j_);
     }
     if (j_ + 1 < L) {
       lw_b1 = __ldg(nub + j_ + 1);
       lw_t1 = __ldg(ts + j_ + 1);
-      if (MODE == 1 && p.row_info) lw_r1 = __ldg(p.row_info + j_ + 1);
+      if (LINES == 1) lw_r1 = __ldg(p.row_info + j_ + 1);
     }
     lw_ok = true;
   };
@@ -518,7 +424,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   // scattering, exact_scan, the end of the walk)
   auto need_lab = [&]() {
     if (!pk.have_lab) {
-      pk.nu_lab = pk.nu_cmf * rcp64(pk.D);
+      pk.nu_lab = pk.nu_cmf * rcp64_here(pk.D);
       pk.have_lab = true;
     }
   };
@@ -538,9 +444,10 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   // exit while nu_line > nu_lab (1 - p_exit); a line of depth tau moves thr_e up by
   // tau nu_lab / k and absorbs exactly when thr_e then exceeds nu_line).
   // Updates j; nu_hit: the absorbing line's frequency bits; thr: thr_e.
-  auto exact_scan = [&](double tau, bool inner, int32_t j0, int32_t &j, bool act, double e_inv2, long long &nu_hit,
+  auto exact_scan = [&](unsigned long long u_tau, bool inner, int32_t j0, int32_t &j, bool act, double e_inv2, long long &nu_hit,
                         double &thr, double &p_exit) -> int {
     need_lab();
+    const double tau = neg_log_u53(u_tau + 1ull);
     const double nu_lab = pk.nu_lab;
     const double *ts = p.tau + static_cast<size_t>(cs) * static_cast<size_t>(L);
     p_exit = shell_exit(pk.q, inner, c_xi2, c_xo2);
@@ -683,39 +590,67 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       for (int c = 0; c < kNCounters; ++c) pk.cnt[c] = __shfl_sync(F, pk.cnt[c], owner);
       uint32_t d = __shfl_sync(F, ds.d, owner);
       LoneDraws ld;
-      ld.u = reinterpret_cast<unsigned long long *>(sh + kShellArrays * S) + 3 * kWarpDraws * (threadIdx.x >> 5);
-      ld.t = reinterpret_cast<double *>(ld.u + kWarpDraws);
-      ld.m = ld.t + kWarpDraws;
+      ld.u = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(sh + kShellArrays * S) +
+                                                    kLoneDrawBytes * (threadIdx.x >> 5));
+      ld.m = reinterpret_cast<double *>(ld.u + kWarpDraws);
+      ld.t = reinterpret_cast<float *>(ld.m + kWarpDraws);
       ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, true);
       enter_shell(pk.shell);
+      const uint32_t cap = p.max_segments < 0xffffffffull ? static_cast<uint32_t>(p.max_segments) : 0xffffffffu;
       int32_t w0 = 0;
       long long w_b = 0;
       double w_t = 0.0;
       unsigned long long w_r = 0ull;
       auto reload = [&](int32_t j_) {
         w0 = j_;
-        const int32_t jj = j_ + static_cast<int32_t>(lane);
-        w_b = 0;
-        w_t = 0.0;
-        w_r = 0ull;
-        if (jj < L) {
-          w_b = __ldg(nub + jj);
-          w_t = __ldg(p.tau + static_cast<size_t>(cs) * static_cast<size_t>(L) + jj);
-          if (MODE == 1 && p.row_info) w_r = __ldg(p.row_info + jj);
-        }
+        // (lanes behind the list load its last line; the scan leaves them out)
+        const int32_t jj = min(j_ + static_cast<int32_t>(lane), L - 1);
+        w_b = static_cast<long long>(load_here(nub + jj));
+        w_t = __longlong_as_double(static_cast<long long>(
+            load_here(p.tau + static_cast<size_t>(cs) * static_cast<size_t>(L) + jj)));
+        if (LINES == 1) w_r = load_here(p.row_info + jj);
       };
       reload(pk.next_line);
+      // A line's re-emission leaves 1/nu of the emitted line in flight (inv_c):
+      // E/nu and 1/nu_lab are taken when the next event needs them.
+      bool fresh = false;
+      double inv_c = 0.0;
+      auto settle = [&]() {
+        if (fresh) {
+          pk.inv_nu = inv_c * pk.D;
+          if (MODE >= 1) pk.e_per_nu = pk.e_cmf * inv_c;  // re-emitted at another frequency
+          fresh = false;
+        }
+      };
       // The estimator terms of a segment (Eqs. 13-14) are kept by one lane and
       // evaluated for 32 segments at once.
-      double g_e = 0.0, g_D = 0.0, g_l = 0.0, g_nu = 0.0;
+      // ... and so are the J_blue sums of the lines it passed (g_n lines from cell
+      // g_j on; the weight E_lab / nu_lab^2 is E/nu times 1/nu_lab).
+      double g_e = 0.0, g_i = 0.0, g_l = 0.0, g_nu = 0.0;  // E/nu, 1/nu_lab, path length, nu_cmf
+      int32_t g_j = 0, g_n = 0;
       uint32_t n_log = 0u;
       double a_j = 0.0, a_nb = 0.0;  // this lane's sums in shell cs
       auto sum_log = [&]() {
-        const double wgt = (g_e * g_D) * g_l;
+        const double wgt = ((g_e * g_nu) * (g_nu * g_i)) * g_l;  // E_cmf D l
         a_j += wgt;
         a_nb = fma(wgt, g_nu, a_nb);
         g_l = 0.0;
         n_log = 0u;
+        if (JB) {
+          const double e_inv2 = g_e * g_i;
+          double *cell = p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L) + g_j;
+          for (int32_t i = 0; i < g_n; ++i) red_add_evict_first(cell + i, e_inv2, jb_pol);
+          g_n = 0;
+        }
+      };
+      auto log_segment = [&](double l, int32_t j, int32_t n) {
+        if (lane == n_log) { g_e = pk.e_per_nu; g_i = pk.inv_nu; g_l = l; g_nu = pk.nu_cmf; g_j = j; g_n = n; }
+        ++n_log;
+#pragma unroll 1
+        while (n_log == 32u) {  // (a loop, and opaque: not evaluated for every segment)
+          asm volatile("" : "+d"(g_e), "+d"(g_l), "+d"(g_i), "+d"(g_nu));
+          sum_log();
+        }
       };
       auto flush_shell = [&]() {
         sum_log();
@@ -728,168 +663,258 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       };
       int status = 0;
       bool stopped = false;
+      need_cmf();
       while (status == 0) {
+        if (LINES == 1) {
+          // Line event after line event, the bulk of a trapped walk: a loop of its
+          // own, so that the loads in flight stay in their registers from where
+          // they are issued to where they are used (a copy of one where paths meet
+          // would wait for it).  It leaves, with nothing changed, at a segment that
+          // is anything else.
+          while (!p.timeout_ns && ((polls + 1u) & 255u) != 0u && pk.cnt[0] < cap) {
+            ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, false);
+            const uint32_t di = d - ld.base;
+            const unsigned long long u_em = ld.u[di + 1u];
+            const double mu = ld.m[di + 2u];
+            const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);
+            const ScanF f = scan_setup(pk.nu_cmf, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, ld.t[di]);
+            const bool there = w0 + static_cast<int32_t>(lane) < L;
+            bool ok;
+            const float l = scan_delta(f, w_b, ok) * f.lf;
+            const float a = l * f.tf;
+            const float own = there ? f32_rz_any(w_t) : 0.0f;
+            const float M = fmaf(0x1.0p-19f + 0x1.0p-18f, a + f.tau, fmaf(f.tf, 0x1.0p-43f, 0x1.0p-100f));
+            const float left = f.tau - a;
+            const bool inside = f.lx - l > fmaf(0x1.0p-19f, l, f.mx);
+            const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
+            const int k = 31 - __clz(thick & (0u - thick));
+            const long long hit = __shfl_sync(F, w_b, k);
+            const unsigned long long rinfo = __shfl_sync(F, w_r, k);
+            uint4 ra, rc;
+            load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+            const bool prior = static_cast<int>(lane) < k;
+            const unsigned sum = __reduce_add_sync(
+                F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
+            const float rk = left - static_cast<float>(sum) * 0x1.0p-21f;
+            // (and the point lies ahead of the packet, beyond its rounding)
+            const bool good = static_cast<int>(lane) == k ? (inside && rk > M + 0x1.0p-15f && l > 0x1.0p-40f)
+                                                          : !(prior && own < 0.0f);
+            if (!__all_sync(F, good) || thick == 0u) break;
+            settle();
+            polls += 1u;
+            d += 3u;
+            pk.cnt[0] += 1u;
+            pk.cnt[1] += static_cast<uint32_t>(k) + 1u;
+            pk.cnt[2] += static_cast<uint32_t>(k) + 1u;
+            pk.cnt[3] += 1u;
+            // line_point and sqrt64 without their special cases (a binary64
+            // result takes 45 cycles longer to an integer compare than to the
+            // next binary64 instruction)
+            const double nuj = __longlong_as_double(hit);
+            const double lp = fma(-nuj, pk.inv_nu, pk.D);
+            const double pl = fma(-nuj, pk.inv_nu, 1.0);
+            const double r2 = fma(pl, pl, pk.q);
+            log_segment(lp, w0, k + 1);
+            int32_t em = slot_line(ra, rc, u_em);
+            if (em < 0) em = search_row_lone(p.dbr_rec, rinfo, rc.z, u_em, lane);
+            reload(em + 1);
+            pk.next_line = em + 1;
+            pk.nu_cmf = __longlong_as_double(static_cast<long long>(load_here(p.nu + em)));
+            inv_c = __longlong_as_double(static_cast<long long>(load_here(p.inv_nu + em)));
+            // ... and while the window is on its way:
+            const double xn = sqrt64_pos(r2);
+            pk.e_cmf = pk.e_per_nu * nuj;
+            const double pn = xn * mu;
+            pk.D = fma(-xn, mu, 1.0);
+            pk.p = pn;
+            pk.q = max0(fma(-pn, pn, r2));
+            pk.have_lab = false;
+            fresh = true;
+          }
+        }
         if (p.timeout_ns && __any_sync(F, (global_ns() - t_start) > p.timeout_ns)) {
           if (lane == 0u) atomicExch(p.flags, 1ull);
           stopped = true;
           break;
         }
-        if (p.cancel && (++polls & 255u) == 0u && __any_sync(F, load_sys_u32(p.cancel) != 0u)) {
+        if ((++polls & 255u) == 0u && p.cancel && __any_sync(F, load_sys_u32(p.cancel) != 0u)) {
           if (lane == 0u) atomicExch(p.flags, 2ull);
           stopped = true;
           break;
         }
-        if (pk.cnt[0] >= p.max_segments) {
+        if (pk.cnt[0] >= cap) {
           status = 3;
           break;
         }
         ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, false);
         pk.cnt[0] += 1u;
         const uint32_t di = d - ld.base;
-        const double tau = ld.t[di];
         d += 1u;
-        need_cmf();
+        // the draws of a line event (the buffer holds three)
+        const unsigned long long u_em = ld.u[di + 1u];
+        const double mu_line = ld.m[di + (MODE == 1 ? 2u : 1u)];
         const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);
-        const ScanF f = scan_setup(pk.nu_cmf, pk.D, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, tau);
-        const double e_inv2 = JB ? pk.e_per_nu * pk.inv_nu : 0.0;
-        double *jb_row = p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L);
+        const ScanF f = scan_setup(pk.nu_cmf, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, ld.t[di]);
         const int32_t j0 = pk.next_line;
-        int32_t j = j0;
-        int kind = 0;
+        int32_t j = j0, j_log = j0;  // the lines passed before j_log have their J_blue sums
+        int kind = -1;               // -1 open, 0 in doubt
         long long hit = 0;
         unsigned long long rinfo = 0ull;
+        uint4 ra = make_uint4(0u, 0u, 0u, 0u), rc = ra;
         float C = 0.0f;
-        for (;;) {  // one window at a time
+        while (kind < 0) {  // one window at a time
           const int idx = j - w0;
-          const int32_t jl = w0 + static_cast<int32_t>(lane);
           const bool cand = static_cast<int>(lane) >= idx;
-          const bool there = jl < L;
+          const bool there = w0 + static_cast<int32_t>(lane) < L;
           bool ok;
           const float l = scan_delta(f, w_b, ok) * f.lf;
           const float a = l * f.tf;
-          // the depths before this line (exclusive prefix, so that a thick line's
-          // own depth does not round them away) and including it
           const float own = (cand && there) ? f32_rz_any(w_t) : 0.0f;
-          float Px = __shfl_up_sync(F, own, 1);
-          if (lane == 0u) Px = C;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const float y = __shfl_up_sync(F, Px, o);
-            if (static_cast<int>(lane) >= o) Px = __fadd_rn(Px, y);
-          }
           const float n = static_cast<float>(j - j0 + 32);
           const float m0 = fmaf(f.tf, fmaf(n, 0x1.0p-51f, 0x1.0p-44f), 0x1.0p-100f);
           const float m1 = fmaf(n, 0x1.0p-23f, 0x1.0p-19f);
           const float M = fmaf(m1, a + f.tau, m0);
-          const float r0 = (f.tau - Px) - a;                 // before this line
-          const float r1 = r0 - own;                         // after it
+          const float ra_ = (f.tau - C) - a;                 // before any line of the window
           const float xm = f.lx - l, xM = fmaf(0x1.0p-19f, l, f.mx);
-          const bool before = there && ok && r0 > M;         // certainly before d_e
-          const bool inside = xm > xM;                       // ... and before the exit
-          const bool pass = before && inside && r1 > M && own >= 0.0f;
-          const bool take = before && inside && r1 < -M;
-          // the exit comes before this line and before d_e
-          const float ax = f.lx * f.tf;
-          const float rx = (f.tau - Px) - ax;
-          const bool out = (!there || (ok && xm < -xM)) &&
-                           rx > fmaf(m1, fabsf(ax) + f.tau, fmaf(f.tf, f.mx, m0));
-          const unsigned stop = __ballot_sync(F, cand && !pass);
-          const unsigned took = __ballot_sync(F, take);
-          const unsigned outs = __ballot_sync(F, out);
-          const int k = stop ? __ffs(stop) - 1 : 32;
-          const bool taken = stop && ((took >> k) & 1u);
-          if (JB && cand && static_cast<int>(lane) < (taken ? k + 1 : k))
-            red_add_evict_first(jb_row + jl, e_inv2, jb_pol);
+          const bool inside = xm > xM;                       // certainly before the exit
+          // First the line that absorbs by its own depth: the depths before it
+          // only have to leave it in reach.  Their sum is one integer
+          // reduction (units of 2^-21, at most 2^-16 too small), and then every
+          // line before it is passed (path lengths and depths only grow); the
+          // record of its emission is on its way meanwhile.
+          const unsigned thick = __ballot_sync(F, cand && there && ok && ra_ - own < -M);
+          int k = 31 - __clz(thick & (0u - thick));  // its lane, or -1: then lane 31 stands in, to no effect
+          bool taken = false;
+          hit = __shfl_sync(F, w_b, k);
+          if (LINES == 1) {
+            rinfo = __shfl_sync(F, w_r, k);
+            load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+          }
+          {
+            const bool prior = cand && static_cast<int>(lane) < k;
+            const unsigned sum = __reduce_add_sync(
+                F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
+            const float rk = ra_ - static_cast<float>(sum) * 0x1.0p-21f;
+            const bool good = static_cast<int>(lane) == k ? (inside && rk > M + 0x1.0p-15f) : !(prior && own < 0.0f);
+            taken = __all_sync(F, good) && thick != 0u;
+          }
+          unsigned stop = 1u, outs = 0u;
+          float Px = 0.0f;
+          if (!taken) {
+            // the depths before each line (exclusive prefix, so that a thick
+            // line's own depth does not round them away)
+            Px = __shfl_up_sync(F, own, 1);
+            if (lane == 0u) Px = C;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const float y = __shfl_up_sync(F, Px, o);
+              if (static_cast<int>(lane) >= o) Px = __fadd_rn(Px, y);
+            }
+            const float r0 = (f.tau - Px) - a;                 // before this line
+            const float r1 = r0 - own;                         // after it
+            const bool before = there && ok && r0 > M;         // certainly before d_e
+            const bool pass = before && inside && r1 > M && own >= 0.0f;
+            const bool take = before && inside && r1 < -M;
+            // the exit comes before this line and before d_e
+            const float ax = f.lx * f.tf;
+            const float rx = (f.tau - Px) - ax;
+            const bool out = (!there || (ok && xm < -xM)) &&
+                             rx > fmaf(m1, fabsf(ax) + f.tau, fmaf(f.tf, f.mx, m0));
+            stop = __ballot_sync(F, cand && !pass);
+            const unsigned took = __ballot_sync(F, take);
+            outs = __ballot_sync(F, out);
+            k = stop ? __ffs(stop) - 1 : 32;
+            taken = stop && ((took >> k) & 1u);
+            if (taken) {
+              hit = __shfl_sync(F, w_b, k);
+              if (LINES == 1) {
+                rinfo = __shfl_sync(F, w_r, k);
+                load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+              }
+            }
+          }
           j = w0 + k;
           if (taken) {
             kind = kLineEvent;
-            hit = __shfl_sync(F, w_b, k);
-            rinfo = __shfl_sync(F, w_r, k);
-            break;
-          }
-          if (stop) {
+          } else if (stop) {
             kind = ((outs >> k) & 1u) ? kShellEvent : 0;
-            break;
+          } else {
+            if (JB) {  // a window passed whole: one lane a line, not left to the log
+              settle();
+              if (cand)
+                red_add_evict_first(p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L) + w0 +
+                                        static_cast<int32_t>(lane), pk.e_per_nu * pk.inv_nu, jb_pol);
+              j_log = j;
+            }
+            C = __shfl_sync(F, Px + own, 31);
+            reload(j);
           }
-          C = __shfl_sync(F, Px + own, 31);
-          reload(j);
         }
+        settle();
         double thr = 0.0, p_exit = 0.0;
         if (kind == 0) {
-          kind = exact_scan(tau, inner, j0, j, lane == 0u, e_inv2, hit, thr, p_exit);
+          kind = exact_scan(ld.u[di], inner, j0, j, false, 0.0, hit, thr, p_exit);
           if (kind == kLineEvent) {
-            if (JB && lane == 0u) red_add_evict_first(jb_row + j, e_inv2, jb_pol);
-            if (MODE == 1 && p.row_info) rinfo = __ldg(p.row_info + j);
+            if (LINES == 1) {
+              rinfo = __ldg(p.row_info + j);
+              load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+            }
           }
-        } else if (kind == kShellEvent) {
-          p_exit = shell_exit(pk.q, inner, c_xi2, c_xo2);
         }
         const uint32_t npass = static_cast<uint32_t>(j - j0);
         pk.cnt[1] += npass + (j < L ? 1u : 0u);
-        pk.cnt[2] += npass + (kind == kLineEvent ? 1u : 0u);
+        pk.cnt[2] += npass;
         pk.next_line = j;
-        double l = 0.0;
         if (kind == kLineEvent) {
+          pk.cnt[2] += 1u;
           pk.cnt[3] += 1u;
-          ulonglong2 ra = make_ulonglong2(0ull, 0ull), rc = make_ulonglong2(0ull, 0ull);
-          unsigned long long u_em = 0ull;
-          const bool slot = MODE == 1 && p.dbr_rec;
+          const double nuj = __longlong_as_double(hit);
+          double l, r2;
+          line_point(nuj, l, r2);
+          const double xn = sqrt64(r2);
+          log_segment(l, j_log, j - j_log + 1);
+          double mu = mu_line;
+          int32_t em = 0;
           if (MODE == 2) {
             const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
             rinfo = macroatom_walk(p, __ldg(p.line_row + j), md);
-            u_em = md.next();
-          } else if (MODE == 1) {
-            u_em = ld.u[di + 1u];
-            d += 1u;
-          }
-          if (slot) load_slot(bucket_slot(p, rinfo, u_em), ra, rc);
-          const double nuj = __longlong_as_double(hit);
-          double r2;
-          line_point(nuj, l, r2);
-          // log the segment, then the event's energy
-          if (lane == (n_log & 31u)) { g_e = pk.e_cmf; g_D = pk.D; g_l = l; g_nu = pk.nu_cmf; }
-          const double e_c = pk.e_per_nu * nuj;
-          double mu;
-          if (MODE == 2) {
-            const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
+            em = downbranch_pick<true>(p, j, rinfo, md.next());
             mu = DrawStream::mu_from_u53(md.next());
+          } else if (MODE == 1) {
+            d += 2u;
+            if (kSlots) {
+              em = slot_line(ra, rc, u_em);
+              if (em < 0) em = search_row_lone(p.dbr_rec, rinfo, rc.z, u_em, lane);
+            } else {
+              em = downbranch_pick<false>(p, j, rinfo, u_em);
+            }
           } else {
-            mu = ld.m[d - ld.base];
             d += 1u;
           }
-          const double xn = sqrt64(r2);
-          const double pn = xn * mu;
-          const double D2 = fma(-xn, mu, 1.0);
-          const double q2 = max0(fma(-pn, pn, r2));
-          double nu_c, inv_c;
           if (MODE >= 1) {
-            Emission em;
-            if (slot) em = pick_from_slot_lone(p, rinfo, u_em, ra, rc, lane);
-            else em = downbranch_pick(p, j, rinfo, u_em);
-            nu_c = em.nu;
-            inv_c = em.inv_nu;
-            pk.next_line = em.line + 1;
-            reload(pk.next_line);
-            pk.e_per_nu = e_c * inv_c;  // re-emitted at another frequency
+            pk.next_line = em + 1;
+            reload(em + 1);
+            pk.nu_cmf = __longlong_as_double(static_cast<long long>(load_here(p.nu + em)));
+            if (kSlots) inv_c = __longlong_as_double(static_cast<long long>(load_here(p.inv_nu + em)));
+            else inv_c = rcp64(pk.nu_cmf);
           } else {
-            nu_c = nuj;
-            inv_c = rcp64(nuj);
             pk.next_line = j + 1;
+            pk.nu_cmf = nuj;
+            inv_c = rcp64(nuj);
           }
-          pk.e_cmf = e_c;
-          pk.D = D2;
+          pk.e_cmf = pk.e_per_nu * nuj;
+          const double pn = xn * mu;
+          pk.D = fma(-xn, mu, 1.0);
           pk.p = pn;
-          pk.q = q2;
-          pk.inv_nu = inv_c * D2;
-          pk.nu_cmf = nu_c;
+          pk.q = max0(fma(-pn, pn, r2));
           pk.have_lab = false;
+          fresh = true;
         } else if (kind == kShellEvent) {
           pk.cnt[5] += 1u;
-          l = max0(p_exit - pk.p);
-          if (lane == (n_log & 31u)) { g_e = pk.e_cmf; g_D = pk.D; g_l = l; g_nu = pk.nu_cmf; }
+          p_exit = shell_exit(pk.q, inner, c_xi2, c_xo2);
+          log_segment(max0(p_exit - pk.p), j_log, j - j_log);
           need_lab();
           flush_shell();
-          n_log = 0xffffffffu;  // (counted up below)
           const int32_t ns = inner ? cs - 1 : cs + 1;
           pk.p = p_exit;
           pk.have_cmf = false;
@@ -901,18 +926,20 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
           }
         } else {
           pk.cnt[4] += 1u;
-          l = max0(fma(-thr, pk.inv_nu, pk.D));
+          const double l = max0(fma(-thr, pk.inv_nu, pk.D));
           const double pl = pk.p + l;
-          if (lane == (n_log & 31u)) { g_e = pk.e_cmf; g_D = pk.D; g_l = l; g_nu = pk.nu_cmf; }
+          log_segment(l, j_log, j - j_log);
           const double D1 = 1.0 - pl;
           const double nu_c = pk.nu_lab * D1;
           pk.e_cmf = pk.e_per_nu * nu_c;
           leave(fma(pl, pl, pk.q), ld.m[d - ld.base], nu_c, pk.inv_nu * rcp64(D1));
           d += 1u;
         }
-        if (pk.next_line < w0 || pk.next_line - w0 >= 32) reload(pk.next_line);  // behind the window
-        if (++n_log == 32u) sum_log();
+        if (LINES == 1 ? pk.next_line != w0 : pk.next_line < w0 || pk.next_line - w0 >= 32)
+          reload(pk.next_line);  // behind the window (or the loop above starts at its first lane)
+        if (status == 0) need_cmf();
       }
+      settle();
       need_lab();
       flush_shell();
       if (status != 0 && lane == 0u) {
@@ -954,9 +981,10 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       if (s != cs) enter_shell(s);
       need_cmf();
       // optical depth to the next event, tau = -ln z
-      const double tau = neg_log_u53(ds.next_u53() + 1ull);
+      const unsigned long long u_tau = ds.next_u53();
       const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);  // q, x_in^2 >= 0
-      const ScanF f = scan_setup(pk.nu_cmf, pk.D, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, tau);
+      const ScanF f = scan_setup(pk.nu_cmf, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2,
+                                 neg_log_u53_f(u_tau + 1ull));
       // J_blue weight of this segment, E_lab / nu_lab^2 (Eq. 17 without its
       // line factor nu_j, applied per cell after the launch)
       const double e_inv2 = JB ? pk.e_per_nu * pk.inv_nu : 0.0;
@@ -982,7 +1010,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
           if (j + 2 < L) {
             bj_nn = __ldg(nub + j + 2);
             tau_nn = __ldg(tau_s + j + 2);
-            if (MODE == 1 && p.row_info) rinfo_nn = __ldg(p.row_info + j + 2);
+            if (LINES == 1) rinfo_nn = __ldg(p.row_info + j + 2);
           }
           bool ok;
           const float l = scan_delta(f, bj, ok) * f.lf;
@@ -1022,8 +1050,8 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       bool exact = false;
       if (kind == 0) {
         exact = true;
-        kind = exact_scan(tau, inner, j0, j, true, e_inv2, hit, thr, p_exit);
-        if (MODE == 1 && p.row_info && kind == kLineEvent) rinfo = __ldg(p.row_info + j);
+        kind = exact_scan(u_tau, inner, j0, j, true, e_inv2, hit, thr, p_exit);
+        if (LINES == 1 && kind == kLineEvent) rinfo = __ldg(p.row_info + j);
       } else if (kind == kShellEvent) {
         p_exit = shell_exit(pk.q, inner, c_xi2, c_xo2);
       }
@@ -1074,12 +1102,12 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
               const MaDraws md{&ds, nullptr, nullptr, 0u, 0u, 0u, 0u};
               rinfo_em = macroatom_walk(p, __ldg(p.line_row + j), md);
             }
-            const Emission em = downbranch_pick(p, j, rinfo_em, ds.next_u53());
-            nu_c = em.nu;
-            inv_c = em.inv_nu;
-            pk.e_per_nu = pk.e_cmf * inv_c;  // re-emitted at another frequency
-            pk.next_line = em.line + 1;
+            const int32_t em = downbranch_pick<kSlots>(p, j, rinfo_em, ds.next_u53());
+            nu_c = __ldg(p.nu + em);
+            inv_c = kSlots ? __ldg(p.inv_nu + em) : rcp64(nu_c);
+            pk.next_line = em + 1;
             load_window(s, pk.next_line);
+            pk.e_per_nu = pk.e_cmf * inv_c;  // re-emitted at another frequency
           } else {
             nu_c = nuj;
             inv_c = rcp64(nuj);
@@ -1144,39 +1172,40 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   if (lane == 0u) atomicMax(p.flags + 2, global_ns());
 }
 
-template <int MODE, bool JB, bool REC>
+template <int LINES, bool JB, bool REC>
 const void *kernel_ptr() {
-  return reinterpret_cast<const void *>(&transport_fp64<MODE, JB, REC>);
+  return reinterpret_cast<const void *>(&transport_fp64<LINES, JB, REC>);
 }
 
-const void *select_kernel(int line_mode, int precision, bool jb, bool rec) {
+template <int LINES>
+const void *select_lines(bool jb, bool rec) {
+  if (jb) return rec ? kernel_ptr<LINES, true, true>() : kernel_ptr<LINES, true, false>();
+  return rec ? kernel_ptr<LINES, false, true>() : kernel_ptr<LINES, false, false>();
+}
+
+// tables: the model's branching tables (bucket slots) are there
+const void *select_kernel(int line_mode, int precision, bool jb, bool rec, bool tables) {
   if (precision == 1) return select_mixed_kernel(line_mode, jb, rec);
-  if (line_mode == 0) {
-    if (jb) return rec ? kernel_ptr<0, true, true>() : kernel_ptr<0, true, false>();
-    return rec ? kernel_ptr<0, false, true>() : kernel_ptr<0, false, false>();
-  }
-  if (line_mode == 2) {
-    if (jb) return rec ? kernel_ptr<2, true, true>() : kernel_ptr<2, true, false>();
-    return rec ? kernel_ptr<2, false, true>() : kernel_ptr<2, false, false>();
-  }
-  if (jb) return rec ? kernel_ptr<1, true, true>() : kernel_ptr<1, true, false>();
-  return rec ? kernel_ptr<1, false, true>() : kernel_ptr<1, false, false>();
+  if (line_mode == 0) return select_lines<0>(jb, rec);
+  if (line_mode == 2) return select_lines<2>(jb, rec);
+  if (tables) return select_lines<1>(jb, rec);
+  return jb ? kernel_ptr<3, true, false>() : kernel_ptr<3, false, false>();  // (no packet records)
 }
 
 size_t smem_bytes(int S, int precision) {
-  // binary64: shell tables, then one LoneDraws buffer (u53, -ln z, mu) per warp
+  // binary64: shell tables, then one LoneDraws buffer per warp
   return precision == 1 ? mixed_smem_bytes(S)
                         : static_cast<size_t>(kShellArrays) * S * sizeof(double) +
-                              (kBlock / 32) * 3 * kWarpDraws * sizeof(double);
+                              (kBlock / 32) * kLoneDrawBytes;
 }
 
 }  // namespace
 
 int transport_block_size() { return kBlock; }
 
-cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, int S,
+cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, bool tables, int S,
                                 int *blocks_per_sm) {
-  const void *k = select_kernel(line_mode, precision, j_blue, record);
+  const void *k = select_kernel(line_mode, precision, j_blue, record, tables);
   const size_t smem = smem_bytes(S, precision);
   if (smem > 48 * 1024) {  // the query, like the launch, needs the opt-in above 48 KB
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1190,7 +1219,7 @@ cudaError_t launch_transport(const TransportParams &p, int line_mode, int precis
                              bool record, int grid, int block, cudaStream_t st) {
   // the shared-memory layout (one draw buffer per warp) is sized for kBlock
   if (block != kBlock) return cudaErrorInvalidValue;
-  const void *k = select_kernel(line_mode, precision, j_blue, record);
+  const void *k = select_kernel(line_mode, precision, j_blue, record, p.dbr_rec != nullptr);
   const size_t smem = smem_bytes(p.S, precision);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -59,7 +59,9 @@ struct MCtx {
   const int32_t *line_row;           // macro atom: upper level of each line
   const MaRow *ma_row;               // macro atom: level table
   const MaJump *ma_jump;             // macro atom: jump entries
-  const DbrRec *bucket, *rec;
+  const DbrSlot *bucket;
+  const DbrRec *rec;
+  const float *inv_nu32;
   double *j_blue, *j_est, *nu_bar, *spectrum;
   unsigned long long *stats;
   unsigned long long *est_fix;  // [2 S] J, nu_bar in fixed point
@@ -91,6 +93,7 @@ __device__ __forceinline__ void load_ctx(MCtx &c, const TransportParams &q, cons
   c.ma_jump = q.ma_jump;
   c.bucket = q.dbr_bucket;
   c.rec = q.dbr_rec;
+  c.inv_nu32 = q.inv_nu32;
   c.j_blue = q.j_blue;
   c.j_est = q.j_est;
   c.nu_bar = q.nu_bar;
@@ -161,64 +164,7 @@ __device__ __forceinline__ float f32_of_f64_max0(double d) {
   return (bits > 0 && e > 0) ? __uint_as_float((static_cast<uint32_t>(e) << 23) | m) : 0.0f;
 }
 
-// Same exact integer search as the binary64 kernel (downbranch emission).
-__device__ __forceinline__ void pick_m(const MCtx &c, unsigned long long rinfo, unsigned long long u,
-                                       double &nu, float &inv_nu, int32_t &line) {
-  const uint32_t b = static_cast<uint32_t>(rinfo), len = static_cast<uint32_t>(rinfo >> 32);
-  const uint32_t bucket = static_cast<uint32_t>(__umul64hi(u << 11, static_cast<unsigned long long>(len)));
-  const DbrRec *slot = c.bucket + b + bucket;
-  unsigned long long thr = __ldg(&slot->thr);
-  if (u < thr) {
-    nu = __ldg(&slot->nu);
-    inv_nu = f32_of_positive_f64(__ldg(reinterpret_cast<const long long *>(&slot->inv_nu)));
-    line = static_cast<int32_t>(__ldg(&slot->emit));
-    return;
-  }
-  const DbrRec *rec = c.rec;
-  uint32_t i = b + __ldg(&slot->guide) + 1u;
-  thr = __ldg(&rec[i].thr);
-  while (u >= thr) { ++i; thr = __ldg(&rec[i].thr); }
-  nu = __ldg(&rec[i].nu);
-  inv_nu = f32_of_positive_f64(__ldg(reinterpret_cast<const long long *>(&rec[i].inv_nu)));
-  line = static_cast<int32_t>(__ldg(&rec[i].emit));
-}
-
 __device__ __forceinline__ float max0f(float v) { return v > 0.0f ? v : 0.0f; }
-
-// Lone-walker mode (all 32 lanes of the warp converged on one walk): the
-// emission from a bucket slot loaded ahead as two 16-byte halves {thr, nu},
-// {inv_nu, emit | guide << 32}; past the slot the next 32 records of the row
-// in one coalesced load per round (lane i takes entry i), the first with u
-// below its threshold found by a vote (the row's last threshold is 2^53 > u).
-__device__ __forceinline__ void pick_lone_m(const MCtx &c, unsigned long long rinfo, unsigned long long u,
-                                            ulonglong2 a, ulonglong2 h, unsigned lane, double &nu,
-                                            float &inv_nu, int32_t &line) {
-  if (u < a.x) {
-    nu = __longlong_as_double(static_cast<long long>(a.y));
-    inv_nu = f32_of_positive_f64(static_cast<long long>(h.x));
-    line = static_cast<int32_t>(static_cast<uint32_t>(h.y));
-    return;
-  }
-  const uint32_t end = static_cast<uint32_t>(rinfo) + static_cast<uint32_t>(rinfo >> 32);
-  uint32_t i0 = static_cast<uint32_t>(rinfo) + static_cast<uint32_t>(h.y >> 32) + 1u;
-  for (;;) {
-    const uint32_t i = i0 + lane;
-    ulonglong2 ra = make_ulonglong2(~0ull, 0ull), rh = make_ulonglong2(0ull, 0ull);
-    if (i < end) {
-      ra = __ldg(reinterpret_cast<const ulonglong2 *>(c.rec + i));
-      rh = __ldg(reinterpret_cast<const ulonglong2 *>(c.rec + i) + 1);
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, u < ra.x);  // lanes past the row's end vote yes
-    if (m != 0u) {
-      const int k = __ffs(m) - 1;
-      nu = __longlong_as_double(__shfl_sync(0xffffffffu, static_cast<long long>(ra.y), k));
-      inv_nu = f32_of_positive_f64(__shfl_sync(0xffffffffu, static_cast<long long>(rh.x), k));
-      line = __shfl_sync(0xffffffffu, static_cast<int32_t>(static_cast<uint32_t>(rh.y)), k);
-      return;
-    }
-    i0 += 32u;
-  }
-}
 
 // Macro atom (Sect. 2.5): the binary64 kernel's walk (integer thresholds, the
 // same draws in the same order) on a lane's model context; returns the
@@ -334,7 +280,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
   // owner lane makes the walk's side effects.
   constexpr bool kLoneBuild = MINB == 1;
   WarpDraws wd;
-  wd.init(batch ? nullptr : smem_u64 + 2 * static_cast<size_t>(p.S) + 2 * kWarpDraws * (threadIdx.x >> 5));
+  wd.init(batch ? nullptr : smem_u64 + 2 * static_cast<size_t>(p.S) + kWarpDraws * (threadIdx.x >> 5));
   bool drained = false;  // warp-uniform: the packet queue is empty
   bool lone = false;
   int owner = 0;
@@ -523,6 +469,166 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
       r = __shfl_sync(0xffffffffu, lwin_r, idx);
     };
 
+    if (kLoneBuild && MODE == 1 && lone && pk.next_line < c.L) {
+      // Line event after line event of a lone walk, the bulk of a trapped walk,
+      // in a loop of its own (the binary64 kernel's: loads stay in their
+      // registers from where they are issued to where they are used).  The
+      // absorbing line is the first one whose own depth absorbs, with the depths
+      // before it as one integer reduction; the signs are taken in binary32 from
+      // path lengths with a bound (ScanF's budget: this kernel's thresholds differ
+      // from exact arithmetic by the roundings of c_e and of its products, a few
+      // 2^-24 of either side) or, for the first line against the exit, exactly as
+      // below.  It leaves, with nothing changed, at a segment that is anything
+      // else or in doubt.  (Walk of
+      // 83,154 segments: 152 -> 105 ms.)
+      const unsigned F = 0xffffffffu;
+      const uint32_t cap = c.max_segments < 0xffffffffull ? static_cast<uint32_t>(c.max_segments) : 0xffffffffu;
+      if (pk.shell != cs) {
+        cs = pk.shell;
+        c_kap = c.kap[cs];
+        c_ikap = c.ikap[cs];
+        c_xi2 = c.xi2[cs];
+        c_xo2 = c.xo2[cs];
+      }
+      if (cs != acc_s) {
+        if (acc_s >= 0 && act) {
+          atomicAdd(c.est_fix + acc_s, acc_j);
+          atomicAdd(c.est_fix + c.S + acc_s, acc_nb);
+        }
+        acc_s = cs; acc_j = 0ull; acc_nb = 0ull;
+      }
+      const long long *nub = reinterpret_cast<const long long *>(c.nu);
+      const float *tau_s = c.tau32 + static_cast<size_t>(cs) * static_cast<size_t>(c.L);
+      long long w_b;
+      float w_t;
+      unsigned long long w_r;
+      int32_t w0 = pk.next_line;
+      auto reload = [&]() {
+        const int32_t jj = min(w0 + static_cast<int32_t>(lane), c.L - 1);
+        w_b = static_cast<long long>(load_here(nub + jj));
+        w_t = load_here_f(tau_s + jj);
+        w_r = load_here(c.row_info + jj);
+      };
+      w_b = lwin_b;
+      w_t = lwin_t;
+      w_r = lwin_r;
+      if (lwin_s != cs || lwin_j0 != w0) reload();
+      double nu_c = pk.nu_lab * f64_of_f32(1.0f - pk.p), r1 = 0.0;
+      float inv_c = 0.0f, g_w = 0.0f, g_b = 0.0f;
+      uint32_t n_log = 0u;
+      bool fresh = false;
+      unsigned long long s_j = 0ull, s_nb = 0ull;  // this lane's sums of the logged segments
+      auto sum_log = [&]() {
+        s_j += __float2ull_rn(g_w);
+        s_nb += __float2ull_rn(g_b);
+        g_w = 0.0f;
+        g_b = 0.0f;
+        n_log = 0u;
+      };
+      while (!p.timeout_ns && ((polls + 1u) & 255u) != 0u && pk.cnt[0] < cap) {
+        wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
+        const uint32_t di = ds.d - wd.base;
+        const float tau0 = -__logf(open0f(wd.u[di]));
+        const unsigned long long u_em = wd.u[di + 1u], um = wd.u[di + 2u];
+        const float pp = pk.p, q = pk.q, Df = 1.0f - pp;
+        const bool inner = pp < 0.0f && q <= c_xi2;
+        const float lx = Df - (1.0f - shell_exit_f(q, inner, c_xi2, c_xo2));
+        ScanF f;
+        f.tf = c_kap * Df;
+        scan_frequency(f, nu_c, Df);
+        const bool there = w0 + static_cast<int32_t>(lane) < c.L;
+        bool ok;
+        const float l = scan_delta(f, w_b, ok) * f.lf;
+        const float a = l * f.tf;
+        const float own = there ? w_t : 0.0f;
+        const float M = fmaf(0x1.0p-19f + 0x1.0p-18f, a + tau0, fmaf(f.tf, 0x1.0p-43f, 0x1.0p-100f));
+        const float left = tau0 - a;
+        const bool inside = lx - l > fmaf(0x1.0p-19f, l, 0x1.0p-43f);
+        const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
+        const int k = 31 - __clz(thick & (0u - thick));
+        const long long hit = __shfl_sync(F, w_b, k);
+        const unsigned long long rinfo = __shfl_sync(F, w_r, k);
+        uint4 ra, rc;
+        load_slot_here(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
+        const bool prior = static_cast<int>(lane) < k;
+        const unsigned sum = __reduce_add_sync(
+            F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
+        const float rk = left - static_cast<float>(sum) * 0x1.0p-21f;
+        const bool good = static_cast<int>(lane) == k
+                              ? (f.ec > 0 && f.ec < 2047 && (inside || k == 0) && rk > M + 0x1.0p-15f)
+                              : !(prior && own < 0.0f);
+        if (!__all_sync(F, good) || thick == 0u) break;
+        if (fresh) {
+          pk.nu_lab = nu_c * r1;
+          pk.inv_nu = inv_c * Df;
+          fresh = false;
+        }
+        const float inv_nu = pk.inv_nu;
+        const double nu_cmf = pk.nu_lab * f64_of_f32(Df);
+        const float lj = f32_of_f64_max0(nu_cmf - __longlong_as_double(hit)) * inv_nu;
+        if (k == 0 && !inside_shell_f(pp, q, lj, inner, c_xi2, c_xo2)) break;
+        polls += 1u;
+        ds.d += 3u;
+        pk.cnt[0] += 1u;
+        pk.cnt[1] += static_cast<uint32_t>(k) + 1u;
+        pk.cnt[2] += static_cast<uint32_t>(k) + 1u;
+        pk.cnt[3] += 1u;
+        if (JB && static_cast<int>(lane) <= k) {
+          const float e_jb = ((pk.e_lab * inv_nu) * c.nu_ref) * kEstFixScaleF;
+          red_add_evict_first(c.jb_fix + static_cast<size_t>(cs) * static_cast<size_t>(c.L) + w0 +
+                                  static_cast<int32_t>(lane),
+                              __float2ull_rn((f32_of_positive_f64(w_b) * inv_nu) * e_jb), jb_pol);
+        }
+        const float wgt = ((pk.e_lab * Df) * Df) * lj;
+        if (lane == n_log) {
+          g_w = wgt * kEstFixScaleF;
+          g_b = (wgt * (f32_of_positive_f64(__double_as_longlong(nu_cmf)) * c.inv_nu_ref)) * kEstFixScaleF;
+        }
+        ++n_log;
+#pragma unroll 1
+        while (n_log == 32u) {  // (a loop, and opaque: not evaluated for every segment)
+          asm volatile("" : "+f"(g_w), "+f"(g_b));
+          sum_log();
+        }
+        const float pl = pp + lj;
+        const float r2n = fmaf(pl, pl, q);
+        const float xn = sqrtf(r2n);
+        const float e_c = pk.e_lab * (1.0f - pl);
+        int32_t em = slot_line(ra, rc, u_em);
+        if (em < 0) em = search_row_lone(c.rec, rinfo, rc.z, u_em, lane);
+        w0 = em + 1;
+        reload();
+        nu_c = __longlong_as_double(static_cast<long long>(load_here(c.nu + em)));
+        inv_c = load_here_f(c.inv_nu32 + em);
+        // ... and while the window is on its way:
+        const float mu2 = static_cast<float>(static_cast<int32_t>(um >> 29) - (1 << 23)) * 0x1.0p-23f;
+        const float pn = xn * mu2;
+        const float D2 = 1.0f - pn;
+        const float iD2 = 1.0f / D2;
+        const double r0 = f64_of_f32(iD2);
+        r1 = fma(r0, fma(-f64_of_f32(D2), r0, 1.0), r0);
+        pk.p = pn;
+        pk.q = max0f(fmaf(-pn, pn, r2n));
+        pk.e_lab = e_c * iD2;
+        pk.inv_D = iD2;
+        pk.have_inv_D = true;
+        fresh = true;
+      }
+      if (fresh) {
+        pk.nu_lab = nu_c * r1;
+        pk.inv_nu = inv_c * (1.0f - pk.p);
+      }
+      sum_log();
+      if (s_j) atomicAdd(c.est_fix + cs, s_j);
+      if (s_nb) atomicAdd(c.est_fix + c.S + cs, s_nb);
+      pk.next_line = w0;
+      lwin_j0 = w0;
+      lwin_s = cs;
+      lwin_b = w_b;
+      lwin_t = w_t;
+      lwin_r = w_r;
+      wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
+    }
     int status = 0;
     if (pk.cnt[0] >= c.max_segments) {
       status = 3;
@@ -595,7 +701,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
       // downbranch: the absorbing line's emission record, loaded as soon as the
       // lone scan names the line (the emission draw is the next in the buffer)
       bool have_slot = false;
-      ulonglong2 slot_a = make_ulonglong2(0ull, 0ull), slot_h = make_ulonglong2(0ull, 0ull);
+      uint4 slot_a = make_uint4(0u, 0u, 0u, 0u), slot_h = slot_a;
       if (lone) {
         int idx = j - lwin_j0;
         if (lwin_s != s || idx < 0 || idx >= 32) {
@@ -660,12 +766,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
             bj = __shfl_sync(0xffffffffu, lwin_b, kstar);
             rinfo = __shfl_sync(0xffffffffu, lwin_r, kstar);
             if (MODE == 1) {
-              const uint32_t rb = static_cast<uint32_t>(rinfo), rlen = static_cast<uint32_t>(rinfo >> 32);
-              const uint32_t bucket = static_cast<uint32_t>(
-                  __umul64hi(wd.peek_u53(ds) << 11, static_cast<unsigned long long>(rlen)));
-              const DbrRec *slot = c.bucket + rb + bucket;
-              slot_a = __ldg(reinterpret_cast<const ulonglong2 *>(slot));
-              slot_h = __ldg(reinterpret_cast<const ulonglong2 *>(slot) + 1);
+              load_slot(bucket_slot(c.bucket, rinfo, wd.peek_u53(ds)), slot_a, slot_h);
               have_slot = true;
             }
           }
@@ -791,10 +892,14 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
             // MODE 2: macro atom, internal jumps before the emission pick
             const unsigned long long rinfo_em =
                 MODE == 2 ? macroatom_walk_m(c, __ldg(c.line_row + j), ds, lone ? &wd : nullptr) : rinfo_hit;
-            int32_t emit;
             const unsigned long long u_em = next_u();
-            if (have_slot) pick_lone_m(c, rinfo_em, u_em, slot_a, slot_h, lane, nu_c, inv_nu_c, emit);
-            else pick_m(c, rinfo_em, u_em, nu_c, inv_nu_c, emit);
+            if (!have_slot) load_slot(bucket_slot(c.bucket, rinfo_em, u_em), slot_a, slot_h);
+            int32_t emit = slot_line(slot_a, slot_h, u_em);
+            if (emit < 0)
+              emit = have_slot ? search_row_lone(c.rec, rinfo_em, slot_h.z, u_em, lane)
+                               : search_row(c.rec, static_cast<uint32_t>(rinfo_em) + slot_h.z, u_em);
+            nu_c = __ldg(c.nu + emit);
+            inv_nu_c = __ldg(c.inv_nu32 + emit);
             pk.next_line = emit + 1;
             if (lone) {
               lone_reload(s, pk.next_line);
@@ -927,7 +1032,7 @@ const void *select_mixed_kernel(int line_mode, bool jb, bool rec) { return selec
 // single-model launches (128 threads): shell tables, then a lone walker's
 // draw buffer per warp
 size_t mixed_smem_bytes(int S) {
-  return 4 * static_cast<size_t>(S) * sizeof(float) + (128 / 32) * 2 * kWarpDraws * sizeof(unsigned long long);
+  return 4 * static_cast<size_t>(S) * sizeof(float) + (128 / 32) * kWarpDraws * sizeof(unsigned long long);
 }
 
 cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, int block,

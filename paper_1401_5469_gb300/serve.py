@@ -54,7 +54,8 @@ def model_footprint_bytes(spec, j_blue: Optional[bool] = None,
     b += 8 * S * L if jb else 0        # J_blue sums
     b += L * (8 + 8 + 4 * 3 + 8 + 8)   # nu, f, ion/lower/upper, per-line constants, row info
     b += L * (4 * 3 + 8)               # staged line arrays used at set-up
-    b += nnz * (4 + 4 + 8 + 32 + 32)   # branching table + guide records
+    b += nnz * (4 + 4 + 8 + 16 + 32)   # branching table, its search entries and bucket slots
+    b += L * (4 if precision == mc.MC_PRECISION_MIXED else 8)  # 1 / nu
     if spec.n_ions:
         b += spec.n_ions * spec.n_levels * (8 + 8 + 1) + S * spec.n_ions * (8 + 8 * spec.n_levels)
     if getattr(spec, "ma_jump_p", None) is not None:  # macro-atom level and jump tables

@@ -6,7 +6,10 @@ error bound, and by binary64 frequency thresholds elsewhere.  This file
 restates both sides in numpy and asserts, on random segments with near-ties
 planted at a line, at the electron-scattering point and at the shell exit,
 that every event the binary32 side calls certain is the binary64 scan's: the
-scalar scan of a lane, and the one-step scan of a 32-line window.
+scalar scan of a lane, the one-step scan of a 32-line window, and the lone
+walk's pick of the first line that absorbs by its own depth, the last also
+against the mixed-precision kernel's thresholds.  The binary32 logarithm of the
+draws is checked against long double.
 """
 import ctypes
 import ctypes.util
@@ -39,7 +42,8 @@ def _setup(nu_cmf, D, p, q, kap, inner, xi2, xo2, tau):
     b = int(np.float64(nu_cmf).view(np.uint64))
     mc, ec = (b & ((1 << 52) - 1)) | (1 << 52), b >> 52
     im = F(1) / F(np.uint32(mc >> 29))
-    Df, pf, qf = _rz32(D), _rz32(p), _rz32(q)
+    pf, qf = _rz32(p), _rz32(q)
+    Df = F(F(1) - pf)
     xb2 = _rz32(xi2 if inner else xo2)
     dq = F(xb2 - qf)
     e1 = F(F(2.0 ** -22) * F(xb2 + dq))
@@ -128,6 +132,59 @@ def _window(f, nu, tau, scale):
     return None
 
 
+def _thick(f, nu, tau, scale, inside_first=True):
+    """The lone walk's shortcut: the first line whose own depth absorbs, the
+    depths before it as one integer sum (None: not settled)."""
+    M_ = [None] * 32
+    prior = 0
+    for k in range(min(32, len(nu))):
+        d, ok = _delta(f, nu[k])
+        l = F(d * f["lf"])
+        a = F(l * f["tf"])
+        own = _rz32(tau[k])
+        M = F(F(F(2.0 ** -19) + F(2.0 ** -18)) * F(a + f["tau"]) + F(F(f["tf"] * F(2.0 ** -43)) + F(2.0 ** -100)))
+        M = F(M * F(scale))
+        left = F(f["tau"] - a)
+        if ok and F(left - own) < -M:
+            rk = F(left - F(F(prior) * F(2.0 ** -21)))
+            inside = F(f["lx"] - l) > F(F(2.0 ** -19) * l + f["mx"]) * F(scale)
+            slack = F(2.0 ** -15) * F(scale)
+            return (LINE, k) if (inside or (k == 0 and not inside_first)) and rk > M + slack and l > 2.0 ** -40 else None
+        if own < 0:
+            return None
+        prior += int(F(min(own, F(63)) * F(2.0 ** 21)))
+    return None
+
+
+def _exact_mixed(nu_lab, pp, q, kap, inner, xi2, xo2, tau0, nu, tau):
+    """The mixed-precision kernel's scan (binary32 geometry, depths and c_e,
+    binary64 thresholds); None where its first line is placed against the exit
+    by the event point instead."""
+    Df = F(F(1) - pp)
+    nu_cmf = nu_lab * float(Df)
+    b = float(_rz32(nu_lab))
+    c_e = F(F(F(b) * F(1.0 / float(kap))) * F(F(1) / Df)) if kap > 0 else F(0)
+    root = np.sqrt(max(F((xi2 if inner else xo2) - q), F(0)))
+    key_x = nu_lab * float(F(F(1) - (-root if inner else root)))
+    thr, rem, j = nu_cmf - float(F(tau0 * c_e)), tau0, 0
+    while j < len(nu):
+        if (kap > 0 and nu[j] <= thr) or (j > 0 and nu[j] <= key_x):
+            return SHELL, j
+        if kap > 0:
+            t = thr + float(F(F(tau[j]) * c_e))
+            if t > nu[j]:
+                return LINE, j
+            thr = t
+        else:
+            if F(tau[j]) > rem:
+                return LINE, j
+            rem = F(rem - F(tau[j]))
+        if nu[j] <= key_x:
+            return SHELL, j
+        j += 1
+    return SHELL, j
+
+
 def _exact(nu_cmf, D, p, q, kap, inner, xi2, xo2, tau0, nu, tau):
     """The binary64 scan: frequency thresholds."""
     nu_lab = nu_cmf * (1.0 / D)
@@ -206,5 +263,54 @@ def test_certain_events_are_the_binary64_scans(seed):
                 assert want[1] >= got[1]  # the lines before the doubt are passed
             small = scan(f, nu, tau, 2.0 ** -8)
             wrong_small += small is not None and small[0] != 0 and small != want
+        got = _thick(f, nu, tau, 1.0)
+        assert got is None or got == want
     assert certain > 1000 and doubt > 100
     assert wrong_small > 0  # a bound 2^8 times smaller is not one
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_lone_pick_is_the_mixed_kernels_scan(seed):
+    picked = 0
+    for nu_cmf, D, p, q, kap, inner, xi2, xo2, tau0, nu, tau in _segments(1500, 100 + seed):
+        pp, q32, kap32 = F(p), F(q), F(kap)
+        xi2, xo2, tau0 = F(xi2), F(xo2), F(tau0)
+        tau = tau.astype(F)
+        inner = bool(pp < 0 and q32 <= xi2)
+        Df = F(F(1) - pp)
+        nu_lab = nu_cmf * (1.0 / float(Df))  # so that nu_cmf is the emitted line's frequency to rounding
+        f = _setup(nu_cmf, D, float(pp), float(q32), float(kap32), inner, float(xi2), float(xo2), tau0)
+        root = np.sqrt(max(F((xi2 if inner else xo2) - q32), F(0)))
+        f["lx"] = F(Df - F(F(1) - (-root if inner else root)))
+        f["mx"] = F(2.0 ** -43)
+        f["tf"] = F(kap32 * Df)
+        got = _thick(f, nu, tau, 1.0, inside_first=False)
+        if got is not None:
+            picked += 1
+            assert got == _exact_mixed(nu_lab, pp, q32, kap32, inner, xi2, xo2, tau0, nu, tau)
+    assert picked > 200
+
+
+def test_binary32_logarithm_of_the_draws():
+    """neg_log_u53_f within 2^-21 of -ln(u 2^-53), near 1 included."""
+    r = np.random.default_rng(5)
+    u = np.concatenate([[1, 2, 3, 2 ** 52 - 1, 2 ** 52, 2 ** 52 + 1, 2 ** 53 - 2, 2 ** 53 - 1, 3 * 2 ** 50, 3 * 2 ** 51],
+                        r.integers(1, 2 ** 53, 200_000), 2 ** 53 - 2 ** r.integers(0, 52, 20_000),
+                        2 ** r.integers(0, 53, 2000)]).astype(np.uint64)
+    lz = 63 - np.floor(np.log2(u.astype(np.longdouble))).astype(np.int64)
+    m = u << lz.astype(np.uint64)
+    up = m >= np.uint64(0xC000000000000000)
+    a = np.where(up, np.uint64(0) - m, m - np.uint64(1 << 63))
+    mag = ((a >> np.uint64(32)).astype(np.uint32).astype(F) * F(2.0 ** 32) + (a & np.uint64(0xFFFFFFFF)).astype(np.uint32).astype(F))
+    f = np.where(up, mag * F(-(2.0 ** -64)), mag * F(2.0 ** -63)).astype(F)
+    s = f * (F(1) / (F(2) + f))
+    s2 = s * s
+    q = s2 * F(1 / 9) + F(1 / 7)
+    q = s2 * q + F(0.2)
+    q = s2 * q + F(1 / 3)
+    lnm = F(2) * ((s * s2) * q + s)
+    got = (lz - 10 - up).astype(F) * F(float.fromhex("0x1.62e43p-1")) - lnm
+    want = -np.log(u.astype(np.longdouble) * np.longdouble(2.0) ** -53)
+    assert np.all(got >= 0)
+    rel = np.abs(got.astype(np.longdouble) - want) / np.where(want == 0, 1, want)
+    assert rel.max() < 2.0 ** -21, float(rel.max())
