@@ -358,7 +358,6 @@ mc_status mc_model_create(const mc_geometry_desc *geom, const mc_line_desc *line
             alloc_n(m, &m->t_rad, S) && alloc_n(m, &m->w, S) &&
             alloc_n(m, &m->norm, S) && alloc_n(m, &m->j_est, S) && alloc_n(m, &m->nu_bar, S) &&
             alloc_n(m, &m->spectrum, static_cast<size_t>(run->spec_bins) + 2) &&
-            alloc_n(m, &m->counters, static_cast<size_t>(kNCounterSlots)) &&
             alloc_n(m, &m->planck_cdf, static_cast<size_t>(kPlanckLmax) + 1);
   if (ok && run->j_blue) ok = alloc_n(m, &m->j_blue, SL);
   if (ok && run->precision == MC_PRECISION_MIXED)
@@ -546,6 +545,11 @@ mc_status mc_model_create(const mc_geometry_desc *geom, const mc_line_desc *line
   int nsm = 1;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
   m->grid = nsm * bps;
+  // the pool: every warp of the grid hands over at most kPoolLive - 1 walks, once
+  m->pool_cap = static_cast<uint32_t>(m->grid) * static_cast<uint32_t>(transport_block_size() / 32) * (kPoolLive - 1u);
+  m->n_counter_words = kNCounterSlots + 2 + (static_cast<size_t>(m->pool_cap) + 1) / 2;
+  if (!alloc_n(m, &m->counters, m->n_counter_words) || !alloc_n(m, &m->pool, m->pool_cap))
+    return bail(MC_ERR_OOM, "device allocation failed");
   e = cudaStreamSynchronize(m->stream);
   if (e != cudaSuccess) return bail(MC_ERR_CUDA, std::string("create: ") + cudaGetErrorString(e));
   *out = m;
@@ -657,7 +661,8 @@ mc_status model_prepare(mc_model *m, cudaStream_t st, bool events) {
     m->ran_plasma = events;
   }
   cudaError_t e = launch_zero(m->j_est, m->S, m->nu_bar, m->S, m->spectrum, m->run.spec_bins + 2,
-                              m->counters, kNCounterSlots, st);
+                              m->counters,
+                              events ? m->n_counter_words : static_cast<size_t>(kNCounterSlots), st);
   if (e != cudaSuccess) return cuda_fail(m, e, "zero");
   m->launches += 1;
   if (m->j_blue) {
@@ -718,6 +723,10 @@ void model_fill_transport(const mc_model *m, TransportParams &p, uint64_t seed, 
   p.stats = m->counters;
   p.work_counter = m->counters + kNStats;
   p.flags = m->counters + kNStats + 1;
+  p.pool = m->pool;
+  p.pool_cap = m->pool_cap;
+  p.pool_ctl = m->counters + kNCounterSlots;
+  p.pool_ready = reinterpret_cast<uint32_t *>(m->counters + kNCounterSlots + 2);
   p.spec_bins = static_cast<int32_t>(m->run.spec_bins);
   p.spec_lo = m->run.spec_nu_lo;
   p.spec_hi = m->run.spec_nu_hi;

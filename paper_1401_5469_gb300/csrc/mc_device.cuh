@@ -430,6 +430,48 @@ struct WarpDraws {
   __device__ __forceinline__ unsigned long long peek_u53(const DrawStream &ds) const { return u[ds.d - base]; }
 };
 
+// The pool of walks handed over.  A walk is written, then its place marked; a
+// taker reads the mark, then claims the place.  Nothing waits: a place given
+// out but not yet marked ends a taker's search, and the warp that is filling it
+// comes back to the pool after its own walk, so every walk is taken.
+__device__ __forceinline__ void pool_put(const TransportParams &p, unsigned place, const PoolWalk &w) {
+  p.pool[place] = w;
+  __threadfence();
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.pool_ready + place), "r"(1u) : "memory");
+}
+// The place of a walk to run, or -1.
+__device__ __forceinline__ int pool_take(const TransportParams &p) {
+  for (int tries = 0; tries < 256; ++tries) {  // (a failed claim: another warp took that one)
+    unsigned long long t, h;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(t) : "l"(p.pool_ctl + 1) : "memory");
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(h) : "l"(p.pool_ctl) : "memory");
+    if (t >= h || t >= p.pool_cap) return -1;
+    uint32_t ready;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(ready) : "l"(p.pool_ready + t) : "memory");
+    if (!ready) return -1;
+    if (atomicCAS(p.pool_ctl + 1, t, t + 1ull) == t) return static_cast<int>(t);
+  }
+  return -1;
+}
+
+// First index j with nu[j] < v (nu strictly descending), by a whole warp: 32
+// probes a round.
+__device__ __forceinline__ int32_t first_redward_warp(const double *nu, int32_t L, double v, unsigned lane) {
+  int32_t lo = 0, n = L;  // the answer is in [lo, lo + n]
+  while (n > 0) {
+    const int32_t step = (n + 31) >> 5;
+    const int32_t end = min((static_cast<int32_t>(lane) + 1) * step, n);  // this lane's probe is the last before it
+    const unsigned m = __ballot_sync(0xffffffffu, __double_as_longlong(__ldg(nu + lo + end - 1)) <
+                                                      __double_as_longlong(v));
+    if (m == 0u) return lo + n;
+    const int32_t k = __ffs(m) - 1;
+    const int32_t to = min((k + 1) * step, n) - 1;  // the answer is at most lo + to
+    lo += k * step;
+    n = to - k * step;
+  }
+  return lo;
+}
+
 // ln(x) for a positive normal binary64 x.
 __device__ __forceinline__ double log_pos(double x) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));

@@ -64,7 +64,10 @@ struct mc_model {
   double *spectrum_v = nullptr;  // [bins + 2] virtual-packet spectrum (allocated on first use)
   uint32_t n_virtual = 0;
   double tau_v_max = 0.0;
-  unsigned long long *counters = nullptr;  // stats [kNStats], work counter, flags
+  unsigned long long *counters = nullptr;  // stats [kNStats], work counter, flags; then the pool's words
+  size_t n_counter_words = 0;
+  mcgpu::PoolWalk *pool = nullptr;         // [pool_cap] walks handed between warps
+  uint32_t pool_cap = 0;
   double *planck_cdf = nullptr;
   int32_t *rec_status = nullptr;
   double *rec_nu = nullptr, *rec_e = nullptr;

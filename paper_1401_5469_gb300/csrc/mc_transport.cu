@@ -37,7 +37,8 @@ namespace mcgpu {
 namespace {
 
 constexpr int kBlock = 128;
-constexpr size_t kLoneDrawBytes = kWarpDraws * (2 * sizeof(double) + sizeof(float));
+// per warp: a walk handed to all lanes, then its draws
+constexpr size_t kLoneBytes = sizeof(PoolWalk) + kWarpDraws * (2 * sizeof(double) + sizeof(float));
 constexpr int kShellArrays = 6;  // x_in^2, x_out^2, x_in, x_out, kappa, 1/kappa
 constexpr int kLineEvent = 1, kElectronEvent = 2, kShellEvent = 3;
 
@@ -159,7 +160,6 @@ __device__ __forceinline__ double inject(const TransportParams &p, const double 
   pk.have_cmf = true;
   pk.have_lab = false;
   pk.shell = 0;
-  pk.next_line = first_redward(p.nu, p.L, nu_cmf);
 #pragma unroll
   for (int c = 0; c < kNCounters; ++c) pk.cnt[c] = 0u;
   return nu_cmf;
@@ -369,8 +369,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   // serves a warp instruction for one lane or 32 in the same time.  (1000
   // packets of a 200-line scatter model: 126 -> 81 us with this and the scan.)
   const unsigned long long n_warps = static_cast<unsigned long long>(gridDim.x) * (kBlock / 32);
-  const unsigned quota = static_cast<unsigned>(
-      min(32ull, (p.n_packets + n_warps - 1ull) / n_warps));
+  const unsigned quota = static_cast<unsigned>(min(32ull, (p.n_packets + n_warps - 1ull) / n_warps));
 
   Packet pk{};
   DrawStream ds;
@@ -524,10 +523,11 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
           pk.pid = static_cast<uint32_t>(p.first_packet + id);
           ds.init(p.key0, p.key1, pk.pid, p.iteration);
           const double nu_cmf0 = inject(p, p.planck_cdf, x0, x0sq, pk, ds);
+          if (quota != 1u) pk.next_line = first_redward(p.nu, L, nu_cmf0);
           alive = true;
           lw_ok = false;
           vdraws = 0u;
-          if (p.n_virtual) {
+          if (p.n_virtual && quota != 1u) {
             spawn_virtual(p, sh, VirtualLaunch{x0, x0sq, nu_cmf0, p.e_cmf, 0, pk.next_line, pk.pid, 0u, true});
             vdraws = static_cast<uint32_t>(p.n_virtual);
           }
@@ -538,7 +538,20 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       }
     }
     const unsigned live = __ballot_sync(0xffffffffu, alive);
-    if (!live && __all_sync(0xffffffffu, finished)) break;
+    if (quota == 1u && needmask && live) {  // the one packet just claimed
+      const int32_t j = first_redward_warp(p.nu, L, __shfl_sync(0xffffffffu, pk.nu_cmf, 0), lane);
+      pk.next_line = j;
+      if (p.n_virtual && lane == 0u) {
+        spawn_virtual(p, sh, VirtualLaunch{x0, x0sq, pk.nu_cmf, p.e_cmf, 0, j, pk.pid, 0u, true});
+        vdraws = static_cast<uint32_t>(p.n_virtual);
+      }
+    }
+    int from_pool = -1;
+    if (!live && __all_sync(0xffffffffu, finished)) {
+      if (p.pool && lane == 0u) from_pool = pool_take(p);
+      from_pool = __shfl_sync(0xffffffffu, from_pool, 0);
+      if (from_pool < 0) break;
+    }
     if (p.timeout_ns) {
       bool late = false;
       if (lane == 0u) late = (global_ns() - t_start) > p.timeout_ns;
@@ -557,41 +570,78 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
         break;
       }
     }
-    if ((drained || quota == 1u) && __popc(live) == 1 && !p.n_virtual) {
-      // ---- lone walk: the queue is empty and one walk of the warp is left.
-      // All 32 lanes take its state and run it to its end, the line list 32
-      // lines at a time (line w0 + lane in each lane, one coalesced load), the
-      // scan of such a window in one step, its draws computed ahead; lane 0
-      // makes the walk's side effects.  The chain of a line event is then two
-      // dependent loads (the emission record, the window behind the emitted
-      // line) and the scan; the event's binary64 arithmetic runs while they
-      // are in flight.
+    const unsigned n_live = __popc(live);
+    bool go_lone = from_pool >= 0;
+    if (!p.n_virtual && (drained || quota == 1u) && n_live != 0u && n_live <= (p.pool ? kPoolLive : 1u))
+      go_lone = n_live == 1u || __all_sync(0xffffffffu, !alive || pk.cnt[0] >= kPoolAge);
+    if (go_lone) {
+      // ---- lone walk: the queue is empty and few walks of the warp are left (or
+      // the launch has few packets for each warp).  The warp hands all but the
+      // oldest to the pool -- walk lengths are heavy-tailed, so that the oldest is
+      // expected to be the longest -- and runs that one with all 32 lanes to its
+      // end, then takes others from the pool.  A walk that shares its warp
+      // advances at 4 to 8 us a segment, a lone one at 1.1 (1.7 with all warps of
+      // the SM in this mode).
+      // All 32 lanes hold the walk's state; the line list comes 32 lines at a
+      // time (line w0 + lane in each lane, one coalesced load), the scan of such a
+      // window in one step, the draws computed ahead; lane 0 makes the walk's side
+      // effects.  The chain of a line event is then two dependent loads (the
+      // emission record, the window behind the emitted line) and the scan; the
+      // event's binary64 arithmetic runs while they are in flight.
       const unsigned F = 0xffffffffu;
-      const int owner = __ffs(live) - 1;
       if (acc_s >= 0) {
         atomicAdd(p.j_est + acc_s, acc_j);
         atomicAdd(p.nu_bar + acc_s, acc_nb);
       }
       acc_s = -1;
-      pk.p = __shfl_sync(F, pk.p, owner);
-      pk.q = __shfl_sync(F, pk.q, owner);
-      pk.nu_lab = __shfl_sync(F, pk.nu_lab, owner);
-      pk.e_per_nu = __shfl_sync(F, pk.e_per_nu, owner);
-      pk.inv_nu = __shfl_sync(F, pk.inv_nu, owner);
-      pk.D = __shfl_sync(F, pk.D, owner);
-      pk.nu_cmf = __shfl_sync(F, pk.nu_cmf, owner);
-      pk.e_cmf = __shfl_sync(F, pk.e_cmf, owner);
-      pk.shell = __shfl_sync(F, pk.shell, owner);
-      pk.next_line = __shfl_sync(F, pk.next_line, owner);
-      pk.pid = __shfl_sync(F, pk.pid, owner);
-      pk.have_cmf = __shfl_sync(F, static_cast<int>(pk.have_cmf), owner) != 0;
-      pk.have_lab = __shfl_sync(F, static_cast<int>(pk.have_lab), owner) != 0;
+      char *warp_mem = reinterpret_cast<char *>(sh + kShellArrays * S) + kLoneBytes * (threadIdx.x >> 5);
+      const PoolWalk *from = p.pool + from_pool;
+      if (from_pool < 0) {
+        const unsigned age = alive ? pk.cnt[0] + 1u : 0u;
+        const unsigned oldest = __reduce_max_sync(F, age);
+        const int owner = __ffs(__ballot_sync(F, age == oldest)) - 1;
+        PoolWalk w;
+        w.f[0] = pk.p; w.f[1] = pk.q; w.f[2] = pk.inv_nu; w.f[3] = pk.e_per_nu;
+        w.f[4] = pk.D; w.f[5] = pk.nu_cmf; w.f[6] = pk.e_cmf; w.f[7] = pk.nu_lab;
+        w.i[0] = static_cast<uint32_t>(pk.shell);
+        w.i[1] = static_cast<uint32_t>(pk.next_line);
+        w.i[2] = pk.pid;
+        w.i[3] = ds.d;
+        w.i[4] = (pk.have_cmf ? 1u : 0u) | (pk.have_lab ? 2u : 0u);
+        w.i[5] = 0u;
 #pragma unroll
-      for (int c = 0; c < kNCounters; ++c) pk.cnt[c] = __shfl_sync(F, pk.cnt[c], owner);
-      uint32_t d = __shfl_sync(F, ds.d, owner);
+        for (int c = 0; c < kNCounters; ++c) w.i[6 + c] = pk.cnt[c];
+#pragma unroll
+        for (int c = 12; c < 16; ++c) w.i[c] = 0u;
+        if (n_live > 1u) {
+          const unsigned others = live & ~(1u << owner);
+          unsigned long long place = 0ull;
+          if (lane == 0u) place = atomicAdd(p.pool_ctl, static_cast<unsigned long long>(n_live - 1u));
+          place = __shfl_sync(F, place, 0) + __popc(others & lanemask_lt);
+          // (the pool holds what every warp can hand over once)
+          if (((others >> lane) & 1u) && place < p.pool_cap) pool_put(p, static_cast<unsigned>(place), w);
+        }
+        if (static_cast<int>(lane) == owner) *reinterpret_cast<PoolWalk *>(warp_mem) = w;
+        from = reinterpret_cast<const PoolWalk *>(warp_mem);
+      }
+      __syncwarp();
+      uint32_t d;
+      {
+        const volatile PoolWalk *w = from;  // (another SM may have written it: not through L1)
+        pk.p = w->f[0]; pk.q = w->f[1]; pk.inv_nu = w->f[2]; pk.e_per_nu = w->f[3];
+        pk.D = w->f[4]; pk.nu_cmf = w->f[5]; pk.e_cmf = w->f[6]; pk.nu_lab = w->f[7];
+        pk.shell = static_cast<int32_t>(w->i[0]);
+        pk.next_line = static_cast<int32_t>(w->i[1]);
+        pk.pid = w->i[2];
+        d = w->i[3];
+        pk.have_cmf = (w->i[4] & 1u) != 0u;
+        pk.have_lab = (w->i[4] & 2u) != 0u;
+#pragma unroll
+        for (int c = 0; c < kNCounters; ++c) pk.cnt[c] = w->i[6 + c];
+      }
+      __syncwarp();
       LoneDraws ld;
-      ld.u = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(sh + kShellArrays * S) +
-                                                    kLoneDrawBytes * (threadIdx.x >> 5));
+      ld.u = reinterpret_cast<unsigned long long *>(warp_mem + sizeof(PoolWalk));
       ld.m = reinterpret_cast<double *>(ld.u + kWarpDraws);
       ld.t = reinterpret_cast<float *>(ld.m + kWarpDraws);
       ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, true);
@@ -1196,7 +1246,7 @@ size_t smem_bytes(int S, int precision) {
   // binary64: shell tables, then one LoneDraws buffer per warp
   return precision == 1 ? mixed_smem_bytes(S)
                         : static_cast<size_t>(kShellArrays) * S * sizeof(double) +
-                              (kBlock / 32) * kLoneDrawBytes;
+                              (kBlock / 32) * kLoneBytes;
 }
 
 }  // namespace

@@ -38,6 +38,7 @@ namespace {
 
 // single-model launches take 128 threads per block, batched ones 64, 128 or 256
 constexpr int kMaxBlock = 256;
+constexpr size_t kLoneWords = sizeof(PoolWalk) / sizeof(unsigned long long) + kWarpDraws;
 constexpr int kLineEvent = 1, kElectronEvent = 2, kShellEvent = 3;
 
 struct PacketM {
@@ -270,7 +271,11 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
 
   PacketM pk;
   DrawStream ds;
-  bool alive = false, finished = false;
+  // few packets are spread over all warps of the grid, so many to each (see the
+  // binary64 kernel)
+  const unsigned long long n_warps = static_cast<unsigned long long>(gridDim.x) * (blockDim.x >> 5);
+  const unsigned quota = static_cast<unsigned>(min(32ull, (p.n_packets + n_warps - 1ull) / n_warps));
+  bool alive = false, finished = lane >= quota;
   // Lone-walker mode (single-model build): once the packet queue is empty and
   // a warp is down to one live walk, every lane takes that walk's state and
   // runs its segments with the owner lane, as in the binary64 kernel: the
@@ -280,10 +285,10 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
   // owner lane makes the walk's side effects.
   constexpr bool kLoneBuild = MINB == 1;
   WarpDraws wd;
-  wd.init(batch ? nullptr : smem_u64 + 2 * static_cast<size_t>(p.S) + kWarpDraws * (threadIdx.x >> 5));
+  unsigned long long *warp_mem = smem_u64 + 2 * static_cast<size_t>(p.S) + kLoneWords * (threadIdx.x >> 5);
+  wd.init(batch ? nullptr : warp_mem + sizeof(PoolWalk) / sizeof(unsigned long long));
   bool drained = false;  // warp-uniform: the packet queue is empty
   bool lone = false;
-  int owner = 0;
   int32_t lwin_j0 = 0, lwin_s = -1;
   long long lwin_b = 0;
   float lwin_t = 0.0f;
@@ -370,7 +375,13 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         }
       }
     }
-    if (!lone && __all_sync(0xffffffffu, finished)) break;
+    int from_pool = -1;
+    if (!lone && __all_sync(0xffffffffu, finished && !alive)) {
+      if (!kLoneBuild || batch || !p.pool) break;
+      if (lane == 0u) from_pool = pool_take(p);
+      from_pool = __shfl_sync(0xffffffffu, from_pool, 0);
+      if (from_pool < 0) break;
+    }
     if (p.timeout_ns) {
       bool late = false;
       if (lane == 0u) late = (global_ns() - t_start) > p.timeout_ns;
@@ -392,53 +403,83 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
     if (kLoneBuild && !batch) {
       if (lone) {
         wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
-      } else if (drained) {
+      } else {
         const unsigned live = __ballot_sync(0xffffffffu, alive);
-        if (__popc(live) == 1) {
-          // the other lanes' packets are done: they hand their estimator sums
-          // over and take the walk's state
-          owner = __ffs(live) - 1;
-          if (!alive && acc_s >= 0) {
+        const unsigned n_live = __popc(live);
+        bool go_lone = from_pool >= 0;
+        if ((drained || quota == 1u) && n_live != 0u && n_live <= (p.pool ? kPoolLive : 1u))
+          go_lone = n_live == 1u || __all_sync(0xffffffffu, !alive || pk.cnt[0] >= kPoolAge);
+        if (go_lone) {
+          // the lanes hand their estimator sums over; the warp keeps its oldest
+          // walk, or takes one from the pool, and all lanes take its state
+          const unsigned F = 0xffffffffu;
+          if (acc_s >= 0) {
             atomicAdd(c.est_fix + acc_s, acc_j);
             atomicAdd(c.est_fix + c.S + acc_s, acc_nb);
           }
-          const unsigned F = 0xffffffffu;
-          pk.nu_lab = __shfl_sync(F, pk.nu_lab, owner);
-          pk.p = __shfl_sync(F, pk.p, owner);
-          pk.q = __shfl_sync(F, pk.q, owner);
-          pk.e_lab = __shfl_sync(F, pk.e_lab, owner);
-          pk.inv_nu = __shfl_sync(F, pk.inv_nu, owner);
-          pk.inv_D = __shfl_sync(F, pk.inv_D, owner);
-          pk.shell = __shfl_sync(F, pk.shell, owner);
-          pk.next_line = __shfl_sync(F, pk.next_line, owner);
-          pk.pid = __shfl_sync(F, pk.pid, owner);
-          pk.have_inv_D = __shfl_sync(F, static_cast<int>(pk.have_inv_D), owner) != 0;
+          acc_s = -1; acc_j = 0ull; acc_nb = 0ull;
+          const PoolWalk *from = p.pool + from_pool;
+          if (from_pool < 0) {
+            const unsigned age = alive ? pk.cnt[0] + 1u : 0u;
+            const unsigned oldest = __reduce_max_sync(F, age);
+            const int owner = __ffs(__ballot_sync(F, age == oldest)) - 1;
+            PoolWalk w;
+            w.f[0] = pk.nu_lab;
 #pragma unroll
-          for (int k = 0; k < kNCounters; ++k) pk.cnt[k] = __shfl_sync(F, pk.cnt[k], owner);
-          ds.k0 = __shfl_sync(F, ds.k0, owner);
-          ds.k1 = __shfl_sync(F, ds.k1, owner);
-          ds.packet = __shfl_sync(F, ds.packet, owner);
-          ds.iteration = __shfl_sync(F, ds.iteration, owner);
-          ds.d = __shfl_sync(F, ds.d, owner);
-          ds.spare_a = __shfl_sync(F, ds.spare_a, owner);
-          ds.spare_b = __shfl_sync(F, ds.spare_b, owner);
-          cs = __shfl_sync(F, cs, owner);
-          c_kap = __shfl_sync(F, c_kap, owner);
-          c_ikap = __shfl_sync(F, c_ikap, owner);
-          c_xi2 = __shfl_sync(F, c_xi2, owner);
-          c_xo2 = __shfl_sync(F, c_xo2, owner);
-          acc_s = __shfl_sync(F, acc_s, owner);
-          acc_j = __shfl_sync(F, acc_j, owner);
-          acc_nb = __shfl_sync(F, acc_nb, owner);
+            for (int k = 1; k < 8; ++k) w.f[k] = 0.0;
+            w.i[0] = static_cast<uint32_t>(pk.shell);
+            w.i[1] = static_cast<uint32_t>(pk.next_line);
+            w.i[2] = pk.pid;
+            w.i[3] = ds.d;
+            w.i[4] = pk.have_inv_D ? 1u : 0u;
+            w.i[5] = __float_as_uint(pk.p);
+#pragma unroll
+            for (int k = 0; k < kNCounters; ++k) w.i[6 + k] = pk.cnt[k];
+            w.i[12] = __float_as_uint(pk.q);
+            w.i[13] = __float_as_uint(pk.e_lab);
+            w.i[14] = __float_as_uint(pk.inv_nu);
+            w.i[15] = __float_as_uint(pk.inv_D);
+            if (n_live > 1u) {
+              const unsigned others = live & ~(1u << owner);
+              unsigned long long place = 0ull;
+              if (lane == 0u) place = atomicAdd(p.pool_ctl, static_cast<unsigned long long>(n_live - 1u));
+              place = __shfl_sync(F, place, 0) + __popc(others & lanemask_lt);
+              // (the pool holds what every warp can hand over once)
+              if (((others >> lane) & 1u) && place < p.pool_cap) pool_put(p, static_cast<unsigned>(place), w);
+            }
+            if (static_cast<int>(lane) == owner) *reinterpret_cast<PoolWalk *>(warp_mem) = w;
+            from = reinterpret_cast<const PoolWalk *>(warp_mem);
+          }
+          __syncwarp();
+          {
+            const volatile PoolWalk *w = from;  // (another SM may have written it: not through L1)
+            pk.nu_lab = w->f[0];
+            pk.shell = static_cast<int32_t>(w->i[0]);
+            pk.next_line = static_cast<int32_t>(w->i[1]);
+            pk.pid = w->i[2];
+            ds.init(c.key0, c.key1, pk.pid, c.iteration);
+            ds.d = w->i[3];
+            pk.have_inv_D = w->i[4] != 0u;
+            pk.p = __uint_as_float(w->i[5]);
+#pragma unroll
+            for (int k = 0; k < kNCounters; ++k) pk.cnt[k] = w->i[6 + k];
+            pk.q = __uint_as_float(w->i[12]);
+            pk.e_lab = __uint_as_float(w->i[13]);
+            pk.inv_nu = __uint_as_float(w->i[14]);
+            pk.inv_D = __uint_as_float(w->i[15]);
+          }
+          __syncwarp();
+          cs = -1;
           lwin_s = -1;
           alive = true;
           lone = true;
+          wd.pid = kNoPacket;
           wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
         }
       }
     }
     if (!alive) continue;
-    const bool act = !lone || static_cast<int>(lane) == owner;  // makes the walk's side effects
+    const bool act = !lone || lane == 0u;  // makes the walk's side effects
     // the walk's next draw: from the warp's buffer in lone mode
     // (a macro atom's internal jumps can take more draws than the buffer holds)
     auto next_u = [&]() -> unsigned long long {
@@ -995,7 +1036,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
     }
   }
   if (cur_model >= 0) {
-    if (acc_s >= 0 && (!lone || static_cast<int>(lane) == owner)) {  // (a launch stopped in lone mode)
+    if (acc_s >= 0 && (!lone || lane == 0u)) {  // (a launch stopped in lone mode)
       atomicAdd(c.est_fix + acc_s, acc_j);
       atomicAdd(c.est_fix + c.S + acc_s, acc_nb);
     }
@@ -1029,10 +1070,10 @@ const void *select_b(int line_mode, bool jb, bool rec) { return select_m<2>(line
 
 const void *select_mixed_kernel(int line_mode, bool jb, bool rec) { return select_m<1>(line_mode, jb, rec); }
 
-// single-model launches (128 threads): shell tables, then a lone walker's
-// draw buffer per warp
+// single-model launches (128 threads): shell tables, then per warp a walk
+// handed to all lanes and the lone walk's draw buffer
 size_t mixed_smem_bytes(int S) {
-  return 4 * static_cast<size_t>(S) * sizeof(float) + (128 / 32) * kWarpDraws * sizeof(unsigned long long);
+  return 4 * static_cast<size_t>(S) * sizeof(float) + (128 / 32) * kLoneWords * sizeof(unsigned long long);
 }
 
 cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, int block,
