@@ -26,7 +26,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # how the registers were allocated.  The binary64 kernel's lone walk repeats a
 # segment's arithmetic in code of its own, which must round alike for the same
 # reason.
-PER_FILE_FLAGS = {"mc_transport_mixed.cu": ["-fmad=false"], "mc_transport.cu": ["-fmad=false"]}
+PER_FILE_FLAGS = {"mc_transport_mixed.cu": ["-fmad=false"], "mc_transport.cu": ["-fmad=false"],
+                  "mc_transport_virtual.cu": ["-fmad=false"]}
 
 
 def nvcc() -> str:

@@ -201,6 +201,7 @@ int transport_block_size();
 cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, bool tables, int S,
                                 int *blocks_per_sm);
 const void *select_mixed_kernel(int line_mode, bool j_blue, bool record);
+const void *select_virtual_kernel(int line_mode, bool j_blue, bool record);  // binary64, with v-packets
 // Batched launches: `block` threads per block (64, 128 or 256).
 cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, int block,
                             int *blocks_per_sm);
