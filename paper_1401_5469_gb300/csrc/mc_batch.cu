@@ -35,7 +35,9 @@ struct mc_batch {
   int grid = 0;
   TransportParams *d_params = nullptr, *h_params = nullptr;  // device table, pinned host staging
   unsigned long long *d_prefix = nullptr, *h_prefix = nullptr;
-  unsigned long long *d_counters = nullptr;  // work counter, flags (kNCounterSlots)
+  unsigned long long *d_counters = nullptr;  // work counter, flags (kNCounterSlots), then the pool's words
+  PoolWalk *d_pool = nullptr;      // [pool_cap] walks handed between warps
+  uint32_t pool_cap = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   std::vector<int> graph_shape;    // per model: 1 if its Sobolev depths were recomputed
@@ -76,6 +78,10 @@ void drop_graph(mc_batch *b) {
   if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
 }
 
+size_t counter_bytes(const mc_batch *b) {
+  return (kNCounterSlots + 2) * sizeof(unsigned long long) + b->pool_cap * sizeof(uint32_t);
+}
+
 // Enqueue one iteration of every model on the batch stream (`capturing`:
 // inside a stream capture, so the timing events become external event nodes).
 mc_status enqueue_iteration(mc_batch *b, int update, bool capturing) {
@@ -84,7 +90,7 @@ mc_status enqueue_iteration(mc_batch *b, int update, bool capturing) {
     const mc_status rc = model_prepare(m, b->stream, false);
     if (rc != MC_OK) return bfail(b, rc, m->err);
   }
-  cudaError_t e = cudaMemsetAsync(b->d_counters, 0, kNCounterSlots * sizeof(unsigned long long), b->stream);
+  cudaError_t e = cudaMemsetAsync(b->d_counters, 0, counter_bytes(b), b->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->d_params, b->h_params, b->models.size() * sizeof(TransportParams),
                         cudaMemcpyHostToDevice, b->stream);
@@ -96,6 +102,10 @@ mc_status enqueue_iteration(mc_batch *b, int update, bool capturing) {
   p.n_packets = b->h_prefix[b->models.size()];
   p.work_counter = b->d_counters;
   p.flags = b->d_counters + 1;
+  p.pool = b->d_pool;
+  p.pool_cap = b->pool_cap;
+  p.pool_ctl = b->d_counters + kNCounterSlots;
+  p.pool_ready = reinterpret_cast<uint32_t *>(b->d_counters + kNCounterSlots + 2);
   e = cudaEventRecordWithFlags(b->t0, b->stream, ev_flags);
   if (e == cudaSuccess) e = launch_transport_batch(p, b->line_mode, b->j_blue, b->record, b->grid,
                                                     static_cast<int>(b->block), b->stream);
@@ -154,7 +164,6 @@ mc_status mc_batch_create(mc_model *const *models, uint32_t n_models, mc_batch *
   cudaError_t e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMallocAsync(&b->d_params, n_models * sizeof(TransportParams), b->stream);
   if (e == cudaSuccess) e = cudaMallocAsync(&b->d_prefix, (n_models + 1) * sizeof(unsigned long long), b->stream);
-  if (e == cudaSuccess) e = cudaMallocAsync(&b->d_counters, kNCounterSlots * sizeof(unsigned long long), b->stream);
   if (e == cudaSuccess) {
     b->h_params = static_cast<TransportParams *>(pinned_get(n_models * sizeof(TransportParams), false));
     b->h_prefix = static_cast<unsigned long long *>(pinned_get((n_models + 1) * sizeof(unsigned long long), false));
@@ -174,6 +183,15 @@ mc_status mc_batch_create(mc_model *const *models, uint32_t n_models, mc_batch *
     return bfail(nullptr, MC_ERR_CUDA, std::string("batch create: ") + cudaGetErrorString(e));
   }
   b->grid = b->nsm * resolved_bps(b);
+  // every warp of a grid with the lone walk (128 threads a block) hands over at
+  // most kPoolLive - 1 walks, once
+  b->pool_cap = static_cast<uint32_t>(b->nsm * b->max_bps[1] * 4) * (kPoolLive - 1u);
+  e = cudaMallocAsync(&b->d_counters, counter_bytes(b), b->stream);
+  if (e == cudaSuccess) e = cudaMallocAsync(&b->d_pool, b->pool_cap * sizeof(PoolWalk), b->stream);
+  if (e != cudaSuccess) {
+    mc_batch_destroy(b);
+    return bfail(nullptr, MC_ERR_CUDA, std::string("batch create: ") + cudaGetErrorString(e));
+  }
   for (mc_model *m : b->models) m->in_batch = true;
   *out = b;
   return MC_OK;
@@ -410,6 +428,7 @@ void mc_batch_destroy(mc_batch *b) {
   if (b->d_params) cudaFreeAsync(b->d_params, b->stream);
   if (b->d_prefix) cudaFreeAsync(b->d_prefix, b->stream);
   if (b->d_counters) cudaFreeAsync(b->d_counters, b->stream);
+  if (b->d_pool) cudaFreeAsync(b->d_pool, b->stream);
   pinned_put(b->h_params);
   pinned_put(b->h_prefix);
   if (b->ev_in) cudaEventDestroy(b->ev_in);

@@ -22,11 +22,11 @@
 // model loads that model's context and first flushes its register
 // accumulators to the previous model.
 //
-// Single-model launches also have the binary64 kernel's lone-walker mode: a
-// warp down to its last live walk runs it with all 32 lanes (32-line windows
-// scanned in one step through a binary32 filter against this kernel's own
-// threshold chain, the emission record loaded as soon as the scan names the
-// line, the walk's draws computed ahead by the warp).
+// It also has the binary64 kernel's lone walks and pool: a warp down to its
+// last walks runs one with all 32 lanes (32-line windows scanned in one step
+// through a binary32 filter against this kernel's own threshold chain, the
+// emission record loaded as soon as the scan names the line, the walk's draws
+// computed ahead by the warp).
 #include <cstdint>
 
 #include "mc_device.cuh"
@@ -236,13 +236,38 @@ __device__ __forceinline__ void flush_stats(Stats &st, unsigned long long *dst) 
   }
 }
 
+// What the pool keeps of a walk (and its model in a batch).
+__device__ __forceinline__ PoolWalk pack_walk(const PacketM &pk, uint32_t d, int32_t model) {
+  PoolWalk w;
+  w.f[0] = pk.nu_lab;
+  w.f[1] = static_cast<double>(model);
+#pragma unroll
+  for (int k = 2; k < 8; ++k) w.f[k] = 0.0;
+  w.i[0] = static_cast<uint32_t>(pk.shell);
+  w.i[1] = static_cast<uint32_t>(pk.next_line);
+  w.i[2] = pk.pid;
+  w.i[3] = d;
+  w.i[4] = pk.have_inv_D ? 1u : 0u;
+  w.i[5] = __float_as_uint(pk.p);
+#pragma unroll
+  for (int k = 0; k < kNCounters; ++k) w.i[6 + k] = pk.cnt[k];
+  w.i[12] = __float_as_uint(pk.q);
+  w.i[13] = __float_as_uint(pk.e_lab);
+  w.i[14] = __float_as_uint(pk.inv_nu);
+  w.i[15] = __float_as_uint(pk.inv_D);
+  return w;
+}
+
 // One kernel source serves a single model (p.n_models == 0) and a batch, so a
 // model's results do not depend on the company it is launched in.  It is
-// compiled twice: MINB = 1 for single models (blocks of 128 threads, three
-// per SM at up to 168 registers, and the lone-walker mode for the last random
-// walks) and MINB = 2 for batches (128 registers: 16 resident warps per SM,
-// for the throughput phase that dominates a batch).  The arithmetic is the
-// same instruction for instruction, lone-walker mode included; the batch
+// compiled twice: MINB = 1 (blocks of 128 threads, three per SM at up to 168
+// registers, with lone walks) for single models and for batches of 128
+// threads a block, and MINB = 2 for batches of 64 or 256 threads (128
+// registers: 16 resident warps per SM, without lone walks).  A batch of 12
+// uneven models (2.9e6 packets): 330 ms a launch with the second (26 ms until
+// the queue is empty, then the longest walks at 2.5 us a segment), 209 ms with
+// the first (34 ms, and 1.3 us); of 40: 577 (156) and 430 (187).  The arithmetic
+// is the same instruction for instruction, lone walks included; the batch
 // tests check the bits.
 template <int MODE, bool JB, bool REC, int MINB>
 __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : MINB)
@@ -255,6 +280,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
   int32_t cur_model = -1;
   unsigned long long *prefix = smem_u64;
   const bool batch = p.n_models > 0;
+  constexpr bool kLoneBuild = MINB == 1;
   if (batch) {
     for (int i = threadIdx.x; i <= p.n_models; i += blockDim.x) prefix[i] = p.batch_prefix[i];
     __syncthreads();
@@ -283,10 +309,11 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
   // lwin_j0 + lane in each lane), scan the window in one step, compute the
   // walk's draws 64 at a time into a per-warp shared buffer, and only the
   // owner lane makes the walk's side effects.
-  constexpr bool kLoneBuild = MINB == 1;
   WarpDraws wd;
-  unsigned long long *warp_mem = smem_u64 + 2 * static_cast<size_t>(p.S) + kLoneWords * (threadIdx.x >> 5);
-  wd.init(batch ? nullptr : warp_mem + sizeof(PoolWalk) / sizeof(unsigned long long));
+  unsigned long long *warp_mem =
+      smem_u64 + (batch ? static_cast<size_t>(p.n_models) + 1 : 2 * static_cast<size_t>(p.S)) +
+      kLoneWords * (threadIdx.x >> 5);
+  wd.init(!kLoneBuild ? nullptr : warp_mem + sizeof(PoolWalk) / sizeof(unsigned long long));
   bool drained = false;  // warp-uniform: the packet queue is empty
   bool lone = false;
   int32_t lwin_j0 = 0, lwin_s = -1;
@@ -377,7 +404,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
     }
     int from_pool = -1;
     if (!lone && __all_sync(0xffffffffu, finished && !alive)) {
-      if (!kLoneBuild || batch || !p.pool) break;
+      if (!kLoneBuild || !p.pool) break;
       if (lane == 0u) from_pool = pool_take(p);
       from_pool = __shfl_sync(0xffffffffu, from_pool, 0);
       if (from_pool < 0) break;
@@ -391,7 +418,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         break;
       }
     }
-    if (p.cancel && (++polls & 255u) == 0u) {  // the host's stop request (mc_cancel)
+    if ((++polls & 255u) == 0u && p.cancel) {  // the host's stop request (mc_cancel)
       uint32_t stop = 0u;
       if (lane == 0u) stop = load_sys_u32(p.cancel);
       stop = __shfl_sync(0xffffffffu, stop, 0);
@@ -400,7 +427,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         break;
       }
     }
-    if (kLoneBuild && !batch) {
+    if (kLoneBuild) {
       if (lone) {
         wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
       } else {
@@ -423,22 +450,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
             const unsigned age = alive ? pk.cnt[0] + 1u : 0u;
             const unsigned oldest = __reduce_max_sync(F, age);
             const int owner = __ffs(__ballot_sync(F, age == oldest)) - 1;
-            PoolWalk w;
-            w.f[0] = pk.nu_lab;
-#pragma unroll
-            for (int k = 1; k < 8; ++k) w.f[k] = 0.0;
-            w.i[0] = static_cast<uint32_t>(pk.shell);
-            w.i[1] = static_cast<uint32_t>(pk.next_line);
-            w.i[2] = pk.pid;
-            w.i[3] = ds.d;
-            w.i[4] = pk.have_inv_D ? 1u : 0u;
-            w.i[5] = __float_as_uint(pk.p);
-#pragma unroll
-            for (int k = 0; k < kNCounters; ++k) w.i[6 + k] = pk.cnt[k];
-            w.i[12] = __float_as_uint(pk.q);
-            w.i[13] = __float_as_uint(pk.e_lab);
-            w.i[14] = __float_as_uint(pk.inv_nu);
-            w.i[15] = __float_as_uint(pk.inv_D);
+            const PoolWalk w = pack_walk(pk, ds.d, cur_model);
             if (n_live > 1u) {
               const unsigned others = live & ~(1u << owner);
               unsigned long long place = 0ull;
@@ -454,6 +466,14 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
           {
             const volatile PoolWalk *w = from;  // (another SM may have written it: not through L1)
             pk.nu_lab = w->f[0];
+            if (batch) {
+              const int32_t model = static_cast<int32_t>(w->f[1]);
+              if (model != cur_model) {
+                if (cur_model >= 0) flush_stats(st, c.stats);
+                load_ctx(c, p.batch[model], p.batch[model].shell32);
+                cur_model = model;
+              }
+            }
             pk.shell = static_cast<int32_t>(w->i[0]);
             pk.next_line = static_cast<int32_t>(w->i[1]);
             pk.pid = w->i[2];
@@ -1076,18 +1096,27 @@ size_t mixed_smem_bytes(int S) {
   return 4 * static_cast<size_t>(S) * sizeof(float) + (128 / 32) * kLoneWords * sizeof(unsigned long long);
 }
 
+// Batched launches of 128 threads a block take the build with the lone walk.
+namespace {
+const void *batch_kernel(int line_mode, bool jb, bool rec, int block) {
+  return block == 128 ? select_m<1>(line_mode, jb, rec) : select_b(line_mode, jb, rec);
+}
+size_t batch_smem_bytes(int n_models, int block) {
+  return (static_cast<size_t>(n_models) + 1 + (block == 128 ? 4 * kLoneWords : 0)) * sizeof(unsigned long long);
+}
+}  // namespace
+
 cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, int block,
                             int *blocks_per_sm) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, select_b(line_mode, j_blue, record), block,
-      static_cast<size_t>(n_models + 1) * sizeof(unsigned long long));
+      blocks_per_sm, batch_kernel(line_mode, j_blue, record, block), block, batch_smem_bytes(n_models, block));
 }
 
 cudaError_t launch_transport_batch(const TransportParams &p, int line_mode, bool j_blue, bool record,
                                    int grid, int block, cudaStream_t st) {
   void *args[] = {const_cast<TransportParams *>(&p)};
-  return cudaLaunchKernel(select_b(line_mode, j_blue, record), dim3(grid), dim3(block), args,
-                          static_cast<size_t>(p.n_models + 1) * sizeof(unsigned long long), st);
+  return cudaLaunchKernel(batch_kernel(line_mode, j_blue, record, block), dim3(grid), dim3(block), args,
+                          batch_smem_bytes(p.n_models, block), st);
 }
 
 }  // namespace mcgpu
