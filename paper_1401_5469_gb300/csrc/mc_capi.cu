@@ -374,7 +374,7 @@ mc_status mc_model_create(const mc_geometry_desc *geom, const mc_line_desc *line
     if (ok && atomic->dbr_offset && meta && run->line_mode != MC_LINE_SCATTER)
       ok = alloc_n(m, &m->dbr_rec, nnz) && alloc_n(m, &m->dbr_bucket, nnz) &&
            alloc_n(m, &m->row_info, L) &&
-           (run->precision == MC_PRECISION_MIXED ? alloc_n(m, &m->inv_nu32, L) : alloc_n(m, &m->inv_nu, L));
+           (run->precision != MC_PRECISION_MIXED || alloc_n(m, &m->inv_nu32, L));
   }
   if (ok) ok = alloc_n(m, &m->n_e, S);
   if (ok) {  // the stop request: one pinned host word the kernels can read
@@ -502,8 +502,8 @@ mc_status mc_model_create(const mc_geometry_desc *geom, const mc_line_desc *line
     if (m->dbr_rec) {
       chk(launch_dbr_setup(static_cast<uint32_t>(nnz), I * K, L, Kc, m->dbr_offset, m->dbr_line,
                            m->dbr_cdf, m->nu, m->line_row, m->dbr_rec, m->dbr_bucket,
-                           m->row_info, m->inv_nu, m->inv_nu32, m->stream));
-      m->launches += 4;
+                           m->row_info, m->inv_nu32, m->stream));
+      m->launches += m->inv_nu32 ? 4 : 3;
     }
     std::vector<MaRow> ma_rows;
     std::vector<MaJump> ma_jumps;
@@ -710,7 +710,7 @@ void model_fill_transport(const mc_model *m, TransportParams &p, uint64_t seed, 
   p.L = static_cast<int32_t>(m->L);
   p.x_in = m->x_in; p.x_out = m->x_out; p.inv_x_in = m->inv_x_in; p.inv_x_out = m->inv_x_out;
   p.inv_kappa = m->inv_kappa; p.row_info = m->row_info; p.dbr_rec = m->dbr_rec;
-  p.dbr_bucket = m->dbr_bucket; p.inv_nu = m->inv_nu; p.inv_nu32 = m->inv_nu32;
+  p.dbr_bucket = m->dbr_bucket; p.inv_nu32 = m->inv_nu32;
   p.kappa = m->kappa;
   p.nu = m->nu; p.tau = m->tau; p.tau32 = m->tau32;
   p.line_row = m->line_row; p.dbr_offset = m->dbr_offset; p.dbr_line = m->dbr_line; p.dbr_cdf = m->dbr_cdf;

@@ -160,47 +160,71 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Reciprocal from the hardware approximation r = rcp.approx.ftz.f64(x) by
-// one second-order correction: with e = 1 - x r (exact up to one rounding),
-// 1/x = r / (1 - e) = r (1 + e + e^2 + ...), so r + r (e + e^2) leaves a
-// relative error of order e^3 -- the cubically convergent form of Newton's
-// reciprocal iteration (Markstein 1990; J.-M. Muller, Elementary Functions,
-// ch. 2).  Three binary64 operations instead of the four of two Newton steps.
-// Within 1 ulp of 1/x for normal |x| in [2^-1000, 2^1000] (tested against
-// IEEE division through mc_selftest_math).
-__device__ __forceinline__ double rcp64_from(double x, double r) {
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-__device__ __forceinline__ double rcp64(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  return rcp64_from(x, r);
-}
-// The same value, evaluated only where it stands (the compiler may evaluate
-// the one above ahead of the branch that needs it).
-__device__ __forceinline__ double rcp64_here(double x) {
-  double r;
-  asm volatile("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  return rcp64_from(x, r);
+// Reciprocal and square root on the integer pipe.  A binary64 instruction
+// occupies its sub-partition's pipe for 64 cycles, and its result reaches another
+// pipe 45 cycles later than the next binary64 instruction; a 32 x 32 -> 64-bit
+// product takes 4.  Both start from the binary32 approximation of the 53-bit
+// significand (24 bits), and take two corrections: the residual exactly, as a
+// 64-bit integer (its upper bits cancel, so that products modulo 2^64 are
+// enough), the correction residual / slope in binary32 with the same
+// approximation.  The first leaves 2^-42 (its rounding and the omitted second-order
+// term), the second 2^-57, and the sum is rounded to 53 bits: within 0.53 ulp
+// (CPU emulation with the approximations two ulps off; the device's are tested
+// through mc_selftest_math).  Newton's iteration in residual form (J.-M. Muller,
+// Elementary Functions, ch. 2).  Before: three and five binary64 instructions
+// from rcp.approx / rsqrt.approx.f64, within 1 ulp.
+
+// round(a b) for |a b| < 2^21, through the low bits of a binary32 sum.
+__device__ __forceinline__ int32_t mul_round(float a, float b) {
+  return __float_as_int(fmaf(a, b, 12582912.0f)) - 0x4b400000;
 }
 
-// Square root of x >= 0 (0 or a normal number) to within 1 ulp, in five
-// binary64 operations: y = rsqrt.approx.ftz.f64(x), t = x y, e = 1 - t y, and
-// sqrt(x) = sqrt(t / y) (1 + O(2^-53)) = t (1 - e)^(-1/2), taken from the
-// Taylor series t (1 + e/2 + 3e^2/8) (the second-order Householder step for
-// 1/sqrt; J.-M. Muller, Elementary Functions, ch. 2).  On GB300 |e| <= 2^-19.0
-// over every high word of [1, 4) (measured), so the first omitted term,
-// 5e^3/16, is below 2^-58 relative.  (CUDA's sqrt rounds correctly but takes
-// about ten binary64 instructions; on GB300 each costs its sub-partition's
-// FP64 pipe ~64 cycles.)
-__device__ __forceinline__ double sqrt64_pos(double x) {  // x > 0
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double t = x * y;
-  const double e = fma(-t, y, 1.0);
-  const double p = fma(0.375, e, 0.5);
-  return fma(t * e, p, t);
+// 1/x for normal |x| in [2^-1000, 2^1000].  HERE: evaluated only where it
+// stands (the compiler may otherwise evaluate it ahead of the branch that needs it).
+template <bool HERE = false>
+__device__ __forceinline__ double rcp64(double x) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+  const uint32_t e = (hi >> 20) & 0x7ffu;
+  const uint32_t mh = (hi & 0xfffffu) | 0x100000u;  // the significand's upper 21 bits
+  const unsigned long long m = (static_cast<unsigned long long>(mh) << 32) | lo;  // 2^52 times [1, 2)
+  const float f32 = static_cast<float>(__funnelshift_l(lo, mh, 11));
+  float y;  // 2^-31 / significand
+  if (HERE) asm volatile("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f32));
+  else asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f32));
+  const float t = fminf(fmaxf(y * 0x1.0p55f, 0x1.0p23f), 0x1.fffffep23f);
+  const uint32_t q0 = (__float_as_uint(t) & 0x7fffffu) | 0x800000u;  // units of 2^-24
+  const long long r0 = static_cast<long long>(0ull - m * q0);        // 2^76 - m q0
+  const int32_t c1 = mul_round(static_cast<float>(static_cast<int32_t>(r0 >> 24)), y * 0x1.0p22f);
+  const unsigned long long q1 = (static_cast<unsigned long long>(q0) << 19) +
+                                static_cast<unsigned long long>(static_cast<long long>(c1));  // 2^-43
+  const long long r1 = static_cast<long long>(0ull - m * q1);        // 2^95 - m q1
+  const int32_t c2 = mul_round(static_cast<float>(static_cast<int32_t>(r1 >> 26)), y * 0x1.0p20f);
+  const unsigned long long f = (q1 << 15) + static_cast<unsigned long long>(static_cast<long long>(c2));  // 2^-58
+  const unsigned long long bits = (static_cast<unsigned long long>(2044u - e) << 52) + ((f + 16ull) >> 5);
+  return __longlong_as_double(static_cast<long long>(bits | (static_cast<unsigned long long>(hi & 0x80000000u) << 32)));
+}
+
+// Square root of a normal x > 0; sqrt64: of 0 too.
+__device__ __forceinline__ double sqrt64_pos(double x) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+  const uint32_t e = hi >> 20, odd = ~e & 1u;
+  const unsigned long long m = (static_cast<unsigned long long>((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  const unsigned long long a = m << (10u + odd);  // 2^62 times [1, 4)
+  const float f = static_cast<float>(static_cast<uint32_t>(a >> 32));
+  float y;  // 2^-15 / sqrt
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
+  const float t = fminf(fmaxf(f * y, 0x1.0p15f), 0x1.fffffep15f);
+  const uint32_t s0 = ((__float_as_uint(t) & 0x7fffffu) | 0x800000u) << 8;  // units of 2^-31
+  const long long r0 = static_cast<long long>(a - static_cast<unsigned long long>(s0) * s0);
+  const int32_t c1 = mul_round(static_cast<float>(static_cast<int32_t>(r0 >> 13)), y * 0x1.0p7f);
+  const unsigned long long s1 = (static_cast<unsigned long long>(s0) << 11) +
+                                static_cast<unsigned long long>(static_cast<long long>(c1));  // 2^-42
+  const long long r1 = static_cast<long long>((a << 22) - s1 * s1);
+  const int32_t c2 = mul_round(static_cast<float>(static_cast<int32_t>(r1 >> 14)), y);
+  const unsigned long long s2 = (s1 << 14) + static_cast<unsigned long long>(static_cast<long long>(c2));  // 2^-56
+  const unsigned long long bits =
+      (static_cast<unsigned long long>(((e + 1023u - odd) >> 1) - 1u) << 52) + ((s2 + 8ull) >> 4);
+  return __longlong_as_double(static_cast<long long>(bits));
 }
 __device__ __forceinline__ double sqrt64(double x) {
   return __double_as_longlong(x) == 0ll ? 0.0 : sqrt64_pos(x);
@@ -317,6 +341,17 @@ __device__ __forceinline__ void load_slot(const DbrSlot *slot, uint4 &a, uint4 &
 __device__ __forceinline__ void load_slot_here(const DbrSlot *slot, uint4 &a, uint4 &c) {
   a = load_here4(slot);
   c = load_here4(reinterpret_cast<const uint4 *>(slot) + 1);
+}
+
+// The same in four 64-bit loads: the mixed kernel's lone walk takes 91 ms with
+// them instead of 102 (the binary64 kernel's 105 instead of 100).
+__device__ __forceinline__ void load_slot_here64(const DbrSlot *slot, uint4 &a, uint4 &c) {
+  const unsigned long long *w = reinterpret_cast<const unsigned long long *>(slot);
+  const unsigned long long w0 = load_here(w), w1 = load_here(w + 1), w2 = load_here(w + 2), w3 = load_here(w + 3);
+  a = make_uint4(static_cast<uint32_t>(w0), static_cast<uint32_t>(w0 >> 32), static_cast<uint32_t>(w1),
+                 static_cast<uint32_t>(w1 >> 32));
+  c = make_uint4(static_cast<uint32_t>(w2), static_cast<uint32_t>(w2 >> 32), static_cast<uint32_t>(w3),
+                 static_cast<uint32_t>(w3 >> 32));
 }
 
 // The emitted line from a loaded slot {thr[3], emit[0]}, {emit[1], emit[2],

@@ -98,8 +98,7 @@ struct TransportParams {
   const MaRow *ma_row;               // [rows] macro-atom levels, or nullptr (no internal jumps)
   const MaJump *ma_jump;             // [n] macro-atom jump entries
   const DbrSlot *dbr_bucket;         // [nnz] the rows' buckets, or nullptr
-  const double *inv_nu;              // [L] 1 / nu (binary64; with dbr_rec)
-  const float *inv_nu32;             // [L] the same truncated to binary32 (mixed; with dbr_rec)
+  const float *inv_nu32;             // [L] 1 / nu truncated to binary32 (mixed; with dbr_rec)
   double *j_est, *nu_bar;            // [S] raw sums
   double *j_blue;                    // [S*L] raw sums or nullptr
   double *spectrum;                  // [bins + 2]
@@ -109,6 +108,7 @@ struct TransportParams {
   uint64_t n_packets;                // packets of this launch
   uint64_t first_packet;             // global id of the first (records are relative)
   uint32_t iteration, key0, key1;
+  uint32_t zero;                     // 0, unknown to the compiler (orders a lone walk's instructions)
   double e_cmf;                      // comoving packet energy, Eq. 10
   double nu_scale;                   // k T_inner / h
   const double *planck_cdf;          // [kPlanckLmax + 1]
@@ -229,7 +229,7 @@ cudaError_t launch_dbr_setup(uint32_t nnz, uint32_t n_rows, uint32_t L, int K,
                              const uint32_t *dbr_offset, const uint32_t *dbr_line,
                              const double *dbr_cdf, const double *nu, const int32_t *line_row,
                              DbrRec *rec, DbrSlot *bucket, unsigned long long *row_info,
-                             double *inv_nu, float *inv_nu32,
+                             float *inv_nu32,
                              cudaStream_t st);
 cudaError_t launch_line_setup(int L, int K, const double *nu, const double *f, const int32_t *ion,
                               const int32_t *lower, const int32_t *upper, const double *g,

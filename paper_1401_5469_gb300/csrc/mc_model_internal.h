@@ -37,8 +37,7 @@ struct mc_model {
   unsigned long long *est_fix = nullptr;  // [2 S] fixed-point J, nu_bar sums (mixed precision)
   mcgpu::DbrRec *dbr_rec = nullptr;
   mcgpu::DbrSlot *dbr_bucket = nullptr;
-  double *inv_nu = nullptr;          // with dbr_rec: 1 / nu (binary64 models)
-  float *inv_nu32 = nullptr;         // ... or the same in binary32 (mixed precision)
+  float *inv_nu32 = nullptr;         // with dbr_rec, mixed precision: 1 / nu truncated to binary32
   mcgpu::MaRow *ma_row = nullptr;    // macro-atom levels (MC_LINE_MACROATOM)
   mcgpu::MaJump *ma_jump = nullptr;
   unsigned long long *row_info = nullptr;

@@ -267,14 +267,12 @@ __global__ void dbr_bucket_kernel(uint32_t nnz, uint32_t n_rows, const uint32_t 
   bucket[e] = r;
 }
 
-// 1 / nu of every line, as binary64 or truncated to binary32 (either may be
-// nullptr; binary32 for line frequencies inside its normal range).
-__global__ void inv_nu_kernel(uint32_t L, const double *nu, double *inv, float *inv32) {
+// 1 / nu of every line truncated to binary32 (line frequencies inside its
+// normal range).
+__global__ void inv_nu_kernel(uint32_t L, const double *nu, float *inv32) {
   const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= L) return;
-  const double v = 1.0 / nu[j];
-  if (inv) inv[j] = v;
-  if (inv32) inv32[j] = __double2float_rz(v);
+  inv32[j] = __double2float_rz(1.0 / nu[j]);
 }
 
 __global__ void row_info_kernel(uint32_t L, const int32_t *line_row, const uint32_t *off,
@@ -389,7 +387,7 @@ cudaError_t launch_dbr_setup(uint32_t nnz, uint32_t n_rows, uint32_t L, int K,
                              const uint32_t *dbr_offset, const uint32_t *dbr_line,
                              const double *dbr_cdf, const double *nu, const int32_t *line_row,
                              DbrRec *rec, DbrSlot *bucket, unsigned long long *row_info,
-                             double *inv_nu, float *inv_nu32, cudaStream_t st) {
+                             float *inv_nu32, cudaStream_t st) {
   (void)K;
   if (nnz > 0) {
     dbr_rec_kernel<<<(nnz + 255) / 256, 256, 0, st>>>(nnz, n_rows, dbr_offset, dbr_line, dbr_cdf, rec);
@@ -397,7 +395,7 @@ cudaError_t launch_dbr_setup(uint32_t nnz, uint32_t n_rows, uint32_t L, int K,
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  inv_nu_kernel<<<(L + 255) / 256, 256, 0, st>>>(L, nu, inv_nu, inv_nu32);
+  if (inv_nu32) inv_nu_kernel<<<(L + 255) / 256, 256, 0, st>>>(L, nu, inv_nu32);
   row_info_kernel<<<(L + 255) / 256, 256, 0, st>>>(L, line_row, dbr_offset, row_info);
   return cudaGetLastError();
 }

@@ -377,12 +377,12 @@ struct MaDraws {
 };
 
 // LINES: what an absorbing line does -- 0 scatter, 1 downbranch, 2 macro atom,
-// 3 downbranch from the caller's table alone (no bucket slots, no 1/nu).
+// 3 downbranch from the caller's table alone (no bucket slots).
 // VIRT: with virtual packets.
 template <int LINES, bool JB, bool REC, bool VIRT>
 __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p) {
   constexpr int MODE = LINES == 3 ? 1 : LINES;
-  constexpr bool kSlots = LINES == 1 || LINES == 2;  // the model's tables: bucket slots, row info, 1/nu
+  constexpr bool kSlots = LINES == 1 || LINES == 2;  // the model's tables: bucket slots, row info
   extern __shared__ double sh[];
   const int32_t S = p.S, L = p.L;
   for (int i = threadIdx.x; i < S; i += blockDim.x) {
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   // scattering, exact_scan, the end of the walk)
   auto need_lab = [&]() {
     if (!pk.have_lab) {
-      pk.nu_lab = pk.nu_cmf * rcp64_here(pk.D);
+      pk.nu_lab = pk.nu_cmf * rcp64<true>(pk.D);
       pk.have_lab = true;
     }
   };
@@ -715,12 +715,14 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
         if (LINES == 1) w_r = load_here(p.row_info + jj);
       };
       reload(pk.next_line);
-      // A line's re-emission leaves 1/nu of the emitted line in flight (inv_c):
-      // E/nu and 1/nu_lab are taken when the next event needs them.
+      // After a line's re-emission E/nu and 1/nu_lab are taken when the next event
+      // needs them: the emitted line's frequency is in flight until then.  (Its
+      // reciprocal from a table of 1/nu arrived later still: 4 MB touched at
+      // random, mostly from DRAM.)
       bool fresh = false;
-      double inv_c = 0.0;
       auto settle = [&]() {
         if (fresh) {
+          const double inv_c = rcp64<true>(pk.nu_cmf);
           pk.inv_nu = inv_c * pk.D;
           if (MODE >= 1) pk.e_per_nu = pk.e_cmf * inv_c;  // re-emitted at another frequency
           fresh = false;
@@ -819,12 +821,14 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
             const double pl = fma(-nuj, pk.inv_nu, 1.0);
             const double r2 = fma(pl, pl, pk.q);
             log_segment(lp, w0, k + 1);
-            int32_t em = slot_line(ra, rc, u_em);
+            // (not before r2 is there: scheduled earlier, it would wait for the
+            // record with the event's arithmetic behind it)
+            int32_t em = slot_line(ra, rc, u_em ^ (static_cast<unsigned long long>(
+                                               static_cast<uint32_t>(__double2hiint(r2)) & p.zero) << 32));
             if (em < 0) em = search_row_lone(p.dbr_rec, rinfo, rc.z, u_em, lane);
             reload(em + 1);
             pk.next_line = em + 1;
             pk.nu_cmf = __longlong_as_double(static_cast<long long>(load_here(p.nu + em)));
-            inv_c = __longlong_as_double(static_cast<long long>(load_here(p.inv_nu + em)));
             // ... and while the window is on its way:
             const double xn = sqrt64_pos(r2);
             pk.e_cmf = pk.e_per_nu * nuj;
@@ -1003,12 +1007,9 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
             pk.next_line = em + 1;
             reload(em + 1);
             pk.nu_cmf = __longlong_as_double(static_cast<long long>(load_here(p.nu + em)));
-            if (kSlots) inv_c = __longlong_as_double(static_cast<long long>(load_here(p.inv_nu + em)));
-            else inv_c = rcp64(pk.nu_cmf);
           } else {
             pk.next_line = j + 1;
             pk.nu_cmf = nuj;
-            inv_c = rcp64(nuj);
           }
           pk.e_cmf = pk.e_per_nu * nuj;
           const double pn = xn * mu;
@@ -1224,7 +1225,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
             }
             const int32_t em = downbranch_pick<kSlots>(p, j, rinfo_em, ds.next_u53());
             nu_c = __ldg(p.nu + em);
-            inv_c = kSlots ? __ldg(p.inv_nu + em) : rcp64(nu_c);
+            inv_c = rcp64(nu_c);
             pk.next_line = em + 1;
             load_window(s, pk.next_line);
             pk.e_per_nu = pk.e_cmf * inv_c;  // re-emitted at another frequency

@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         const long long hit = __shfl_sync(F, w_b, k);
         const unsigned long long rinfo = __shfl_sync(F, w_r, k);
         uint4 ra, rc;
-        load_slot_here(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
+        load_slot_here64(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
         const bool prior = static_cast<int>(lane) < k;
         const unsigned sum = __reduce_add_sync(
             F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);

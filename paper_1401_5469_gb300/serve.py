@@ -55,7 +55,7 @@ def model_footprint_bytes(spec, j_blue: Optional[bool] = None,
     b += L * (8 + 8 + 4 * 3 + 8 + 8)   # nu, f, ion/lower/upper, per-line constants, row info
     b += L * (4 * 3 + 8)               # staged line arrays used at set-up
     b += nnz * (4 + 4 + 8 + 16 + 32)   # branching table, its search entries and bucket slots
-    b += L * (4 if precision == mc.MC_PRECISION_MIXED else 8)  # 1 / nu
+    b += 4 * L if precision == mc.MC_PRECISION_MIXED else 0  # 1 / nu in binary32
     b += 152 * 12 * 3 * (128 + 4)      # walks handed between warps (12 warps an SM, 3 walks each)
     if spec.n_ions:
         b += spec.n_ions * spec.n_levels * (8 + 8 + 1) + S * spec.n_ions * (8 + 8 * spec.n_levels)
