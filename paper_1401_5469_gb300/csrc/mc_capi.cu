@@ -361,7 +361,8 @@ mc_status mc_model_create(const mc_geometry_desc *geom, const mc_line_desc *line
             alloc_n(m, &m->planck_cdf, static_cast<size_t>(kPlanckLmax) + 1);
   if (ok && run->j_blue) ok = alloc_n(m, &m->j_blue, SL);
   if (ok && run->precision == MC_PRECISION_MIXED)
-    ok = alloc_n(m, &m->shell32, 4 * static_cast<size_t>(S)) && alloc_n(m, &m->est_fix, 2 * static_cast<size_t>(S));
+    ok = alloc_n(m, &m->shell32, 4 * static_cast<size_t>(S)) && alloc_n(m, &m->est_fix, est_copies(S) * 2 * static_cast<size_t>(S));
+  if (ok && run->precision != MC_PRECISION_MIXED) ok = alloc_n(m, &m->est_part, est_copies(S) * 2 * static_cast<size_t>(S));
   if (ok && meta) ok = alloc_n(m, &m->line_row, L) && alloc_n(m, &m->lev_l, L) && alloc_n(m, &m->lev_u, L);
   if (ok && atomic) {
     const size_t IK = static_cast<size_t>(I) * K;
@@ -624,6 +625,7 @@ mc_status mc_run_iteration_range(mc_model *m, uint64_t seed, uint32_t iteration,
     return fail(m, MC_ERR_INVALID_ARG, "n_packets exceeds max_packets of the packet records");
   if (!(t_inner > 0.0) || !std::isfinite(t_inner)) return fail(m, MC_ERR_INVALID_ARG, "t_inner must be positive");
   if (m->in_batch) return fail(m, MC_ERR_INVALID_ARG, "the model belongs to a batch; run it through the batch");
+  m->spread = n_packets >= kSpreadPackets;
   mc_status st = model_prepare(m, m->stream, true);
   if (st != MC_OK) return st;
   TransportParams p{};
@@ -660,7 +662,11 @@ mc_status model_prepare(mc_model *m, cudaStream_t st, bool events) {
     if (events) cudaEventRecord(m->ev[kEvPlasma1], st);
     m->ran_plasma = events;
   }
-  cudaError_t e = launch_zero(m->j_est, m->S, m->nu_bar, m->S, m->spectrum, m->run.spec_bins + 2,
+  // (j_est and nu_bar are written from the copies after the launch, if it uses them)
+  const bool copies = m->est_part && m->spread;
+  cudaError_t e = launch_zero(copies ? m->est_part : m->j_est,
+                              copies ? est_copies(m->S) * 2 * static_cast<size_t>(m->S) : m->S, m->nu_bar,
+                              copies ? 0 : m->S, m->spectrum, m->run.spec_bins + 2,
                               m->counters,
                               events ? m->n_counter_words : static_cast<size_t>(kNCounterSlots), st);
   if (e != cudaSuccess) return cuda_fail(m, e, "zero");
@@ -671,7 +677,7 @@ mc_status model_prepare(mc_model *m, cudaStream_t st, bool events) {
     m->launches += 1;
   }
   if (m->est_fix) {
-    e = cudaMemsetAsync(m->est_fix, 0, 2 * static_cast<size_t>(m->S) * sizeof(unsigned long long), st);
+    e = cudaMemsetAsync(m->est_fix, 0, est_copies(m->S) * 2 * static_cast<size_t>(m->S) * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return cuda_fail(m, e, "zero fixed-point estimators");
   }
   if (m->spectrum_v && m->n_virtual) {
@@ -683,6 +689,12 @@ mc_status model_prepare(mc_model *m, cudaStream_t st, bool events) {
 
 mc_status model_finish_transport(mc_model *m, const TransportParams &p, cudaStream_t st) {
   if (!m->est_fix) {
+    if (p.est_part) {
+      const cudaError_t es = launch_est_sum(m->est_part, static_cast<int>(p.est_copies), static_cast<int>(m->S),
+                                            m->j_est, m->nu_bar, st);
+      if (es != cudaSuccess) return cuda_fail(m, es, "estimator sums");
+      m->launches += 1;
+    }
     if (!m->j_blue) return MC_OK;
     // binary64: J_blue cells hold sums of E_lab / nu_lab^2; times nu_j
     const cudaError_t e = launch_jblue_times_nu(m->j_blue, m->nu, static_cast<int>(m->S),
@@ -691,7 +703,7 @@ mc_status model_finish_transport(mc_model *m, const TransportParams &p, cudaStre
     m->launches += 1;
     return MC_OK;
   }
-  cudaError_t e = launch_est_from_fix(m->est_fix, static_cast<int>(m->S), p.e_cmf, p.nu_scale,
+  cudaError_t e = launch_est_from_fix(m->est_fix, static_cast<int>(p.est_copies), static_cast<int>(m->S), p.e_cmf, p.nu_scale,
                                       m->j_est, m->nu_bar, st);
   if (e != cudaSuccess) return cuda_fail(m, e, "estimator conversion");
   m->launches += 1;
@@ -748,6 +760,8 @@ void model_fill_transport(const mc_model *m, TransportParams &p, uint64_t seed, 
   p.cancel = m->cancel_dev;
   p.shell32 = m->shell32;
   p.est_fix = m->est_fix;
+  p.est_part = m->spread ? m->est_part : nullptr;
+  p.est_copies = est_copies(m->S);
   p.inv_nu_ref = 1.0 / p.nu_scale;
 }
 

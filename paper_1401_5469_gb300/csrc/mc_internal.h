@@ -80,6 +80,16 @@ struct PoolWalk {
 constexpr unsigned kPoolLive = 4;
 constexpr uint32_t kPoolAge = 128;
 
+// Copies of the J and nu_bar sums, the blocks spread over them: a shell's sums
+// are two addresses that every packet crossing it adds to.  1e4 packets of the
+// 2000-line scatter model: 365 -> 279 us, 1e5 of a 5000-line one 1.06 -> 0.80 ms,
+// mixed 285 -> 234 us and 1.17 -> 0.74 ms (one copy -> 64).  A binary64 launch of
+// fewer packets than kSpreadPackets adds to the result itself (summing the
+// copies takes a launch of 3 us).
+constexpr uint32_t kEstCopies = 64;
+constexpr uint64_t kSpreadPackets = 4096;
+inline uint32_t est_copies(uint32_t S) { return S > 4096 / kEstCopies ? (4096 / S > 0 ? 4096 / S : 1) : kEstCopies; }
+
 // Everything the transport kernel reads or writes.
 struct TransportParams {
   int32_t S, L;
@@ -118,7 +128,9 @@ struct TransportParams {
   double *rec_nu, *rec_e;
   unsigned long long *rec_cnt;       // [n * kNCounters]
   const float *shell32;              // [4 S] binary32 shell table (mixed; batched launch)
-  unsigned long long *est_fix;       // [2 S] mixed: J, nu_bar sums in fixed point (see below)
+  unsigned long long *est_fix;       // [est_copies 2 S] mixed: J, nu_bar sums in fixed point (see below)
+  double *est_part;                  // [est_copies 2 S] binary64: J, nu_bar sums, or nullptr: in j_est, nu_bar
+  uint32_t est_copies;               // block b adds to copy b % est_copies
   double inv_nu_ref;                 // mixed: 1 / (k T_inner / h), scale of nu in nu_bar
   const TransportParams *batch;      // batched launch: per-model parameters, or nullptr
   const unsigned long long *batch_prefix;  // [n_models + 1] packet offsets of the models
@@ -216,8 +228,10 @@ cudaError_t launch_jblue_from_fix(double *j_blue, size_t n, double e_cmf, double
 // Binary64 J_blue: the transport sums E_lab / nu_lab^2 per (shell, line);
 // this multiplies every cell by its line frequency nu_j (Eq. 17).
 cudaError_t launch_jblue_times_nu(double *j_blue, const double *nu, int S, int L, cudaStream_t st);
-cudaError_t launch_est_from_fix(const unsigned long long *fix, int S, double e_cmf, double nu_ref,
+cudaError_t launch_est_from_fix(const unsigned long long *fix, int copies, int S, double e_cmf, double nu_ref,
                                 double *j_est, double *nu_bar, cudaStream_t st);
+// j_est, nu_bar = the sums over the copies (binary64).
+cudaError_t launch_est_sum(const double *part, int copies, int S, double *j_est, double *nu_bar, cudaStream_t st);
 cudaError_t launch_ionization(const IonParams &p, cudaStream_t st);  // two kernels
 cudaError_t launch_populations(const PlasmaParams &p, cudaStream_t st);
 cudaError_t launch_sobolev_tau(const PlasmaParams &p, cudaStream_t st);

@@ -34,7 +34,9 @@ struct mc_model {
   double *x_in = nullptr, *x_out = nullptr, *inv_x_in = nullptr, *inv_x_out = nullptr;
   double *kappa = nullptr, *inv_kappa = nullptr;
   float *shell32 = nullptr;  // [4 S] binary32 x_in^2, x_out^2, kappa', 1/kappa' (mixed precision)
-  unsigned long long *est_fix = nullptr;  // [2 S] fixed-point J, nu_bar sums (mixed precision)
+  unsigned long long *est_fix = nullptr;  // [copies 2 S] fixed-point J, nu_bar sums (mixed precision)
+  double *est_part = nullptr;             // [copies 2 S] their binary64 counterpart
+  bool spread = true;                     // the next launch uses est_part (binary64)
   mcgpu::DbrRec *dbr_rec = nullptr;
   mcgpu::DbrSlot *dbr_bucket = nullptr;
   float *inv_nu32 = nullptr;         // with dbr_rec, mixed precision: 1 / nu truncated to binary32

@@ -309,12 +309,27 @@ __global__ void jblue_times_nu_kernel(double *jb, const double *nu, int S, int L
   }
 }
 
-__global__ void est_from_fix_kernel(const unsigned long long *fix, int S, double e_cmf, double nu_ref,
+// One warp a sum (shell s of J, then of nu_bar), lanes over the copies.
+__global__ void est_from_fix_kernel(const unsigned long long *fix, int copies, int S, double e_cmf, double nu_ref,
                                     double *j_est, double *nu_bar) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  j_est[s] = (static_cast<double>(fix[s]) * (1.0 / kEstFixScale)) * e_cmf;
-  nu_bar[s] = ((static_cast<double>(fix[S + s]) * (1.0 / kEstFixScale)) * e_cmf) * nu_ref;
+  const int i = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (i >= 2 * S) return;
+  unsigned long long v = 0ull;
+  for (int c = lane; c < copies; c += 32) v += fix[static_cast<size_t>(c) * 2 * S + i];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane != 0) return;
+  const double e = (static_cast<double>(v) * (1.0 / kEstFixScale)) * e_cmf;
+  if (i < S) j_est[i] = e;
+  else nu_bar[i - S] = e * nu_ref;
+}
+
+__global__ void est_sum_kernel(const double *part, int copies, int S, double *j_est, double *nu_bar) {
+  const int i = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (i >= 2 * S) return;
+  double v = 0.0;
+  for (int c = lane; c < copies; c += 32) v += part[static_cast<size_t>(c) * 2 * S + i];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) (i < S ? j_est : nu_bar - S)[i] = v;
 }
 
 __global__ void to_f32_kernel(const double *in, float *out, size_t n) {
@@ -411,9 +426,14 @@ cudaError_t launch_jblue_times_nu(double *j_blue, const double *nu, int S, int L
   return cudaGetLastError();
 }
 
-cudaError_t launch_est_from_fix(const unsigned long long *fix, int S, double e_cmf, double nu_ref,
+cudaError_t launch_est_from_fix(const unsigned long long *fix, int copies, int S, double e_cmf, double nu_ref,
                                 double *j_est, double *nu_bar, cudaStream_t st) {
-  est_from_fix_kernel<<<(S + 63) / 64, 64, 0, st>>>(fix, S, e_cmf, nu_ref, j_est, nu_bar);
+  est_from_fix_kernel<<<S, 64, 0, st>>>(fix, copies, S, e_cmf, nu_ref, j_est, nu_bar);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_est_sum(const double *part, int copies, int S, double *j_est, double *nu_bar, cudaStream_t st) {
+  est_sum_kernel<<<S, 64, 0, st>>>(part, copies, S, j_est, nu_bar);
   return cudaGetLastError();
 }
 

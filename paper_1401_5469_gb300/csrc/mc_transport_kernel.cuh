@@ -412,6 +412,10 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   const unsigned long long n_warps = static_cast<unsigned long long>(gridDim.x) * (kBlock / 32);
   const unsigned quota = static_cast<unsigned>(min(32ull, (p.n_packets + n_warps - 1ull) / n_warps));
 
+  // this block's copy of the estimator sums
+  double *j_sum = p.est_part ? p.est_part + static_cast<size_t>(blockIdx.x % p.est_copies) * 2 * S : p.j_est;
+  double *nb_sum = p.est_part ? j_sum + S : p.nu_bar;
+
   Packet pk{};
   DrawStream ds;
   bool alive = false, finished = lane >= quota;
@@ -643,8 +647,8 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       // event's binary64 arithmetic runs while they are in flight.
       const unsigned F = 0xffffffffu;
       if (acc_s >= 0) {
-        atomicAdd(p.j_est + acc_s, acc_j);
-        atomicAdd(p.nu_bar + acc_s, acc_nb);
+        atomicAdd(j_sum + acc_s, acc_j);
+        atomicAdd(nb_sum + acc_s, acc_nb);
       }
       acc_s = -1;
       char *warp_mem = reinterpret_cast<char *>(sh + kShellArrays * S) + kLoneBytes * (threadIdx.x >> 5);
@@ -761,8 +765,8 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       auto flush_shell = [&]() {
         sum_log();
         if (rawkey(a_j) > 0) {
-          atomicAdd(p.j_est + cs, a_j);
-          atomicAdd(p.nu_bar + cs, a_nb);
+          atomicAdd(j_sum + cs, a_j);
+          atomicAdd(nb_sum + cs, a_nb);
         }
         a_j = 0.0;
         a_nb = 0.0;
@@ -1194,8 +1198,8 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       const double wgt = (pk.e_cmf * pk.D) * l;
       if (s != acc_s) {
         if (acc_s >= 0) {
-          atomicAdd(p.j_est + acc_s, acc_j);
-          atomicAdd(p.nu_bar + acc_s, acc_nb);
+          atomicAdd(j_sum + acc_s, acc_j);
+          atomicAdd(nb_sum + acc_s, acc_nb);
         }
         acc_s = s; acc_j = 0.0; acc_nb = 0.0;
       }
@@ -1283,8 +1287,8 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
   }
   if (VIRT && n_vq) fly_virtual(p, sh, vq, n_vq, lane);
   if (acc_s >= 0) {
-    atomicAdd(p.j_est + acc_s, acc_j);
-    atomicAdd(p.nu_bar + acc_s, acc_nb);
+    atomicAdd(j_sum + acc_s, acc_j);
+    atomicAdd(nb_sum + acc_s, acc_nb);
   }
   unsigned long long st[kNStats] = {n_esc, n_reab, n_cap, n_seg, n_chk, n_res, n_lint, n_esca, n_shell};
 #pragma unroll

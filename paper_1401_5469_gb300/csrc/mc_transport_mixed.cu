@@ -65,7 +65,7 @@ struct MCtx {
   const float *inv_nu32;
   double *j_blue, *j_est, *nu_bar, *spectrum;
   unsigned long long *stats;
-  unsigned long long *est_fix;  // [2 S] J, nu_bar in fixed point
+  unsigned long long *est_fix;  // [2 S] J, nu_bar in fixed point (this block's copy)
   unsigned long long *jb_fix;   // [S L] J_blue in fixed point (the j_blue buffer, converted after the launch)
   float inv_nu_ref, nu_ref;
   const double *planck;
@@ -100,7 +100,7 @@ __device__ __forceinline__ void load_ctx(MCtx &c, const TransportParams &q, cons
   c.nu_bar = q.nu_bar;
   c.spectrum = q.spectrum;
   c.stats = q.stats;
-  c.est_fix = q.est_fix;
+  c.est_fix = q.est_fix + static_cast<size_t>(blockIdx.x % q.est_copies) * 2 * q.S;
   c.jb_fix = reinterpret_cast<unsigned long long *>(q.j_blue);
   c.inv_nu_ref = static_cast<float>(q.inv_nu_ref);
   c.nu_ref = static_cast<float>(q.nu_scale);
