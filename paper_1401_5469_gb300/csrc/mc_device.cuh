@@ -143,6 +143,11 @@ __device__ __forceinline__ unsigned long long load_here(const void *a) {
   asm volatile("ld.global.nc.b64 %0, [%1];" : "=l"(v) : "l"(a));
   return v;
 }
+__device__ __forceinline__ uint32_t load_here32(const void *a) {
+  uint32_t v;
+  asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(a));
+  return v;
+}
 __device__ __forceinline__ float load_here_f(const float *a) {
   float v;
   asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(a));
@@ -464,6 +469,34 @@ struct WarpDraws {
   // The draw take_u53 returns next, without taking it.
   __device__ __forceinline__ unsigned long long peek_u53(const DrawStream &ds) const { return u[ds.d - base]; }
 };
+
+// A macro atom's internal jumps (Sect. 2.5) by a whole warp (a lone walk): a jump's targets in coalesced
+// loads, 32 entries a round, the first with the draw below its threshold by a vote.
+template <class Draws>
+__device__ __forceinline__ unsigned long long macroatom_walk_lone(const MaRow *rows, const MaJump *jumps, int32_t row,
+                                                                  const Draws &md, unsigned lane) {
+  for (uint32_t n = 0; n < kMaMaxJumps; ++n) {
+    const MaRow *mr = rows + row;
+    const unsigned long long thr = __ldg(&mr->jump_thr);
+    const uint2 jb = __ldg(reinterpret_cast<const uint2 *>(&mr->jump_begin));  // begin, length
+    const uint2 db = __ldg(reinterpret_cast<const uint2 *>(&mr->dbr_begin));
+    const unsigned long long za = md.next();
+    if (!(za < thr)) return static_cast<unsigned long long>(db.x) | (static_cast<unsigned long long>(db.y) << 32);
+    const unsigned long long zb = md.next();
+    const MaJump *jp = jumps + jb.x;
+    for (uint32_t i0 = 0;; i0 += 32u) {  // (the last threshold is 2^53 > zb; past the end the last entry)
+      const uint32_t i = min(i0 + lane, jb.y - 1u);
+      const unsigned m = __ballot_sync(0xffffffffu, zb < __ldg(&jp[i].thr));
+      const int32_t t = __ldg(&jp[i].target);
+      if (m != 0u || i0 + 32u >= jb.y) {
+        row = __shfl_sync(0xffffffffu, t, m != 0u ? __ffs(m) - 1 : 31);
+        break;
+      }
+    }
+  }
+  const uint2 db = __ldg(reinterpret_cast<const uint2 *>(&rows[row].dbr_begin));
+  return static_cast<unsigned long long>(db.x) | (static_cast<unsigned long long>(db.y) << 32);
+}
 
 // The pool of walks handed over.  A walk is written, then its place marked; a
 // taker reads the mark, then claims the place.  Nothing waits: a place given

@@ -126,6 +126,27 @@ __device__ __forceinline__ unsigned long long macroatom_walk(const TransportPara
   return static_cast<unsigned long long>(db.x) | (static_cast<unsigned long long>(db.y) << 32);
 }
 
+// The emitted line of entries [lo, hi] of the caller's table by a whole warp: the
+// first entry k with u 2^-53 < cdf[k] (the last's cdf is 1), 32 probes a round.
+__device__ __forceinline__ int32_t search_cdf_lone(const TransportParams &p, uint32_t lo, uint32_t hi,
+                                                   unsigned long long u, unsigned lane) {
+  const long long kz = __double_as_longlong(static_cast<double>(u) * 0x1.0p-53);
+  const long long *cb = reinterpret_cast<const long long *>(p.dbr_cdf);
+  while (lo < hi) {
+    const uint32_t n = hi - lo, step = (n + 31u) >> 5;
+    const uint32_t i = lo + min((lane + 1u) * step, n) - 1u;
+    const unsigned m = __ballot_sync(0xffffffffu, kz < __ldg(cb + i));
+    if (m == 0u) {
+      lo = hi;
+    } else {
+      const uint32_t k = static_cast<uint32_t>(__ffs(m)) - 1u;
+      hi = lo + min((k + 1u) * step, n) - 1u;
+      lo += k * step;
+    }
+  }
+  return static_cast<int32_t>(__ldg(p.dbr_line + lo));
+}
+
 // max(v, 0) through the integer keys (no binary64 instruction).
 __device__ __forceinline__ double max0(double v) { return rawkey(v) > 0 ? v : 0.0; }
 
@@ -380,7 +401,7 @@ struct MaDraws {
 // 3 downbranch from the caller's table alone (no bucket slots).
 // VIRT: with virtual packets.
 template <int LINES, bool JB, bool REC, bool VIRT>
-__global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p) {
+__global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParams p) {
   constexpr int MODE = LINES == 3 ? 1 : LINES;
   constexpr bool kSlots = LINES == 1 || LINES == 2;  // the model's tables: bucket slots, row info
   extern __shared__ double sh[];
@@ -717,6 +738,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
         w_t = __longlong_as_double(static_cast<long long>(
             load_here(p.tau + static_cast<size_t>(cs) * static_cast<size_t>(L) + jj)));
         if (LINES == 1) w_r = load_here(p.row_info + jj);
+        if (LINES >= 2) w_r = load_here32(p.line_row + jj);
       };
       reload(pk.next_line);
       // After a line's re-emission E/nu and 1/nu_lab are taken when the next event
@@ -775,7 +797,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
       bool stopped = false;
       need_cmf();
       while (status == 0) {
-        if (LINES == 1) {
+        if (LINES != 0) {
           // Line event after line event, the bulk of a trapped walk: a loop of its
           // own, so that the loads in flight stay in their registers from where
           // they are issued to where they are used (a copy of one where paths meet
@@ -784,8 +806,8 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
           while (!p.timeout_ns && ((polls + 1u) & 255u) != 0u && pk.cnt[0] < cap) {
             ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, false);
             const uint32_t di = d - ld.base;
-            const unsigned long long u_em = ld.u[di + 1u];
-            const double mu = ld.m[di + 2u];
+            unsigned long long u_em = ld.u[di + 1u];
+            double mu = ld.m[di + 2u];
             const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);
             const ScanF f = scan_setup(pk.nu_cmf, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, ld.t[di]);
             const bool there = w0 + static_cast<int32_t>(lane) < L;
@@ -799,9 +821,14 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
             const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
             const int k = 31 - __clz(thick & (0u - thick));
             const long long hit = __shfl_sync(F, w_b, k);
-            const unsigned long long rinfo = __shfl_sync(F, w_r, k);
+            unsigned long long rinfo = __shfl_sync(F, w_r, k);
             uint4 ra, rc;
-            load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+            uint32_t row_lo = 0u, row_hi = 0u;
+            if (LINES == 1) load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+            if (LINES == 3) {
+              row_lo = load_here32(p.dbr_offset + rinfo);
+              row_hi = load_here32(p.dbr_offset + rinfo + 1);
+            }
             const bool prior = static_cast<int>(lane) < k;
             const unsigned sum = __reduce_add_sync(
                 F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
@@ -810,9 +837,20 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
             const bool good = static_cast<int>(lane) == k ? (inside && rk > M + 0x1.0p-15f && l > 0x1.0p-40f)
                                                           : !(prior && own < 0.0f);
             if (!__all_sync(F, good) || thick == 0u) break;
+            d += 1u;
+            if (LINES == 2) {  // internal jumps, then the record of the level they end in
+              const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
+              rinfo = macroatom_walk_lone(p.ma_row, p.ma_jump, static_cast<int32_t>(rinfo), md, lane);
+              u_em = md.next();
+              load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+              mu = d - ld.base < kWarpDraws ? ld.m[d - ld.base] : DrawStream::mu_from_u53(u53_past_buffer(
+                  p.key0, p.key1, pk.pid, p.iteration, d));
+              d += 1u;
+            } else {
+              d += 2u;
+            }
             settle();
             polls += 1u;
-            d += 3u;
             pk.cnt[0] += 1u;
             pk.cnt[1] += static_cast<uint32_t>(k) + 1u;
             pk.cnt[2] += static_cast<uint32_t>(k) + 1u;
@@ -825,11 +863,16 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
             const double pl = fma(-nuj, pk.inv_nu, 1.0);
             const double r2 = fma(pl, pl, pk.q);
             log_segment(lp, w0, k + 1);
-            // (not before r2 is there: scheduled earlier, it would wait for the
-            // record with the event's arithmetic behind it)
-            int32_t em = slot_line(ra, rc, u_em ^ (static_cast<unsigned long long>(
-                                               static_cast<uint32_t>(__double2hiint(r2)) & p.zero) << 32));
-            if (em < 0) em = search_row_lone(p.dbr_rec, rinfo, rc.z, u_em, lane);
+            int32_t em;
+            if (kSlots) {
+              // (not before r2 is there: scheduled earlier, it would wait for the
+              // record with the event's arithmetic behind it)
+              em = slot_line(ra, rc, u_em ^ (static_cast<unsigned long long>(
+                                         static_cast<uint32_t>(__double2hiint(r2)) & p.zero) << 32));
+              if (em < 0) em = search_row_lone(p.dbr_rec, rinfo, rc.z, u_em, lane);
+            } else {
+              em = search_cdf_lone(p, row_lo, row_hi - 1u, u_em, lane);
+            }
             reload(em + 1);
             pk.next_line = em + 1;
             pk.nu_cmf = __longlong_as_double(static_cast<long long>(load_here(p.nu + em)));
@@ -993,7 +1036,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
           int32_t em = 0;
           if (MODE == 2) {
             const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
-            rinfo = macroatom_walk(p, __ldg(p.line_row + j), md);
+            rinfo = macroatom_walk_lone(p.ma_row, p.ma_jump, __ldg(p.line_row + j), md, lane);
             em = downbranch_pick<true>(p, j, rinfo, md.next());
             mu = DrawStream::mu_from_u53(md.next());
           } else if (MODE == 1) {
@@ -1057,7 +1100,7 @@ __global__ void __launch_bounds__(kBlock) transport_fp64(const TransportParams p
             vdraws += static_cast<uint32_t>(p.n_virtual);
           }
         }
-        if (LINES == 1 ? pk.next_line != w0 : pk.next_line < w0 || pk.next_line - w0 >= 32)
+        if (LINES != 0 ? pk.next_line != w0 : pk.next_line < w0 || pk.next_line - w0 >= 32)
           reload(pk.next_line);  // behind the window (or the loop above starts at its first lane)
         if (status == 0) need_cmf();
       }

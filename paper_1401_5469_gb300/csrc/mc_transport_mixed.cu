@@ -179,6 +179,12 @@ __device__ __forceinline__ unsigned long long ma_draw(DrawStream &ds, const Warp
   return u53_past_buffer(ds.k0, ds.k1, ds.packet, ds.iteration, ds.d - 1u);
 }
 
+struct LoneMaDraws {
+  DrawStream *ds;
+  const WarpDraws *wd;
+  __device__ __forceinline__ unsigned long long next() const { return ma_draw(*ds, wd); }
+};
+
 __device__ __forceinline__ unsigned long long macroatom_walk_m(const MCtx &c, int32_t row, DrawStream &ds,
                                                                const WarpDraws *wd) {
   for (uint32_t n = 0; n < kMaMaxJumps; ++n) {
@@ -530,7 +536,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
       r = __shfl_sync(0xffffffffu, lwin_r, idx);
     };
 
-    if (kLoneBuild && MODE == 1 && lone && pk.next_line < c.L) {
+    if (kLoneBuild && MODE >= 1 && lone && pk.next_line < c.L) {
       // Line event after line event of a lone walk, the bulk of a trapped walk,
       // in a loop of its own (the binary64 kernel's: loads stay in their
       // registers from where they are issued to where they are used).  The
@@ -568,12 +574,13 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         const int32_t jj = min(w0 + static_cast<int32_t>(lane), c.L - 1);
         w_b = static_cast<long long>(load_here(nub + jj));
         w_t = load_here_f(tau_s + jj);
-        w_r = load_here(c.row_info + jj);
+        if (MODE == 1) w_r = load_here(c.row_info + jj);
+        else w_r = load_here32(c.line_row + jj);
       };
       w_b = lwin_b;
       w_t = lwin_t;
       w_r = lwin_r;
-      if (lwin_s != cs || lwin_j0 != w0) reload();
+      if (MODE == 2 || lwin_s != cs || lwin_j0 != w0) reload();
       double nu_c = pk.nu_lab * f64_of_f32(1.0f - pk.p), r1 = 0.0;
       float inv_c = 0.0f, g_w = 0.0f, g_b = 0.0f;
       uint32_t n_log = 0u;
@@ -590,7 +597,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
         const uint32_t di = ds.d - wd.base;
         const float tau0 = -__logf(open0f(wd.u[di]));
-        const unsigned long long u_em = wd.u[di + 1u], um = wd.u[di + 2u];
+        unsigned long long u_em = wd.u[di + 1u], um = wd.u[di + 2u];
         const float pp = pk.p, q = pk.q, Df = 1.0f - pp;
         const bool inner = pp < 0.0f && q <= c_xi2;
         const float lx = Df - (1.0f - shell_exit_f(q, inner, c_xi2, c_xo2));
@@ -608,9 +615,9 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
         const int k = 31 - __clz(thick & (0u - thick));
         const long long hit = __shfl_sync(F, w_b, k);
-        const unsigned long long rinfo = __shfl_sync(F, w_r, k);
+        unsigned long long rinfo = __shfl_sync(F, w_r, k);
         uint4 ra, rc;
-        load_slot_here64(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
+        if (MODE == 1) load_slot_here64(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
         const bool prior = static_cast<int>(lane) < k;
         const unsigned sum = __reduce_add_sync(
             F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
@@ -629,7 +636,16 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         const float lj = f32_of_f64_max0(nu_cmf - __longlong_as_double(hit)) * inv_nu;
         if (k == 0 && !inside_shell_f(pp, q, lj, inner, c_xi2, c_xo2)) break;
         polls += 1u;
-        ds.d += 3u;
+        if (MODE == 2) {  // internal jumps, then the record of the level they end in
+          ds.d += 1u;
+          const LoneMaDraws md{&ds, &wd};
+          rinfo = macroatom_walk_lone(c.ma_row, c.ma_jump, static_cast<int32_t>(rinfo), md, lane);
+          u_em = md.next();
+          load_slot_here64(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
+          um = md.next();
+        } else {
+          ds.d += 3u;
+        }
         pk.cnt[0] += 1u;
         pk.cnt[1] += static_cast<uint32_t>(k) + 1u;
         pk.cnt[2] += static_cast<uint32_t>(k) + 1u;
