@@ -103,6 +103,14 @@ __device__ __forceinline__ float f32_rz_small(double d) {
   return __uint_as_float((a >= 0x38100000u ? m : 0u) | (hi & 0x80000000u));
 }
 
+// The same for a depth: at most the largest finite value.
+__device__ __forceinline__ float f32_rz_below_inf(double d) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(d)), lo = static_cast<uint32_t>(__double2loint(d));
+  const uint32_t a = min(hi & 0x7fffffffu, 0x47efffffu);
+  const uint32_t m = __funnelshift_l(lo, a - 0x38000000u, 3);
+  return __uint_as_float((a >= 0x38100000u ? m : 0u) | (hi & 0x80000000u));
+}
+
 // v < 0, excluding -0 (its pattern is the most negative integer).
 __device__ __forceinline__ bool strictly_negative(double v) {
   const long long b = __double_as_longlong(v);
@@ -330,12 +338,16 @@ __device__ __forceinline__ float neg_log_u53_f(unsigned long long u) {
 // bucket floor(z n), whose slot settles most draws.
 // The bucket slot of draw u in the row of rinfo (begin | length << 32):
 // floor(u n / 2^53) in two 32-bit products.
-__device__ __forceinline__ const DbrSlot *bucket_slot(const DbrSlot *slots, unsigned long long rinfo,
-                                                      unsigned long long u) {
+__device__ __forceinline__ uint32_t bucket_index(unsigned long long rinfo, unsigned long long u) {
   const uint32_t b = static_cast<uint32_t>(rinfo), len = static_cast<uint32_t>(rinfo >> 32);
   const unsigned long long lo = static_cast<unsigned long long>(static_cast<uint32_t>(u)) * len;
   const unsigned long long s = static_cast<unsigned long long>(static_cast<uint32_t>(u >> 32)) * len + (lo >> 32);
-  return slots + b + static_cast<uint32_t>(s >> 21);
+  return b + static_cast<uint32_t>(s >> 21);  // (row offsets are 32-bit: so is every index)
+}
+
+__device__ __forceinline__ const DbrSlot *bucket_slot(const DbrSlot *slots, unsigned long long rinfo,
+                                                      unsigned long long u) {
+  return slots + bucket_index(rinfo, u);
 }
 
 __device__ __forceinline__ void load_slot(const DbrSlot *slot, uint4 &a, uint4 &c) {

@@ -20,7 +20,7 @@ size_t smem_bytes(int S, int precision, bool virt) {
   // binary64: shell tables, then per warp a lone walk's state and draws, and the
   // queued launches of v-packets
   return precision == 1 ? mixed_smem_bytes(S)
-                        : static_cast<size_t>(kShellArrays) * S * sizeof(double) +
+                        : shell_words(S) * sizeof(double) +
                               (kBlock / 32) * (kLoneBytes + (virt ? kVirtualQueue * sizeof(VirtualLaunch) : 0));
 }
 

@@ -40,8 +40,10 @@ namespace {
 
 constexpr int kBlock = 128;
 // per warp: a walk handed to all lanes, then its draws
-constexpr size_t kLoneBytes = sizeof(PoolWalk) + kWarpDraws * (2 * sizeof(double) + sizeof(float));
-constexpr int kShellArrays = 6;  // x_in^2, x_out^2, x_in, x_out, kappa, 1/kappa
+constexpr size_t kDrawBytes = kWarpDraws * (2 * sizeof(double) + sizeof(float));
+constexpr size_t kLoneBytes = sizeof(PoolWalk) + kDrawBytes + 32 * 2 * sizeof(double2);
+// doubles of the shell tables x_in^2, x_out^2, x_in, x_out, kappa (what follows is 16-byte aligned)
+__host__ __device__ constexpr size_t shell_words(int S) { return (5 * static_cast<size_t>(S) + 1) & ~size_t{1}; }
 constexpr int kLineEvent = 1, kElectronEvent = 2, kShellEvent = 3;
 
 struct Packet {
@@ -334,10 +336,10 @@ __device__ __noinline__ void fly_virtual(const TransportParams &p, const double 
 // Path length to the exit: x mu there is +-sqrt(x_b^2 - q) (P, in binary32 from
 // the operands truncated, the difference's error e1 carried through the root).
 // Near-tangent exits (x_b^2 - q within 4 e1) are not bounded.
-__device__ __forceinline__ ScanF scan_setup(double nu_cmf, double p, double q, float kap, bool inner,
+__device__ __forceinline__ ScanF scan_setup(double nu_cmf, float pf, float qf, float kap, bool inner,
                                             float xi2, float xo2, float tau) {
   ScanF f;
-  const float pf = f32_rz_small(p), qf = f32_rz_small(q), Df = 1.0f - pf;
+  const float Df = 1.0f - pf;
   f.tf = kap * Df;
   f.tau = tau;
   const float xb2 = inner ? xi2 : xo2;
@@ -413,10 +415,9 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
     sh[2 * S + i] = xi;
     sh[3 * S + i] = xo;
     sh[4 * S + i] = kap;
-    sh[5 * S + i] = p.inv_kappa ? p.inv_kappa[i] : (kap > 0.0 ? 1.0 / kap : 0.0);
   }
   __syncthreads();
-  const double *s_xi2 = sh, *s_xo2 = sh + S, *s_kap = sh + 4 * S, *s_ikap = sh + 5 * S;
+  const double *s_xi2 = sh, *s_xo2 = sh + S, *s_kap = sh + 4 * S;
   const double x0 = sh[2 * S], x0sq = sh[0];
 
   const unsigned lane = threadIdx.x & 31u;
@@ -443,7 +444,7 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
   bool drained = false;  // warp-uniform: the packet queue is empty
   uint32_t vdraws = 0u;  // v-packet draws used by this lane's packet
   // the warp's queued launches (VIRT)
-  VirtualLaunch *vq = reinterpret_cast<VirtualLaunch *>(reinterpret_cast<char *>(sh + kShellArrays * S) +
+  VirtualLaunch *vq = reinterpret_cast<VirtualLaunch *>(reinterpret_cast<char *>(sh + shell_words(S)) +
                                                         (kBlock / 32) * kLoneBytes) +
                       kVirtualQueue * (threadIdx.x >> 5);
   unsigned n_vq = 0u;
@@ -538,7 +539,7 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
     long long key_e = kKeyNegInf;
     thr = 0.0;
     if (thomson) {
-      c_e = (nu_lab * s_ikap[cs]) * rcp64(pk.D);  // nu_lab / k, k = kappa' D
+      c_e = (nu_lab * (p.inv_kappa ? __ldg(p.inv_kappa + cs) : 1.0 / kap)) * rcp64(pk.D);  // nu_lab / k, k = kappa' D
       thr = fma(-tau, c_e, pk.nu_cmf);
     }
     for (int32_t i = j0; i < j; ++i) {
@@ -672,7 +673,7 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
         atomicAdd(nb_sum + acc_s, acc_nb);
       }
       acc_s = -1;
-      char *warp_mem = reinterpret_cast<char *>(sh + kShellArrays * S) + kLoneBytes * (threadIdx.x >> 5);
+      char *warp_mem = reinterpret_cast<char *>(sh + shell_words(S)) + kLoneBytes * (threadIdx.x >> 5);
       const PoolWalk *from = p.pool + from_pool;
       if (from_pool < 0) {
         const unsigned age = alive ? pk.cnt[0] + 1u : 0u;
@@ -754,34 +755,38 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
           fresh = false;
         }
       };
-      // The estimator terms of a segment (Eqs. 13-14) are kept by one lane and
-      // evaluated for 32 segments at once.
-      // ... and so are the J_blue sums of the lines it passed (g_n lines from cell
-      // g_j on; the weight E_lab / nu_lab^2 is E/nu times 1/nu_lab).
-      double g_e = 0.0, g_i = 0.0, g_l = 0.0, g_nu = 0.0;  // E/nu, 1/nu_lab, path length, nu_cmf
-      int32_t g_j = 0, g_n = 0;
+      // The estimator terms of a segment (Eqs. 13-14) are logged in shared memory
+      // (all lanes store the same values to one place) and evaluated for 32 segments
+      // at once, a lane each.
+      double2 *lg_x = reinterpret_cast<double2 *>(warp_mem + sizeof(PoolWalk) + kDrawBytes);
       uint32_t n_log = 0u;
       double a_j = 0.0, a_nb = 0.0;  // this lane's sums in shell cs
       auto sum_log = [&]() {
-        const double wgt = ((g_e * g_nu) * (g_nu * g_i)) * g_l;  // E_cmf D l
-        a_j += wgt;
-        a_nb = fma(wgt, g_nu, a_nb);
-        g_l = 0.0;
-        n_log = 0u;
-        if (JB) {
-          const double e_inv2 = g_e * g_i;
-          double *cell = p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L) + g_j;
-          for (int32_t i = 0; i < g_n; ++i) red_add_evict_first(cell + i, e_inv2, jb_pol);
-          g_n = 0;
+        __syncwarp();
+        double wgt = 0.0, nu = 0.0;
+        if (lane < n_log) {
+          const double2 x = lg_x[2u * lane], y = lg_x[2u * lane + 1u];
+          nu = y.y;
+          wgt = ((x.x * nu) * (nu * x.y)) * y.x;  // E_cmf D l
         }
+        __syncwarp();
+        a_j += wgt;
+        a_nb = fma(wgt, nu, a_nb);
+        n_log = 0u;
+      };
+      auto put_log = [&](double l) {
+        lg_x[2u * n_log] = make_double2(pk.e_per_nu, pk.inv_nu);
+        lg_x[2u * n_log + 1u] = make_double2(l, pk.nu_cmf);  // path length, nu_cmf
+        ++n_log;
       };
       auto log_segment = [&](double l, int32_t j, int32_t n) {
-        if (lane == n_log) { g_e = pk.e_per_nu; g_i = pk.inv_nu; g_l = l; g_nu = pk.nu_cmf; g_j = j; g_n = n; }
-        ++n_log;
-#pragma unroll 1
-        while (n_log == 32u) {  // (a loop, and opaque: not evaluated for every segment)
-          asm volatile("" : "+d"(g_e), "+d"(g_l), "+d"(g_i), "+d"(g_nu));
-          sum_log();
+        if (n_log == 32u) sum_log();
+        put_log(l);
+        if (JB) {
+          const double e_inv2 = pk.e_per_nu * pk.inv_nu;
+          double *cell = p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L) + j;
+          for (int32_t i = static_cast<int32_t>(lane); __any_sync(F, i < n); i += 32)
+            if (i < n) red_add_evict_first(cell + i, e_inv2, jb_pol);
         }
       };
       auto flush_shell = [&]() {
@@ -803,92 +808,123 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
           // they are issued to where they are used (a copy of one where paths meet
           // would wait for it).  It leaves, with nothing changed, at a segment that
           // is anything else.
-          while (!p.timeout_ns && ((polls + 1u) & 255u) != 0u && pk.cnt[0] < cap) {
+          // What bounds it is the number of its instructions: a lone warp issues one in
+          // 4 to 5 cycles (fixed-latency stalls 3.1 of the 5.9 cycles between issues,
+          // waits for loads 0.6), 416 of them a segment before these steps.  So the
+          // segments it may take are counted out beforehand (to the next look at the
+          // stop word, the cap, 32 logged, three draws each), its counters are two, a
+          // segment's estimator terms are two shared stores, and the J_blue terms of
+          // the lines passed one atomic of the lanes.  A walk of 94,495 segments alone:
+          // 100.4 -> 76.7 ms, with J_blue (and its zeroing, which leaves the caches
+          // cold) 96.0 -> 89.8; 5e4 lines, 1e5 packets: 32.6 -> 25.5 ms.
+          bool certain = !p.timeout_ns;
+          while (certain) {
+            if (n_log == 32u) sum_log();
             ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, false);
-            const uint32_t di = d - ld.base;
-            unsigned long long u_em = ld.u[di + 1u];
-            double mu = ld.m[di + 2u];
-            const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);
-            const ScanF f = scan_setup(pk.nu_cmf, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, ld.t[di]);
-            const bool there = w0 + static_cast<int32_t>(lane) < L;
-            bool ok;
-            const float l = scan_delta(f, w_b, ok) * f.lf;
-            const float a = l * f.tf;
-            const float own = there ? f32_rz_any(w_t) : 0.0f;
-            const float M = fmaf(0x1.0p-19f + 0x1.0p-18f, a + f.tau, fmaf(f.tf, 0x1.0p-43f, 0x1.0p-100f));
-            const float left = f.tau - a;
-            const bool inside = f.lx - l > fmaf(0x1.0p-19f, l, f.mx);
-            const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
-            const int k = 31 - __clz(thick & (0u - thick));
-            const long long hit = __shfl_sync(F, w_b, k);
-            unsigned long long rinfo = __shfl_sync(F, w_r, k);
-            uint4 ra, rc;
-            uint32_t row_lo = 0u, row_hi = 0u;
-            if (LINES == 1) load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
-            if (LINES == 3) {
-              row_lo = load_here32(p.dbr_offset + rinfo);
-              row_hi = load_here32(p.dbr_offset + rinfo + 1);
-            }
-            const bool prior = static_cast<int>(lane) < k;
-            const unsigned sum = __reduce_add_sync(
-                F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
-            const float rk = left - static_cast<float>(sum) * 0x1.0p-21f;
-            // (and the point lies ahead of the packet, beyond its rounding)
-            const bool good = static_cast<int>(lane) == k ? (inside && rk > M + 0x1.0p-15f && l > 0x1.0p-40f)
-                                                          : !(prior && own < 0.0f);
-            if (!__all_sync(F, good) || thick == 0u) break;
-            d += 1u;
-            if (LINES == 2) {  // internal jumps, then the record of the level they end in
-              const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
-              rinfo = macroatom_walk_lone(p.ma_row, p.ma_jump, static_cast<int32_t>(rinfo), md, lane);
-              u_em = md.next();
-              load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
-              mu = d - ld.base < kWarpDraws ? ld.m[d - ld.base] : DrawStream::mu_from_u53(u53_past_buffer(
-                  p.key0, p.key1, pk.pid, p.iteration, d));
-              d += 1u;
-            } else {
-              d += 2u;
-            }
-            settle();
-            polls += 1u;
-            pk.cnt[0] += 1u;
-            pk.cnt[1] += static_cast<uint32_t>(k) + 1u;
-            pk.cnt[2] += static_cast<uint32_t>(k) + 1u;
-            pk.cnt[3] += 1u;
-            // line_point and sqrt64 without their special cases (a binary64
-            // result takes 45 cycles longer to an integer compare than to the
-            // next binary64 instruction)
-            const double nuj = __longlong_as_double(hit);
-            const double lp = fma(-nuj, pk.inv_nu, pk.D);
-            const double pl = fma(-nuj, pk.inv_nu, 1.0);
-            const double r2 = fma(pl, pl, pk.q);
-            log_segment(lp, w0, k + 1);
-            int32_t em;
-            if (kSlots) {
-              // (not before r2 is there: scheduled earlier, it would wait for the
-              // record with the event's arithmetic behind it)
-              em = slot_line(ra, rc, u_em ^ (static_cast<unsigned long long>(
-                                         static_cast<uint32_t>(__double2hiint(r2)) & p.zero) << 32));
-              if (em < 0) em = search_row_lone(p.dbr_rec, rinfo, rc.z, u_em, lane);
-            } else {
-              em = search_cdf_lone(p, row_lo, row_hi - 1u, u_em, lane);
-            }
-            reload(em + 1);
-            pk.next_line = em + 1;
-            pk.nu_cmf = __longlong_as_double(static_cast<long long>(load_here(p.nu + em)));
-            // ... and while the window is on its way:
-            const double xn = sqrt64_pos(r2);
-            pk.e_cmf = pk.e_per_nu * nuj;
-            const double pn = xn * mu;
-            pk.D = fma(-xn, mu, 1.0);
-            pk.p = pn;
-            pk.q = max0(fma(-pn, pn, r2));
-            pk.have_lab = false;
-            fresh = true;
-            if (VIRT) {
-              queue_virtual(lane == 0u, VirtualLaunch{xn, r2, pk.nu_cmf, pk.e_cmf, cs, em + 1, pk.pid, vdraws});
-              vdraws += static_cast<uint32_t>(p.n_virtual);
-            }
+            uint32_t di = d - ld.base, n_ev = 0u, n_line = 0u;
+            uint32_t room = min(min(255u - (polls & 255u), cap - pk.cnt[0]), 32u - n_log);
+            if (LINES != 2) room = min(room, (kWarpDraws - di) / 3u);
+            if (room == 0u) break;
+#pragma unroll 1
+            do {
+              unsigned long long u_em = ld.u[di + 1u];
+              double mu = ld.m[di + 2u];
+              const float pf = f32_rz_small(pk.p), qf = f32_rz_small(pk.q);
+              // (truncation keeps the order, and at equality the exit is not bounded)
+              const bool inner = pf < 0.0f && qf <= f_xi2;
+              const ScanF f = scan_setup(pk.nu_cmf, pf, qf, f_kap, inner, f_xi2, f_xo2, ld.t[di]);
+              // (each lane the record index of its own line, while the scan runs)
+              const uint32_t my_slot = LINES == 1 ? bucket_index(w_r, u_em) : 0u;
+              const bool there = w0 + static_cast<int32_t>(lane) < L;
+              bool ok;
+              const float l = scan_delta(f, w_b, ok) * f.lf;
+              const float a = l * f.tf;
+              const float own = there ? f32_rz_below_inf(w_t) : 0.0f;
+              const float M = fmaf(0x1.0p-19f + 0x1.0p-18f, a + f.tau, fmaf(f.tf, 0x1.0p-43f, 0x1.0p-100f));
+              const float left = f.tau - a;
+              const bool inside = f.lx - l > fmaf(0x1.0p-19f, l, f.mx);
+              const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
+              const int k = 31 - __clz(thick & (0u - thick));
+              const long long hit = __shfl_sync(F, w_b, k);
+              uint4 ra, rc;
+              uint32_t row_lo = 0u, row_hi = 0u;
+              if (LINES == 1) load_slot_here(p.dbr_bucket + __shfl_sync(F, my_slot, k), ra, rc);
+              unsigned long long rinfo = __shfl_sync(F, w_r, k);
+              if (LINES == 3) {
+                row_lo = load_here32(p.dbr_offset + rinfo);
+                row_hi = load_here32(p.dbr_offset + rinfo + 1);
+              }
+              const bool prior = static_cast<int>(lane) < k;
+              const unsigned sum = __reduce_add_sync(
+                  F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
+              const float rk = left - static_cast<float>(sum) * 0x1.0p-21f;
+              // (and the point lies ahead of the packet, beyond its rounding)
+              const bool good = static_cast<int>(lane) == k ? (inside && rk > M + 0x1.0p-15f && l > 0x1.0p-40f)
+                                                            : !(prior && own < 0.0f);
+              certain = __all_sync(F, good) && thick != 0u;
+              if (!certain) break;
+              if (LINES == 2) {  // internal jumps, then the record of the level they end in
+                d = ld.base + di + 1u;
+                const MaDraws md{nullptr, &ld, &d, p.key0, p.key1, pk.pid, p.iteration};
+                rinfo = macroatom_walk_lone(p.ma_row, p.ma_jump, static_cast<int32_t>(rinfo), md, lane);
+                u_em = md.next();
+                load_slot_here(bucket_slot(p.dbr_bucket, rinfo, u_em), ra, rc);
+                mu = d - ld.base < kWarpDraws ? ld.m[d - ld.base] : DrawStream::mu_from_u53(u53_past_buffer(
+                    p.key0, p.key1, pk.pid, p.iteration, d));
+                di = d + 1u - ld.base;
+              } else {
+                di += 3u;
+              }
+              settle();
+              n_ev += 1u;
+              n_line += static_cast<uint32_t>(k);
+              // line_point and sqrt64 without their special cases (a binary64
+              // result takes 45 cycles longer to an integer compare than to the
+              // next binary64 instruction)
+              const double nuj = __longlong_as_double(hit);
+              const double lp = fma(-nuj, pk.inv_nu, pk.D);
+              const double pl = fma(-nuj, pk.inv_nu, 1.0);
+              const double r2 = fma(pl, pl, pk.q);
+              put_log(lp);
+              if (JB) {
+                const double e_inv2 = pk.e_per_nu * pk.inv_nu;
+                if (static_cast<int>(lane) <= k)
+                  red_add_evict_first(p.j_blue + static_cast<size_t>(cs) * static_cast<size_t>(L) + w0 +
+                                          static_cast<int32_t>(lane), e_inv2, jb_pol);
+              }
+              int32_t em;
+              if (kSlots) {
+                // (not before r2 is there: scheduled earlier, it would wait for the
+                // record with the event's arithmetic behind it)
+                em = slot_line(ra, rc, u_em ^ (static_cast<unsigned long long>(
+                                           static_cast<uint32_t>(__double2hiint(r2)) & p.zero) << 32));
+                if (em < 0) em = search_row_lone(p.dbr_rec, rinfo, rc.z, u_em, lane);
+              } else {
+                em = search_cdf_lone(p, row_lo, row_hi - 1u, u_em, lane);
+              }
+              reload(em + 1);
+              pk.next_line = em + 1;
+              pk.nu_cmf = __longlong_as_double(static_cast<long long>(load_here(p.nu + em)));
+              // ... and while the window is on its way:
+              const double xn = sqrt64_pos(r2);
+              pk.e_cmf = pk.e_per_nu * nuj;
+              const double pn = xn * mu;
+              pk.D = fma(-xn, mu, 1.0);
+              pk.p = pn;
+              pk.q = max0(fma(-pn, pn, r2));
+              pk.have_lab = false;
+              fresh = true;
+              if (VIRT) {
+                queue_virtual(lane == 0u, VirtualLaunch{xn, r2, pk.nu_cmf, pk.e_cmf, cs, em + 1, pk.pid, vdraws});
+                vdraws += static_cast<uint32_t>(p.n_virtual);
+              }
+            } while (n_ev != room && (LINES != 2 || di + 3u <= kWarpDraws));
+            polls += n_ev;
+            pk.cnt[0] += n_ev;
+            pk.cnt[1] += n_line + n_ev;
+            pk.cnt[2] += n_line + n_ev;
+            pk.cnt[3] += n_ev;
+            d = ld.base + di;
           }
         }
         if (p.timeout_ns && __any_sync(F, (global_ns() - t_start) > p.timeout_ns)) {
@@ -913,7 +949,7 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
         const unsigned long long u_em = ld.u[di + 1u];
         const double mu_line = ld.m[di + (MODE == 1 ? 2u : 1u)];
         const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);
-        const ScanF f = scan_setup(pk.nu_cmf, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2, ld.t[di]);
+        const ScanF f = scan_setup(pk.nu_cmf, f32_rz_small(pk.p), f32_rz_small(pk.q), f_kap, inner, f_xi2, f_xo2, ld.t[di]);
         const int32_t j0 = pk.next_line;
         int32_t j = j0, j_log = j0;  // the lines passed before j_log have their J_blue sums
         int kind = -1;               // -1 open, 0 in doubt
@@ -1151,7 +1187,7 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
       // optical depth to the next event, tau = -ln z
       const unsigned long long u_tau = ds.next_u53();
       const bool inner = strictly_negative(pk.p) && rawkey(pk.q) <= rawkey(c_xi2);  // q, x_in^2 >= 0
-      const ScanF f = scan_setup(pk.nu_cmf, pk.p, pk.q, f_kap, inner, f_xi2, f_xo2,
+      const ScanF f = scan_setup(pk.nu_cmf, f32_rz_small(pk.p), f32_rz_small(pk.q), f_kap, inner, f_xi2, f_xo2,
                                  neg_log_u53_f(u_tau + 1ull));
       // J_blue weight of this segment, E_lab / nu_lab^2 (Eq. 17 without its
       // line factor nu_j, applied per cell after the launch)

@@ -593,103 +593,117 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         g_b = 0.0f;
         n_log = 0u;
       };
-      while (!p.timeout_ns && ((polls + 1u) & 255u) != 0u && pk.cnt[0] < cap) {
+      // (The segments of the inner loop are counted out beforehand, as in the
+      // binary64 kernel: to the next look at the stop word, the cap, 32 logged,
+      // three draws each.)
+      bool certain = !p.timeout_ns;
+      while (certain) {
+        if (n_log == 32u) sum_log();
         wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
-        const uint32_t di = ds.d - wd.base;
-        const float tau0 = -__logf(open0f(wd.u[di]));
-        unsigned long long u_em = wd.u[di + 1u], um = wd.u[di + 2u];
-        const float pp = pk.p, q = pk.q, Df = 1.0f - pp;
-        const bool inner = pp < 0.0f && q <= c_xi2;
-        const float lx = Df - (1.0f - shell_exit_f(q, inner, c_xi2, c_xo2));
-        ScanF f;
-        f.tf = c_kap * Df;
-        scan_frequency(f, nu_c, Df);
-        const bool there = w0 + static_cast<int32_t>(lane) < c.L;
-        bool ok;
-        const float l = scan_delta(f, w_b, ok) * f.lf;
-        const float a = l * f.tf;
-        const float own = there ? w_t : 0.0f;
-        const float M = fmaf(0x1.0p-19f + 0x1.0p-18f, a + tau0, fmaf(f.tf, 0x1.0p-43f, 0x1.0p-100f));
-        const float left = tau0 - a;
-        const bool inside = lx - l > fmaf(0x1.0p-19f, l, 0x1.0p-43f);
-        const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
-        const int k = 31 - __clz(thick & (0u - thick));
-        const long long hit = __shfl_sync(F, w_b, k);
-        unsigned long long rinfo = __shfl_sync(F, w_r, k);
-        uint4 ra, rc;
-        if (MODE == 1) load_slot_here64(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
-        const bool prior = static_cast<int>(lane) < k;
-        const unsigned sum = __reduce_add_sync(
-            F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
-        const float rk = left - static_cast<float>(sum) * 0x1.0p-21f;
-        const bool good = static_cast<int>(lane) == k
-                              ? (f.ec > 0 && f.ec < 2047 && (inside || k == 0) && rk > M + 0x1.0p-15f)
-                              : !(prior && own < 0.0f);
-        if (!__all_sync(F, good) || thick == 0u) break;
-        if (fresh) {
-          pk.nu_lab = nu_c * r1;
-          pk.inv_nu = inv_c * Df;
-          fresh = false;
-        }
-        const float inv_nu = pk.inv_nu;
-        const double nu_cmf = pk.nu_lab * f64_of_f32(Df);
-        const float lj = f32_of_f64_max0(nu_cmf - __longlong_as_double(hit)) * inv_nu;
-        if (k == 0 && !inside_shell_f(pp, q, lj, inner, c_xi2, c_xo2)) break;
-        polls += 1u;
-        if (MODE == 2) {  // internal jumps, then the record of the level they end in
-          ds.d += 1u;
-          const LoneMaDraws md{&ds, &wd};
-          rinfo = macroatom_walk_lone(c.ma_row, c.ma_jump, static_cast<int32_t>(rinfo), md, lane);
-          u_em = md.next();
-          load_slot_here64(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
-          um = md.next();
-        } else {
-          ds.d += 3u;
-        }
-        pk.cnt[0] += 1u;
-        pk.cnt[1] += static_cast<uint32_t>(k) + 1u;
-        pk.cnt[2] += static_cast<uint32_t>(k) + 1u;
-        pk.cnt[3] += 1u;
-        if (JB && static_cast<int>(lane) <= k) {
-          const float e_jb = ((pk.e_lab * inv_nu) * c.nu_ref) * kEstFixScaleF;
-          red_add_evict_first(c.jb_fix + static_cast<size_t>(cs) * static_cast<size_t>(c.L) + w0 +
-                                  static_cast<int32_t>(lane),
-                              __float2ull_rn((f32_of_positive_f64(w_b) * inv_nu) * e_jb), jb_pol);
-        }
-        const float wgt = ((pk.e_lab * Df) * Df) * lj;
-        if (lane == n_log) {
-          g_w = wgt * kEstFixScaleF;
-          g_b = (wgt * (f32_of_positive_f64(__double_as_longlong(nu_cmf)) * c.inv_nu_ref)) * kEstFixScaleF;
-        }
-        ++n_log;
+        uint32_t di = ds.d - wd.base, n_ev = 0u, n_line = 0u;
+        uint32_t room = min(min(255u - (polls & 255u), cap - pk.cnt[0]), 32u - n_log);
+        if (MODE != 2) room = min(room, (kWarpDraws - di) / 3u);
+        if (room == 0u) break;
 #pragma unroll 1
-        while (n_log == 32u) {  // (a loop, and opaque: not evaluated for every segment)
-          asm volatile("" : "+f"(g_w), "+f"(g_b));
-          sum_log();
-        }
-        const float pl = pp + lj;
-        const float r2n = fmaf(pl, pl, q);
-        const float xn = sqrtf(r2n);
-        const float e_c = pk.e_lab * (1.0f - pl);
-        int32_t em = slot_line(ra, rc, u_em);
-        if (em < 0) em = search_row_lone(c.rec, rinfo, rc.z, u_em, lane);
-        w0 = em + 1;
-        reload();
-        nu_c = __longlong_as_double(static_cast<long long>(load_here(c.nu + em)));
-        inv_c = load_here_f(c.inv_nu32 + em);
-        // ... and while the window is on its way:
-        const float mu2 = static_cast<float>(static_cast<int32_t>(um >> 29) - (1 << 23)) * 0x1.0p-23f;
-        const float pn = xn * mu2;
-        const float D2 = 1.0f - pn;
-        const float iD2 = 1.0f / D2;
-        const double r0 = f64_of_f32(iD2);
-        r1 = fma(r0, fma(-f64_of_f32(D2), r0, 1.0), r0);
-        pk.p = pn;
-        pk.q = max0f(fmaf(-pn, pn, r2n));
-        pk.e_lab = e_c * iD2;
-        pk.inv_D = iD2;
-        pk.have_inv_D = true;
-        fresh = true;
+        do {
+          const float tau0 = -__logf(open0f(wd.u[di]));
+          unsigned long long u_em = wd.u[di + 1u], um = wd.u[di + 2u];
+          const float pp = pk.p, q = pk.q, Df = 1.0f - pp;
+          const bool inner = pp < 0.0f && q <= c_xi2;
+          const float lx = Df - (1.0f - shell_exit_f(q, inner, c_xi2, c_xo2));
+          ScanF f;
+          f.tf = c_kap * Df;
+          scan_frequency(f, nu_c, Df);
+          // (each lane the record index of its own line, while the scan runs)
+          const uint32_t my_slot = MODE == 1 ? bucket_index(w_r, u_em) : 0u;
+          const bool there = w0 + static_cast<int32_t>(lane) < c.L;
+          bool ok;
+          const float l = scan_delta(f, w_b, ok) * f.lf;
+          const float a = l * f.tf;
+          const float own = there ? w_t : 0.0f;
+          const float M = fmaf(0x1.0p-19f + 0x1.0p-18f, a + tau0, fmaf(f.tf, 0x1.0p-43f, 0x1.0p-100f));
+          const float left = tau0 - a;
+          const bool inside = lx - l > fmaf(0x1.0p-19f, l, 0x1.0p-43f);
+          const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
+          const int k = 31 - __clz(thick & (0u - thick));
+          const long long hit = __shfl_sync(F, w_b, k);
+          uint4 ra, rc;
+          if (MODE == 1) load_slot_here64(c.bucket + __shfl_sync(F, my_slot, k), ra, rc);
+          unsigned long long rinfo = __shfl_sync(F, w_r, k);
+          const bool prior = static_cast<int>(lane) < k;
+          const unsigned sum = __reduce_add_sync(
+              F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
+          const float rk = left - static_cast<float>(sum) * 0x1.0p-21f;
+          const bool good = static_cast<int>(lane) == k
+                                ? (f.ec > 0 && f.ec < 2047 && (inside || k == 0) && rk > M + 0x1.0p-15f)
+                                : !(prior && own < 0.0f);
+          certain = __all_sync(F, good) && thick != 0u;
+          if (!certain) break;
+          if (fresh) {
+            pk.nu_lab = nu_c * r1;
+            pk.inv_nu = inv_c * Df;
+            fresh = false;
+          }
+          const float inv_nu = pk.inv_nu;
+          const double nu_cmf = pk.nu_lab * f64_of_f32(Df);
+          const float lj = f32_of_f64_max0(nu_cmf - __longlong_as_double(hit)) * inv_nu;
+          certain = k != 0 || inside_shell_f(pp, q, lj, inner, c_xi2, c_xo2);
+          if (!certain) break;
+          if (MODE == 2) {  // internal jumps, then the record of the level they end in
+            ds.d = wd.base + di + 1u;
+            const LoneMaDraws md{&ds, &wd};
+            rinfo = macroatom_walk_lone(c.ma_row, c.ma_jump, static_cast<int32_t>(rinfo), md, lane);
+            u_em = md.next();
+            load_slot_here64(bucket_slot(c.bucket, rinfo, u_em), ra, rc);
+            um = md.next();
+            di = ds.d - wd.base;
+          } else {
+            di += 3u;
+          }
+          n_ev += 1u;
+          n_line += static_cast<uint32_t>(k);
+          if (JB && static_cast<int>(lane) <= k) {
+            const float e_jb = ((pk.e_lab * inv_nu) * c.nu_ref) * kEstFixScaleF;
+            red_add_evict_first(c.jb_fix + static_cast<size_t>(cs) * static_cast<size_t>(c.L) + w0 +
+                                    static_cast<int32_t>(lane),
+                                __float2ull_rn((f32_of_positive_f64(w_b) * inv_nu) * e_jb), jb_pol);
+          }
+          const float wgt = ((pk.e_lab * Df) * Df) * lj;
+          if (lane == n_log) {
+            g_w = wgt * kEstFixScaleF;
+            g_b = (wgt * (f32_of_positive_f64(__double_as_longlong(nu_cmf)) * c.inv_nu_ref)) * kEstFixScaleF;
+          }
+          ++n_log;
+          const float pl = pp + lj;
+          const float r2n = fmaf(pl, pl, q);
+          const float xn = sqrtf(r2n);
+          const float e_c = pk.e_lab * (1.0f - pl);
+          int32_t em = slot_line(ra, rc, u_em);
+          if (em < 0) em = search_row_lone(c.rec, rinfo, rc.z, u_em, lane);
+          w0 = em + 1;
+          reload();
+          nu_c = __longlong_as_double(static_cast<long long>(load_here(c.nu + em)));
+          inv_c = load_here_f(c.inv_nu32 + em);
+          // ... and while the window is on its way:
+          const float mu2 = static_cast<float>(static_cast<int32_t>(um >> 29) - (1 << 23)) * 0x1.0p-23f;
+          const float pn = xn * mu2;
+          const float D2 = 1.0f - pn;
+          const float iD2 = 1.0f / D2;
+          const double r0 = f64_of_f32(iD2);
+          r1 = fma(r0, fma(-f64_of_f32(D2), r0, 1.0), r0);
+          pk.p = pn;
+          pk.q = max0f(fmaf(-pn, pn, r2n));
+          pk.e_lab = e_c * iD2;
+          pk.inv_D = iD2;
+          pk.have_inv_D = true;
+          fresh = true;
+        } while (n_ev != room && (MODE != 2 || di + 3u <= kWarpDraws));
+        polls += n_ev;
+        pk.cnt[0] += n_ev;
+        pk.cnt[1] += n_line + n_ev;
+        pk.cnt[2] += n_line + n_ev;
+        pk.cnt[3] += n_ev;
+        ds.d = wd.base + di;
       }
       if (fresh) {
         pk.nu_lab = nu_c * r1;
