@@ -183,7 +183,7 @@ mc_status mc_batch_create(mc_model *const *models, uint32_t n_models, mc_batch *
     return bfail(nullptr, MC_ERR_CUDA, std::string("batch create: ") + cudaGetErrorString(e));
   }
   b->grid = b->nsm * resolved_bps(b);
-  // every warp of a grid with the lone walk (128 threads a block) hands over at
+  // every warp of a grid with the lone walk (blocks of 128 threads) hands over at
   // most kPoolLive - 1 walks, once
   b->pool_cap = static_cast<uint32_t>(b->nsm * b->max_bps[1] * 4) * (kPoolLive - 1u);
   e = cudaMallocAsync(&b->d_counters, counter_bytes(b), b->stream);

@@ -268,11 +268,12 @@ __device__ __forceinline__ PoolWalk pack_walk(const PacketM &pk, uint32_t d, int
 // model's results do not depend on the company it is launched in.  It is
 // compiled twice: MINB = 1 (blocks of 128 threads, three per SM at up to 168
 // registers, with lone walks) for single models and for batches of 128
-// threads a block, and MINB = 2 for batches of 64 or 256 threads (128
-// registers: 16 resident warps per SM, without lone walks).  A batch of 12
+// threads a block, and MINB = 2 for batches of 64 or 256 threads or of many
+// models (128 registers: 16 resident warps per SM, without lone walks).  A batch of 12
 // uneven models (2.9e6 packets): 330 ms a launch with the second (26 ms until
 // the queue is empty, then the longest walks at 2.5 us a segment), 209 ms with
-// the first (34 ms, and 1.3 us); of 40: 577 (156) and 430 (187).  The arithmetic
+// the first (34 ms, and 1.3 us), 185 since the lone loop takes fewer
+// instructions; of 40: 577 (156) and 430 (187), now 397.  The arithmetic
 // is the same instruction for instruction, lone walks included; the batch
 // tests check the bits.
 template <int MODE, bool JB, bool REC, int MINB>
@@ -546,8 +547,8 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
       // from exact arithmetic by the roundings of c_e and of its products, a few
       // 2^-24 of either side) or, for the first line against the exit, exactly as
       // below.  It leaves, with nothing changed, at a segment that is anything
-      // else or in doubt.  (Walk of
-      // 83,154 segments: 152 -> 105 ms.)
+      // else or in doubt.  (Walk of 83,154 segments alone: 152 -> 91 ms, and 87 with
+      // fewer instructions in the loop; 74 without J_blue.)
       const unsigned F = 0xffffffffu;
       const uint32_t cap = c.max_segments < 0xffffffffull ? static_cast<uint32_t>(c.max_segments) : 0xffffffffu;
       if (pk.shell != cs) {
@@ -1126,26 +1127,33 @@ size_t mixed_smem_bytes(int S) {
   return 4 * static_cast<size_t>(S) * sizeof(float) + (128 / 32) * kLoneWords * sizeof(unsigned long long);
 }
 
-// Batched launches of 128 threads a block take the build with the lone walk.
+// Batched launches of 128 threads a block take the build with the lone walk, up
+// to kLoneModels models.  Two batches on their own streams, model iterations/s
+// with it and without: 2 x 8 models 78 and 45, 2 x 16 91 and 63, 2 x 32 133 and
+// 111, 2 x 64 170 and 155, 2 x 128 188 and 189 (256 models, ten iterations with
+// updates: 18.7 and 19.7 models/s): there one batch's queue fills the other's tail.
 namespace {
-const void *batch_kernel(int line_mode, bool jb, bool rec, int block) {
-  return block == 128 ? select_m<1>(line_mode, jb, rec) : select_b(line_mode, jb, rec);
+constexpr int kLoneModels = 96;
+bool lone_batch(int n_models, int block) { return block == 128 && n_models <= kLoneModels; }
+const void *batch_kernel(int line_mode, bool jb, bool rec, int n_models, int block) {
+  return lone_batch(n_models, block) ? select_m<1>(line_mode, jb, rec) : select_b(line_mode, jb, rec);
 }
 size_t batch_smem_bytes(int n_models, int block) {
-  return (static_cast<size_t>(n_models) + 1 + (block == 128 ? 4 * kLoneWords : 0)) * sizeof(unsigned long long);
+  return (static_cast<size_t>(n_models) + 1 + (lone_batch(n_models, block) ? 4 * kLoneWords : 0)) *
+         sizeof(unsigned long long);
 }
 }  // namespace
 
 cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, int block,
                             int *blocks_per_sm) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, batch_kernel(line_mode, j_blue, record, block), block, batch_smem_bytes(n_models, block));
+      blocks_per_sm, batch_kernel(line_mode, j_blue, record, n_models, block), block, batch_smem_bytes(n_models, block));
 }
 
 cudaError_t launch_transport_batch(const TransportParams &p, int line_mode, bool j_blue, bool record,
                                    int grid, int block, cudaStream_t st) {
   void *args[] = {const_cast<TransportParams *>(&p)};
-  return cudaLaunchKernel(batch_kernel(line_mode, j_blue, record, block), dim3(grid), dim3(block), args,
+  return cudaLaunchKernel(batch_kernel(line_mode, j_blue, record, p.n_models, block), dim3(grid), dim3(block), args,
                           batch_smem_bytes(p.n_models, block), st);
 }
 

@@ -11,8 +11,8 @@ model), transports the packets and updates T_R and W (Sect. 2.8).  With
 transported (the draws of a packet depend only on its id), e.g. a single long
 random walk.  With --batched M: the first M models of the batched workload
 (generation seed 1401), mixed precision, one batched launch per iteration
-with a fixed shape (128 threads per block, 4 resident blocks per SM, largest
-models first).  Prints one JSON line of totals and kernel times per
+with a fixed shape (128 threads per block, up to 4 resident blocks per SM,
+largest models first).  Prints one JSON line of totals and kernel times per
 iteration.  Used for profiling captures.
 """
 from __future__ import annotations
