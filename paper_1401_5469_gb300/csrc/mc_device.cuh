@@ -360,7 +360,7 @@ __device__ __forceinline__ void load_slot_here(const DbrSlot *slot, uint4 &a, ui
   c = load_here4(reinterpret_cast<const uint4 *>(slot) + 1);
 }
 
-// The same in four 64-bit loads: the mixed kernel's lone walk takes 91 ms with
+// The same in four 64-bit loads: the mixed kernel's lone walk took 91 ms with
 // them instead of 102 (the binary64 kernel's 105 instead of 100).
 __device__ __forceinline__ void load_slot_here64(const DbrSlot *slot, uint4 &a, uint4 &c) {
   const unsigned long long *w = reinterpret_cast<const unsigned long long *>(slot);

@@ -76,8 +76,10 @@ struct PoolWalk {
 // pool 163, 40.9, 9.9; with 4 and 128 113, 34.6, 7.1; 8 and 512 121, 34.0, 7.4;
 // 4 and 512 114, 33.9, 7.5.  Mixed 177, 45.7, 11.0 -> 132, 34.8, 8.5.  The age
 // keeps short walks (scatter lists: under 100 segments) where they are: handed
-// over at any age, 1e5 of them took 4.1 instead of 1.1 ms.
-constexpr unsigned kPoolLive = 4;
+// over at any age, 1e5 of them took 4.1 instead of 1.1 ms.  3 in place of 4
+// keeps the pool, which every model has, at 0.48 MB instead of 0.72 (105 and 105 ms,
+// 25.5 and 26.6, 6.4 and 6.4; mixed 115 and 116 ms, 29.3 and 30.4, 7.6 and 7.6).
+constexpr unsigned kPoolLive = 3;
 constexpr uint32_t kPoolAge = 128;
 
 // Copies of the J and nu_bar sums, the blocks spread over them: a shell's sums

@@ -22,11 +22,12 @@
 //    registers and are flushed once per shell change;
 //  * a warp down to its last live walk runs it with all 32 lanes (the lone
 //    walk), and few packets are spread over all warps.
-// Longest walk of the 500,000-line model (94,495 segments) alone: 212 ms with a
-// binary64 scan, 165 ms with the scan in binary32, 107 ms with the lone walk's
-// line-event loop (2.25 -> 1.13 us a segment; bound by its binary64 chain, 14
-// instructions of 64 cycles, beside two dependent L2 loads of ~400 cycles);
-// its 1e6-packet iteration 236 -> 155 ms (queue 9.9 -> 5.9 ms).
+// Longest walk of the 500,000-line model (94,495 segments) alone, with J_blue: 212
+// ms with a binary64 scan, 165 ms with the scan in binary32, 107 ms with the lone
+// walk's line-event loop, 96 ms with reciprocal and square root on the integer
+// pipe, 90 ms with fewer instructions in that loop (2.25 -> 0.95 us a segment,
+// 0.81 without J_blue; bound by the instructions of one warp, see there); its
+// 1e6-packet iteration 236 -> 105 ms (queue 9.9 -> 6.2 ms).
 #pragma once
 
 #include <cstdint>
@@ -659,14 +660,14 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
       // oldest to the pool -- walk lengths are heavy-tailed, so that the oldest is
       // expected to be the longest -- and runs that one with all 32 lanes to its
       // end, then takes others from the pool.  A walk that shares its warp
-      // advances at 4 to 8 us a segment, a lone one at 1.1 (1.7 with all warps of
-      // the SM in this mode).
+      // advances at 4 to 8 us a segment, a lone one at 0.8 to 0.95 (1.5 with all
+      // warps of the SM in this mode).
       // All 32 lanes hold the walk's state; the line list comes 32 lines at a
       // time (line w0 + lane in each lane, one coalesced load), the scan of such a
       // window in one step, the draws computed ahead; lane 0 makes the walk's side
-      // effects.  The chain of a line event is then two dependent loads (the
-      // emission record, the window behind the emitted line) and the scan; the
-      // event's binary64 arithmetic runs while they are in flight.
+      // effects.  The loads of a line event are then two dependent ones (the
+      // emission record, the window behind the emitted line); the event's binary64
+      // arithmetic runs while they are in flight.
       const unsigned F = 0xffffffffu;
       if (acc_s >= 0) {
         atomicAdd(j_sum + acc_s, acc_j);
