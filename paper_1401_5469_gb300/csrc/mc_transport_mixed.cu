@@ -635,8 +635,11 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
           const unsigned sum = __reduce_add_sync(
               F, prior ? __float2uint_rd(fminf(fmaxf(own, 0.0f), 63.0f) * 0x1.0p21f) : 0u);
           const float rk = left - static_cast<float>(sum) * 0x1.0p-21f;
+          // (a line at or behind the packet, up to 2^-24 of the frequency after a
+          // scattering or a crossing, has l = 0 here and a depth below 0 before it)
           const bool good = static_cast<int>(lane) == k
-                                ? (f.ec > 0 && f.ec < 2047 && (inside || k == 0) && rk > M + 0x1.0p-15f)
+                                ? (f.ec > 0 && f.ec < 2047 && (inside || k == 0) && l > 0.0f &&
+                                   rk > M + 0x1.0p-15f)
                                 : !(prior && own < 0.0f);
           certain = __all_sync(F, good) && thick != 0u;
           if (!certain) break;
