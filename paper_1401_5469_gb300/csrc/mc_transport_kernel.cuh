@@ -219,7 +219,8 @@ __device__ __forceinline__ int spectrum_bin(const TransportParams &p, double nu_
 // each: a random walk then does not wait for its own v-packets on one lane (and
 // a lone walk's 32 lanes have work of their own).  Each lane loads four lines
 // ahead, and sums depths in fixed point (units of 2^-52), which takes no
-// binary64 instruction for a line.
+// binary64 instruction for a line; a sum that reaches 512 moves to a binary64 one
+// (a depth is not bounded, and negative ones may bring a sum back).
 
 struct VirtualLaunch {
   double x, r2, nu_cmf, e_cmf;  // radius (units of c t_exp), its square, comoving nu and E
@@ -234,8 +235,7 @@ __device__ __forceinline__ double vdraw_open0(const TransportParams &p, uint32_t
   return __ull2double_rn(u + 1ull) * 0x1.0p-53;
 }
 
-// A depth in units of 2^-52, rounded to nearest; 1024 at most in magnitude
-// (e^-1024 is 0).
+// A depth in units of 2^-52, rounded to nearest; 1024 (2^62) at most in magnitude.
 __device__ __forceinline__ long long depth_fix(double t) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(t));
   const int e = static_cast<int>((b >> 52) & 0x7ffull) - 1023;
@@ -254,7 +254,11 @@ __device__ __noinline__ void fly_virtual(const TransportParams &p, const double 
   const double *s_xi2 = sh, *s_xo2 = sh + S, *s_kap = sh + 4 * S;
   const long long *nub = reinterpret_cast<const long long *>(p.nu);
   const bool cut = rawkey(p.tau_v_max) > 0;
-  const long long cap = cut ? depth_fix(p.tau_v_max) : 1ll << 62;
+  auto cut_left = [&](double t) {
+    const long long v = depth_fix(t);
+    return cut && v < 1ll << 62 ? v : 0x7fffffffffffffffll;
+  };
+  auto in_range = [](long long v) { return static_cast<unsigned long long>(v + (1ll << 61)) < 1ull << 62; };
   __syncwarp();
   for (unsigned t = lane; t < count * nv; t += 32u) {
     const unsigned k = t / nv, i = t - k * nv;
@@ -268,7 +272,15 @@ __device__ __noinline__ void fly_virtual(const TransportParams &p, const double 
     const double inv_nv = rcp64(static_cast<double>(p.n_virtual));
     const double e_v = (v.shell < 0 ? v.e_cmf * (2.0 * mu_v) : v.e_cmf * (0.5 * (1.0 - mu_min))) * inv_nv;
     const double nu_lab = v.nu_cmf * iD;
-    long long tau = 0;
+    // the depth so far: deep + tau 2^-52, |tau| < 2^61 (512) unless over the cut;
+    // cap: what the cut leaves for tau (nothing exceeds the largest integer)
+    long long tau = 0, cap = cut_left(p.tau_v_max);
+    double deep = 0.0;
+    auto add_deep = [&](double t) {
+      deep += t + static_cast<double>(tau) * 0x1.0p-52;
+      tau = 0;
+      cap = cut_left(p.tau_v_max - deep);
+    };
     int32_t s = v.shell < 0 ? 0 : v.shell, j = v.next_line;
     for (;;) {
       const double xi2 = s_xi2[s], xo2 = s_xo2[s];
@@ -287,16 +299,35 @@ __device__ __noinline__ void fly_virtual(const TransportParams &p, const double 
           b[c] = __ldg(nub + jj);
           d[c] = __ldg(tau_s + jj);
         }
+        bool wide = false;  // line j's depth leaves tau's range
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          in = in && j < L && b[c] > key_exit && tau <= cap;
+          in = in && j < L && b[c] > key_exit;
           if (in) {
-            tau += depth_fix(d[c]);
-            ++j;
+            const long long sum = tau + depth_fix(d[c]);
+            in = sum <= cap;
+            wide = in && !in_range(sum);
+            if (wide) {
+              in = false;
+            } else {
+              tau = sum;
+              ++j;
+            }
           }
         }
+        if (wide) {
+          add_deep(__ldg(tau_s + j));
+          ++j;
+          in = tau <= cap;
+        }
       }
-      tau += depth_fix((s_kap[s] * (1.0 - pc)) * max0(p_exit - pc));
+      if (tau > cap) break;
+      {
+        const double t = (s_kap[s] * (1.0 - pc)) * max0(p_exit - pc);
+        const long long sum = tau + depth_fix(t);
+        if (sum <= cap && !in_range(sum)) add_deep(t);
+        else tau = sum;
+      }
       pc = p_exit;
       s += inner ? -1 : 1;
       // over the cut; out; or met the inner boundary (only by rounding)
@@ -304,7 +335,7 @@ __device__ __noinline__ void fly_virtual(const TransportParams &p, const double 
     }
     if (s >= S && tau <= cap)
       atomicAdd(p.spectrum_v + spectrum_bin(p, nu_lab),
-                (e_v * iD) * exp(-(static_cast<double>(tau) * 0x1.0p-52)));
+                (e_v * iD) * exp(-(deep + static_cast<double>(tau) * 0x1.0p-52)));
   }
   __syncwarp();
 }
