@@ -494,7 +494,9 @@ typedef struct {
     const double *nu;                     /* [L] device, strictly descending */
     const double *tau;                    /* [S*L] device, shell-major Sobolev depths */
     int32_t line_mode;                    /* MC_LINE_SCATTER or MC_LINE_DOWNBRANCH */
-    const int32_t *line_row;              /* [L] device: ion*n_levels + upper (downbranch) */
+    const int32_t *line_row;              /* [L] device: ion*n_levels + upper (downbranch);
+                                             read of any line, looked up in dbr_offset only
+                                             where the line's depth is positive */
     const uint32_t *dbr_offset, *dbr_line;/* device branching table (downbranch) */
     const double *dbr_cdf;
     uint64_t seed;

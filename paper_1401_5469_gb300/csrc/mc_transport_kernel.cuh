@@ -875,14 +875,15 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
               const float M = fmaf(0x1.0p-19f + 0x1.0p-18f, a + f.tau, fmaf(f.tf, 0x1.0p-43f, 0x1.0p-100f));
               const float left = f.tau - a;
               const bool inside = f.lx - l > fmaf(0x1.0p-19f, l, f.mx);
-              const unsigned thick = __ballot_sync(F, there && ok && left - own < -M);
+              // (a line of the caller's table that cannot absorb need not have a row)
+              const unsigned thick = __ballot_sync(F, there && ok && left - own < -M && (LINES != 3 || own > 0.0f));
               const int k = 31 - __clz(thick & (0u - thick));
               const long long hit = __shfl_sync(F, w_b, k);
               uint4 ra, rc;
               uint32_t row_lo = 0u, row_hi = 0u;
               if (LINES == 1) load_slot_here(p.dbr_bucket + __shfl_sync(F, my_slot, k), ra, rc);
               unsigned long long rinfo = __shfl_sync(F, w_r, k);
-              if (LINES == 3) {
+              if (LINES == 3 && thick != 0u) {
                 row_lo = load_here32(p.dbr_offset + rinfo);
                 row_hi = load_here32(p.dbr_offset + rinfo + 1);
               }
