@@ -74,13 +74,18 @@ struct PoolWalk {
 // from which warps that have nothing left take them.  Measured (ms a launch;
 // binary64 500k lines and 1e6 packets, 50k and 1e5, 20k and 2e4): without the
 // pool 163, 40.9, 9.9; with 4 and 128 113, 34.6, 7.1; 8 and 512 121, 34.0, 7.4;
-// 4 and 512 114, 33.9, 7.5.  Mixed 177, 45.7, 11.0 -> 132, 34.8, 8.5.  The age
-// keeps short walks (scatter lists: under 100 segments) where they are: handed
-// over at any age, 1e5 of them took 4.1 instead of 1.1 ms.  3 in place of 4
-// keeps the pool, which every model has, at 0.48 MB instead of 0.72 (105 and 105 ms,
-// 25.5 and 26.6, 6.4 and 6.4; mixed 115 and 116 ms, 29.3 and 30.4, 7.6 and 7.6).
+// 4 and 512 114, 33.9, 7.5.  Mixed 177, 45.7, 11.0 -> 132, 34.8, 8.5.  3 in place of 4
+// keeps the pool at 0.48 MB instead of 0.72 (105 and 105 ms, 25.5 and 26.6, 6.4 and
+// 6.4; mixed 115 and 116 ms, 29.3 and 30.4, 7.6 and 7.6).
+// The age keeps walks that end soon where they are: with no warp idle, three of
+// them one after the other take longer than side by side.  Ages 128, 384 and 512:
+// 1e5 walks cut at 300 segments, mixed 2.86, 1.62 and 1.60 ms (without the pool
+// 1.64), binary64 2.53, 1.50 and 1.50 (1.49); 5000 lines, 5 shells and 1e6 packets,
+// mixed 7.5, 6.2 and 6.2 (6.4); 20,000 scattering lines, 2e5 packets, mixed 5.07, 4.36
+// and 4.37 (4.32), binary64 4.66, 3.93 and 4.12 (4.45); the long walks gain the same: 5e4
+// lines and 1e5 packets 31.6, 32.3 and 32.3 (48.0), 2e4 and 2e4 5.74, 5.87 and 6.05 (8.6).
 constexpr unsigned kPoolLive = 3;
-constexpr uint32_t kPoolAge = 128;
+constexpr uint32_t kPoolAge = 384;
 
 // Copies of the J and nu_bar sums, the blocks spread over them: a shell's sums
 // are two addresses that every packet crossing it adds to.  1e4 packets of the

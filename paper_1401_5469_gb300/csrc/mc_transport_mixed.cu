@@ -39,6 +39,11 @@ namespace {
 // single-model launches take 128 threads per block, batched ones 64, 128 or 256
 constexpr int kMaxBlock = 256;
 constexpr size_t kLoneWords = sizeof(PoolWalk) / sizeof(unsigned long long) + kWarpDraws;
+// A lone walk tries its line-event loop within so many segments of its last line
+// event: every try scans the window once more where it is not one.  50,000
+// packets through 400 shells, one segment in eight a line event: 39.0 -> 33.3 ms;
+// trapped walks as before.
+constexpr int kLoopTries = 3;
 constexpr int kLineEvent = 1, kElectronEvent = 2, kShellEvent = 3;
 
 struct PacketM {
@@ -323,6 +328,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
   wd.init(!kLoneBuild ? nullptr : warp_mem + sizeof(PoolWalk) / sizeof(unsigned long long));
   bool drained = false;  // warp-uniform: the packet queue is empty
   bool lone = false;
+  int tries = 0;
   int32_t lwin_j0 = 0, lwin_s = -1;
   long long lwin_b = 0;
   float lwin_t = 0.0f;
@@ -500,6 +506,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
           lwin_s = -1;
           alive = true;
           lone = true;
+          tries = kLoopTries;
           wd.pid = kNoPacket;
           wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
         }
@@ -537,7 +544,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
       r = __shfl_sync(0xffffffffu, lwin_r, idx);
     };
 
-    if (kLoneBuild && MODE >= 1 && lone && pk.next_line < c.L) {
+    if (kLoneBuild && MODE >= 1 && lone && tries > 0 && pk.next_line < c.L) {
       // Line event after line event of a lone walk, the bulk of a trapped walk,
       // in a loop of its own (the binary64 kernel's: loads stay in their
       // registers from where they are issued to where they are used).  The
@@ -965,6 +972,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
       acc_nb += __float2ull_rn((wgt * (f32_of_positive_f64(__double_as_longlong(nu_cmf)) * c.inv_nu_ref)) *
                                kEstFixScaleF);
       pk.next_line = j;
+      if (MODE >= 1) tries = kind == kLineEvent ? kLoopTries : tries - 1;
       if (kind == kShellEvent) {
         pk.cnt[5] += 1u;
         const int32_t ns = inner ? s - 1 : s + 1;
