@@ -166,7 +166,8 @@ typedef struct {
     uint64_t max_packets;       /* largest n_packets of any run (sizes packet records) */
     uint64_t max_segments;      /* per-packet segment cap; 0 = 1e6 */
     double delta_t;             /* simulated time interval of Eq. 10, s; 0 = 1 s */
-    uint64_t timeout_ns;        /* transport-kernel deadline; 0 = none */
+    uint64_t timeout_ns;        /* transport-kernel deadline, looked at every segment, by a
+                                   walk alone in its warp every 256 segments (0.3 ms); 0 = none */
 } mc_run_desc;
 
 /* Optional device allocator (e.g. a framework's caching allocator).  alloc

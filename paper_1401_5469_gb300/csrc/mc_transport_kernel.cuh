@@ -844,12 +844,12 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
           // 4 to 5 cycles (fixed-latency stalls 3.1 of the 5.9 cycles between issues,
           // waits for loads 0.6), 416 of them a segment before these steps.  So the
           // segments it may take are counted out beforehand (to the next look at the
-          // stop word, the cap, 32 logged, three draws each), its counters are two, a
+          // clock and the stop word, the cap, 32 logged, three draws each), its counters are two, a
           // segment's estimator terms are two shared stores, and the J_blue terms of
           // the lines passed one atomic of the lanes.  A walk of 94,495 segments alone:
           // 100.4 -> 76.7 ms, with J_blue (and its zeroing, which leaves the caches
           // cold) 96.0 -> 89.8; 5e4 lines, 1e5 packets: 32.6 -> 25.5 ms.
-          bool certain = !p.timeout_ns;
+          bool certain = true;
           while (certain) {
             if (n_log == 32u) sum_log();
             ld.keep(d, pk.pid, p.iteration, p.key0, p.key1, lane, false);

@@ -602,9 +602,9 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         n_log = 0u;
       };
       // (The segments of the inner loop are counted out beforehand, as in the
-      // binary64 kernel: to the next look at the stop word, the cap, 32 logged,
-      // three draws each.)
-      bool certain = !p.timeout_ns;
+      // binary64 kernel: to the next look at the clock and the stop word, the cap, 32
+      // logged, three draws each.)
+      bool certain = true;
       while (certain) {
         if (n_log == 32u) sum_log();
         wd.keep_u(ds, c.key0, c.key1, c.iteration, lane);
