@@ -549,7 +549,10 @@ mc_status mc_model_create(const mc_geometry_desc *geom, const mc_line_desc *line
   // the pool: every warp of the grid hands over at most kPoolLive - 1 walks, once
   m->pool_cap = static_cast<uint32_t>(m->grid) * static_cast<uint32_t>(transport_block_size() / 32) * (kPoolLive - 1u);
   m->n_counter_words = kNCounterSlots + 2 + (static_cast<size_t>(m->pool_cap) + 1) / 2;
-  if (!alloc_n(m, &m->counters, m->n_counter_words) || !alloc_n(m, &m->pool, m->pool_cap))
+  // (a mixed-precision model's own is allocated by its first run by itself: batches
+  // have one of theirs)
+  if (!alloc_n(m, &m->counters, m->n_counter_words) ||
+      (run->precision != MC_PRECISION_MIXED && !alloc_n(m, &m->pool, m->pool_cap)))
     return bail(MC_ERR_OOM, "device allocation failed");
   e = cudaStreamSynchronize(m->stream);
   if (e != cudaSuccess) return bail(MC_ERR_CUDA, std::string("create: ") + cudaGetErrorString(e));
@@ -626,6 +629,7 @@ mc_status mc_run_iteration_range(mc_model *m, uint64_t seed, uint32_t iteration,
   if (!(t_inner > 0.0) || !std::isfinite(t_inner)) return fail(m, MC_ERR_INVALID_ARG, "t_inner must be positive");
   if (m->in_batch) return fail(m, MC_ERR_INVALID_ARG, "the model belongs to a batch; run it through the batch");
   m->spread = n_packets >= kSpreadPackets;
+  if (!m->pool) alloc_n(m, &m->pool, m->pool_cap);  // (without one walks stay in their warps)
   mc_status st = model_prepare(m, m->stream, true);
   if (st != MC_OK) return st;
   TransportParams p{};

@@ -57,7 +57,9 @@ def model_footprint_bytes(spec, j_blue: Optional[bool] = None,
     b += nnz * (4 + 4 + 8 + 16 + 32)   # branching table, its search entries and bucket slots
     b += 4 * L if precision == mc.MC_PRECISION_MIXED else 0  # 1 / nu in binary32
     b += 16 * min(64 * S, 4096)        # copies of the J and nu_bar sums
-    b += 152 * 12 * 2 * (128 + 4)      # walks handed between warps (12 warps an SM, 2 walks each)
+    # walks handed between warps: 152 SMs, 12 warps (every build of the kernels takes 160 or
+    # 168 registers), 2 walks each; a model's own, or in a batch the share of the batch's
+    b += 152 * 12 * 2 * (128 + 4)
     if spec.n_ions:
         b += spec.n_ions * spec.n_levels * (8 + 8 + 1) + S * spec.n_ions * (8 + 8 * spec.n_levels)
     if getattr(spec, "ma_jump_p", None) is not None:  # macro-atom level and jump tables
