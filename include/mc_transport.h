@@ -536,8 +536,9 @@ mc_status mc_transport_noalloc(const mc_noalloc_args *args, void *stream);
  *        ref = sqrt(x) (IEEE, correctly rounded)
  *   fn = MC_MATH_APPROX: in = double x[n] > 0 (normal); ours = 1 - x y^2 with
  *        y = rsqrt.approx.ftz.f64(x), ref = 1 - x r with r = rcp.approx.ftz.f64(x)
- *        (each by one fma after the product x y): the residuals that the
- *        square root's and the reciprocal's corrections assume small
+ *        (each by one fma after the product x y): the residuals of the two
+ *        binary64 approximations, which no transport kernel uses any more (the
+ *        binary32 ones, which they do, show in MC_MATH_RCP and MC_MATH_SQRT)
  *
  * `in`, `ours` and `ref` are HOST arrays of n elements (0 < n <= 2^28); the
  * call allocates device memory, runs synchronously and frees it (a test

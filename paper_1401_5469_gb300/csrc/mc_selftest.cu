@@ -1,9 +1,9 @@
 // mc_selftest_math: evaluates the device arithmetic that the transport
 // kernels use in place of CUDA's functions (the table-driven logarithms and
-// the Newton reciprocal and square root of mc_device.cuh) side by side with
-// CUDA's own log, IEEE division and IEEE square root, and the residuals of
-// the hardware approximations those start from, on inputs the caller
-// chooses.  A diagnostic for accuracy tests; not on the transport path.
+// the reciprocal and square root of mc_device.cuh) side by side with CUDA's own
+// log, IEEE division and IEEE square root, and the residuals of the binary64
+// hardware approximations (which no kernel starts from any more: the
+// reciprocal and the root take the binary32 ones), on inputs the caller chooses.  A diagnostic for accuracy tests; not on the transport path.
 #include <cstdint>
 #include <string>
 
