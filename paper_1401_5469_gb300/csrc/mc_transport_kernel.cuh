@@ -263,7 +263,8 @@ __device__ __noinline__ void fly_virtual(const TransportParams &p, const double 
   for (unsigned t = lane; t < count * nv; t += 32u) {
     const unsigned k = t / nv, i = t - k * nv;
     const VirtualLaunch v = queue[k];
-    const double ri = sh[2 * S] * rcp64(v.x);  // x_in[0] / x
+    // x_in[0] / x with its remainder: 1 where x is x_in[0], and 1 - ri^2 loses nothing
+    const double ix = rcp64(v.x), r0 = sh[2 * S] * ix, ri = fma(fma(-r0, v.x, sh[2 * S]), ix, r0);
     const double mu_min = -sqrt64(max0(fma(-ri, ri, 1.0)));
     const double mu_v = fma(1.0 - mu_min, vdraw_open0(p, v.pid, v.first_draw + i), mu_min);
     double pc = v.x * mu_v;
