@@ -36,7 +36,8 @@ struct mc_batch {
   TransportParams *d_params = nullptr, *h_params = nullptr;  // device table, pinned host staging
   unsigned long long *d_prefix = nullptr, *h_prefix = nullptr;
   unsigned long long *d_counters = nullptr;  // work counter, flags (kNCounterSlots), then the pool's words
-  PoolWalk *d_pool = nullptr;      // [pool_cap] walks handed between warps
+  bool lone = false;               // blocks of 128 threads run lone walks
+  PoolWalk *d_pool = nullptr;      // [pool_cap] walks handed between warps (lone)
   uint32_t pool_cap = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -107,7 +108,7 @@ mc_status enqueue_iteration(mc_batch *b, int update, bool capturing) {
   p.pool_ctl = b->d_counters + kNCounterSlots;
   p.pool_ready = reinterpret_cast<uint32_t *>(b->d_counters + kNCounterSlots + 2);
   e = cudaEventRecordWithFlags(b->t0, b->stream, ev_flags);
-  if (e == cudaSuccess) e = launch_transport_batch(p, b->line_mode, b->j_blue, b->record, b->grid,
+  if (e == cudaSuccess) e = launch_transport_batch(p, b->line_mode, b->j_blue, b->record, b->lone, b->grid,
                                                     static_cast<int>(b->block), b->stream);
   if (e == cudaSuccess) e = cudaEventRecordWithFlags(b->t1, b->stream, ev_flags);
   if (e != cudaSuccess) return bcuda(b, e, "batched transport");
@@ -155,6 +156,9 @@ mc_status mc_batch_create(mc_model *const *models, uint32_t n_models, mc_batch *
   b->line_mode = m0->run.line_mode;
   b->j_blue = m0->j_blue != nullptr;
   b->record = m0->run.record_packets != 0;
+  uint32_t most_lines = 0;
+  for (uint32_t i = 0; i < n_models; ++i) most_lines = std::max(most_lines, models[i]->L);
+  b->lone = batch_lone(static_cast<int>(n_models), most_lines);
   b->order.resize(n_models);
   std::iota(b->order.begin(), b->order.end(), 0u);
   for (uint32_t i = 0; i < n_models; ++i) b->models.push_back(models[i]);
@@ -175,7 +179,7 @@ mc_status mc_batch_create(mc_model *const *models, uint32_t n_models, mc_batch *
   if (e == cudaSuccess) e = cudaEventCreate(&b->t1);
   const int blocks[3] = {64, 128, 256};
   for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-    e = batch_occupancy(b->line_mode, b->j_blue, b->record, static_cast<int>(n_models), blocks[k],
+    e = batch_occupancy(b->line_mode, b->j_blue, b->record, static_cast<int>(n_models), b->lone, blocks[k],
                         &b->max_bps[k]);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, m0->device);
   if (e != cudaSuccess || b->max_bps[0] <= 0 || b->max_bps[1] <= 0 || b->max_bps[2] <= 0) {
@@ -185,9 +189,9 @@ mc_status mc_batch_create(mc_model *const *models, uint32_t n_models, mc_batch *
   b->grid = b->nsm * resolved_bps(b);
   // every warp of a grid with the lone walk (blocks of 128 threads) hands over at
   // most kPoolLive - 1 walks, once
-  b->pool_cap = static_cast<uint32_t>(b->nsm * b->max_bps[1] * 4) * (kPoolLive - 1u);
+  if (b->lone) b->pool_cap = static_cast<uint32_t>(b->nsm * b->max_bps[1] * 4) * (kPoolLive - 1u);
   e = cudaMallocAsync(&b->d_counters, counter_bytes(b), b->stream);
-  if (e == cudaSuccess) e = cudaMallocAsync(&b->d_pool, b->pool_cap * sizeof(PoolWalk), b->stream);
+  if (e == cudaSuccess && b->lone) e = cudaMallocAsync(&b->d_pool, b->pool_cap * sizeof(PoolWalk), b->stream);
   if (e != cudaSuccess) {
     mc_batch_destroy(b);
     return bfail(nullptr, MC_ERR_CUDA, std::string("batch create: ") + cudaGetErrorString(e));

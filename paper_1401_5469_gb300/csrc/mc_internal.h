@@ -221,10 +221,12 @@ cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool 
                                 int *blocks_per_sm);
 const void *select_mixed_kernel(int line_mode, bool j_blue, bool record);
 const void *select_virtual_kernel(int line_mode, bool j_blue, bool record);  // binary64, with v-packets
-// Batched launches: `block` threads per block (64, 128 or 256).
-cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, int block,
+// Batched launches: `block` threads per block (64, 128 or 256); lone: with 128,
+// the build with lone walks and the pool (batch_lone: worth it for such a batch).
+bool batch_lone(int n_models, uint32_t most_lines);
+cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, bool lone, int block,
                             int *blocks_per_sm);
-cudaError_t launch_transport_batch(const TransportParams &p, int line_mode, bool j_blue, bool record,
+cudaError_t launch_transport_batch(const TransportParams &p, int line_mode, bool j_blue, bool record, bool lone,
                                    int grid, int block, cudaStream_t st);
 size_t mixed_smem_bytes(int S);
 cudaError_t launch_to_f32(const double *in, float *out, size_t n, cudaStream_t st);

@@ -273,8 +273,8 @@ __device__ __forceinline__ PoolWalk pack_walk(const PacketM &pk, uint32_t d, int
 // model's results do not depend on the company it is launched in.  It is
 // compiled twice: MINB = 1 (blocks of 128 threads, three per SM at up to 168
 // registers, with lone walks) for single models and for batches of 128
-// threads a block, and MINB = 2 for batches of 64 or 256 threads or of many
-// models (128 registers: 16 resident warps per SM, without lone walks).  A batch of 12
+// threads a block, and MINB = 2 for batches of 64 or 256 threads, of many models
+// or of short line lists (128 registers: 16 resident warps per SM, without lone walks).  A batch of 12
 // uneven models (2.9e6 packets): 330 ms a launch with the second (26 ms until
 // the queue is empty, then the longest walks at 2.5 us a segment), 209 ms with
 // the first (34 ms, and 1.3 us), 185 since the lone loop takes fewer
@@ -1138,34 +1138,42 @@ size_t mixed_smem_bytes(int S) {
   return 4 * static_cast<size_t>(S) * sizeof(float) + (128 / 32) * kLoneWords * sizeof(unsigned long long);
 }
 
-// Batched launches of 128 threads a block take the build with the lone walk, up
-// to kLoneModels models.  Two batches on their own streams, model iterations/s
+// Whether a batch's launches of 128 threads a block take the build with the lone
+// walk.  Up to kLoneModels models:  Two batches on their own streams, model iterations/s
 // with it and without: 2 x 8 models 78 and 45, 2 x 16 91 and 63, 2 x 32 133 and
 // 111, 2 x 64 170 and 155, 2 x 128 188 and 189 (256 models, ten iterations with
 // updates: 18.7 and 19.7 models/s): there one batch's queue fills the other's tail.
-namespace {
-constexpr int kLoneModels = 96;
-bool lone_batch(int n_models, int block) { return block == 128 && n_models <= kLoneModels; }
-const void *batch_kernel(int line_mode, bool jb, bool rec, int n_models, int block) {
-  return lone_batch(n_models, block) ? select_m<1>(line_mode, jb, rec) : select_b(line_mode, jb, rec);
+// And only where a model's line list is long, for walks to be trapped in: 8 models
+// of 1e5 packets, ms with it and without: 3000 lines 4.90 and 4.01, 6000 7.67 and 6.59,
+// 12,000 14.5 and 14.4, 25,000 31.0 and 37.8, 50,000 63 and 82; of 3000 packets 1.03 and 0.91,
+// 2.10 and 1.74, 5.2 and 6.4, 11.9 and 19.4, 15.6 and 31.3.
+constexpr int kLoneModels = 96, kLoneLines = 10'000;
+bool batch_lone(int n_models, uint32_t most_lines) {
+  return n_models <= kLoneModels && most_lines >= static_cast<uint32_t>(kLoneLines);
 }
-size_t batch_smem_bytes(int n_models, int block) {
-  return (static_cast<size_t>(n_models) + 1 + (lone_batch(n_models, block) ? 4 * kLoneWords : 0)) *
+
+namespace {
+const void *batch_kernel(int line_mode, bool jb, bool rec, bool lone, int block) {
+  return lone && block == 128 ? select_m<1>(line_mode, jb, rec) : select_b(line_mode, jb, rec);
+}
+size_t batch_smem_bytes(int n_models, bool lone, int block) {
+  return (static_cast<size_t>(n_models) + 1 + (lone && block == 128 ? 4 * kLoneWords : 0)) *
          sizeof(unsigned long long);
 }
 }  // namespace
 
-cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, int block,
+cudaError_t batch_occupancy(int line_mode, bool j_blue, bool record, int n_models, bool lone, int block,
                             int *blocks_per_sm) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, batch_kernel(line_mode, j_blue, record, n_models, block), block, batch_smem_bytes(n_models, block));
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm,
+                                                       batch_kernel(line_mode, j_blue, record, lone, block), block,
+                                                       batch_smem_bytes(n_models, lone, block));
 }
 
-cudaError_t launch_transport_batch(const TransportParams &p, int line_mode, bool j_blue, bool record,
+cudaError_t launch_transport_batch(const TransportParams &p, int line_mode, bool j_blue, bool record, bool lone,
                                    int grid, int block, cudaStream_t st) {
   void *args[] = {const_cast<TransportParams *>(&p)};
-  return cudaLaunchKernel(batch_kernel(line_mode, j_blue, record, p.n_models, block), dim3(grid), dim3(block), args,
-                          batch_smem_bytes(p.n_models, block), st);
+  return cudaLaunchKernel(batch_kernel(line_mode, j_blue, record, lone, block), dim3(grid), dim3(block), args,
+                          batch_smem_bytes(p.n_models, lone, block), st);
 }
 
 }  // namespace mcgpu

@@ -1,6 +1,9 @@
 """Walks that end soon gain nothing from running one after the other: a launch
 of many walks cut at 300 segments takes no longer in the build with lone walks
-and the pool than side by side in the build without (blocks of 256 threads)."""
+and the pool than side by side in the build without (blocks of 256 threads);
+batches of short line lists take that build with either block size, and the
+two give the same bits on both sides of the line count between them."""
+import numpy as np
 import pytest
 
 from paper_1401_5469_gb300 import synth
@@ -29,3 +32,57 @@ def test_many_short_walks_stay_side_by_side():
         b.close()
         m.close()
     assert ms[128] < 1.3 * ms[256], ms
+
+
+def _batch(mc, specs, block, reps):
+    models = [mc.Model(s, precision=mc.MC_PRECISION_MIXED) for s in specs]
+    for m in models:
+        m.set_plasma()
+    b = mc.Batch(models)
+    b.set_launch(block=block)
+    times = []
+    for _ in range(reps):
+        b.run_iteration([7 + k for k in range(len(specs))], 0, [s.n_packets for s in specs],
+                        [s.t_inner for s in specs], update=False)
+        b.synchronize()
+        times.append(b.transport_ms())
+    sums = [np.concatenate(m.estimators()[:2]) for m in models]
+    b.close()
+    for m in models:
+        m.close()
+    return min(times), sums
+
+
+def test_batches_of_short_lists_run_side_by_side():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1401_5469_gb300 import mc
+    specs = [synth.downbranch_model(n_lines=3000 + k, n_shells=12, n_packets=100_000, seed=k) for k in range(8)]
+    (t128, s128), (t256, s256) = (_batch(mc, specs, block, 8) for block in (128, 256))
+    assert t128 < 1.1 * t256, (t128, t256)  # 4.90 and 4.01 ms in the two builds
+    for a, b in zip(s128, s256):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_lines", [9_999, 10_000])
+def test_same_bits_on_both_sides_of_the_line_count(n_lines):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1401_5469_gb300 import mc
+    specs = [synth.downbranch_model(n_lines=n, n_shells=9, n_packets=3001, seed=n) for n in (2000, n_lines, 900)]
+    for a, b in zip(*(_batch(mc, specs, block, 1)[1] for block in (128, 256))):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_models", [96, 97])
+def test_same_bits_on_both_sides_of_the_model_count(n_models):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1401_5469_gb300 import mc
+    specs = [synth.downbranch_model(n_lines=12_000 if k == 5 else 1000 + 37 * (k % 9), n_shells=5 + k % 7,
+                                    n_packets=200 + 11 * k) for k in range(n_models)]
+    for a, b in zip(*(_batch(mc, specs, block, 1)[1] for block in (128, 256))):
+        assert np.array_equal(a, b)
