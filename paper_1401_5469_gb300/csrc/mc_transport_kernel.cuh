@@ -26,8 +26,8 @@
 // ms with a binary64 scan, 165 ms with the scan in binary32, 107 ms with the lone
 // walk's line-event loop, 96 ms with reciprocal and square root on the integer
 // pipe, 90 ms with fewer instructions in that loop (2.25 -> 0.95 us a segment,
-// 0.81 without J_blue; bound by the instructions of one warp, see there); its
-// 1e6-packet iteration 236 -> 105 ms (queue 9.9 -> 6.2 ms).
+// 0.81 without J_blue; bound by one warp's fixed latencies and its loads alike, see
+// there); its 1e6-packet iteration 236 -> 104 to 119 ms (queue 9.9 -> 6.2 ms).
 #pragma once
 
 #include <cstdint>
@@ -220,7 +220,9 @@ __device__ __forceinline__ int spectrum_bin(const TransportParams &p, double nu_
 // a lone walk's 32 lanes have work of their own).  Each lane loads four lines
 // ahead, and sums depths in fixed point (units of 2^-52), which takes no
 // binary64 instruction for a line; a sum that reaches 512 moves to a binary64 one
-// (a depth is not bounded, and negative ones may bring a sum back).
+// (a depth is not bounded, and negative ones may bring a sum back; the check of
+// every line takes 1e5 packets of a 1e5-line model, three v-packets a launch and a
+// cut of 30, from 65.2 to 68.0 ms; 416 when each lane flew its own launches).
 
 struct VirtualLaunch {
   double x, r2, nu_cmf, e_cmf;  // radius (units of c t_exp), its square, comoving nu and E
@@ -841,15 +843,17 @@ __global__ void __launch_bounds__(kBlock, 3) transport_fp64(const TransportParam
           // they are issued to where they are used (a copy of one where paths meet
           // would wait for it).  It leaves, with nothing changed, at a segment that
           // is anything else.
-          // What bounds it is the number of its instructions: a lone warp issues one in
-          // 4 to 5 cycles (fixed-latency stalls 3.1 of the 5.9 cycles between issues,
-          // waits for loads 0.6), 416 of them a segment before these steps.  So the
-          // segments it may take are counted out beforehand (to the next look at the
-          // clock and the stop word, the cap, 32 logged, three draws each), its counters are two, a
-          // segment's estimator terms are two shared stores, and the J_blue terms of
-          // the lines passed one atomic of the lanes.  A walk of 94,495 segments alone:
-          // 100.4 -> 76.7 ms, with J_blue (and its zeroing, which leaves the caches
-          // cold) 96.0 -> 89.8; 5e4 lines, 1e5 packets: 32.6 -> 25.5 ms.
+          // What bounded it was the number of its instructions (a lone warp issued
+          // one in 5.9 cycles, 3.1 of them fixed latencies and 0.6 waits for loads; 416 a
+          // segment).  So the segments it may take are counted out beforehand (to the
+          // next look at the clock and the stop word, the cap, 32 logged, three draws
+          // each), its counters are two, a segment's estimator terms are two shared
+          // stores, and the J_blue terms of the lines passed one atomic of the lanes:
+          // 361 a segment, and of the cycles between two 2.4 are fixed latencies, 1.1
+          // shuffles, conversions and binary64, and 2.3 waits for the two dependent
+          // loads, which the instructions no longer cover.  A walk of 94,495 segments
+          // alone: 100.4 -> 76.0 ms, with J_blue (and its zeroing, which leaves the
+          // caches cold) 96.0 -> 89.8; 5e4 lines, 1e5 packets: 32.6 -> 25.5 ms.
           bool certain = true;
           while (certain) {
             if (n_log == 32u) sum_log();

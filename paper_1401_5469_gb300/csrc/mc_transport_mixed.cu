@@ -314,13 +314,13 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
   const unsigned long long n_warps = static_cast<unsigned long long>(gridDim.x) * (blockDim.x >> 5);
   const unsigned quota = static_cast<unsigned>(min(32ull, (p.n_packets + n_warps - 1ull) / n_warps));
   bool alive = false, finished = lane >= quota;
-  // Lone-walker mode (single-model build): once the packet queue is empty and
-  // a warp is down to one live walk, every lane takes that walk's state and
-  // runs its segments with the owner lane, as in the binary64 kernel: the
-  // lanes load the line list 32 lines at a time in one coalesced load (line
-  // lwin_j0 + lane in each lane), scan the window in one step, compute the
-  // walk's draws 64 at a time into a per-warp shared buffer, and only the
-  // owner lane makes the walk's side effects.
+  // Lone walks (kLoneBuild): once the packet queue is empty and few walks of a
+  // warp are left, or a walk comes from the pool, every lane takes one walk's
+  // state and runs its segments, as in the binary64 kernel: the lanes load the
+  // line list 32 lines at a time in one coalesced load (line lwin_j0 + lane in
+  // each lane), scan the window in one step, compute the walk's draws 64 at a
+  // time into a per-warp shared buffer, and only lane 0 makes the walk's side
+  // effects.
   WarpDraws wd;
   unsigned long long *warp_mem =
       smem_u64 + (batch ? static_cast<size_t>(p.n_models) + 1 : 2 * static_cast<size_t>(p.S)) +
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
   // the lane's current shell and its constants (reloaded on a shell or model change)
   int32_t cs = -1;
   float c_kap = 0.0f, c_ikap = 0.0f, c_xi2 = 0.0f, c_xo2 = 0.0f;
-  // single-model build: lines next_line, next_line + 1 of the next segment,
+  // MINB == 1: lines next_line, next_line + 1 of the next segment,
   // loaded by the event that began it (see the binary64 kernel)
   bool lw_ok = false;
   long long lw_b0 = 0, lw_b1 = 0;
@@ -1058,7 +1058,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 128 : kMaxBlock, MINB == 1 ? 3 : M
         pk.have_inv_D = true;
       }
     }
-    if (status != 0 && !act) {  // lone mode, not the owner lane: drop the adopted walk
+    if (status != 0 && !act) {  // a lone walk, not lane 0: drop it
       alive = false;
       lone = false;
       acc_s = -1;
