@@ -73,7 +73,7 @@ TRAFFIC_CAPTURE = {
     "dram_bytes_per_launch": 604.93e6 + 112.88e6,
     "sources": ("paper_1401_5469_gb300/csrc/mc_transport.cu", "paper_1401_5469_gb300/csrc/mc_transport_kernel.cuh",
                 "paper_1401_5469_gb300/csrc/mc_device.cuh", "paper_1401_5469_gb300/csrc/mc_internal.h"),
-    "sha256": "87e469a89077ead90a019e3fbf2f3cbe738eb70108c40628d3cdfd520552c6c0",
+    "sha256": "43ba5359bca38d4b425767e9bd182f0fca81386cd2c65c7e40b614acacc9e238",
 }
 
 

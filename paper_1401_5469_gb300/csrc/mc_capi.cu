@@ -541,13 +541,14 @@ mc_status mc_model_create(const mc_geometry_desc *geom, const mc_line_desc *line
   }
   int bps = 0;
   e = transport_occupancy(run->line_mode, run->precision, run->j_blue != 0, run->record_packets != 0,
-                          m->dbr_rec != nullptr, static_cast<int>(S), &bps);
+                          m->dbr_rec != nullptr, static_cast<int>(S), static_cast<int>(L), &bps);
   if (e != cudaSuccess || bps <= 0) return bail(MC_ERR_CUDA, "transport occupancy query failed");
   int nsm = 1;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
   m->grid = nsm * bps;
   // the pool: every warp of the grid hands over at most kPoolLive - 1 walks, once
-  m->pool_cap = static_cast<uint32_t>(m->grid) * static_cast<uint32_t>(transport_block_size() / 32) * (kPoolLive - 1u);
+  if (run->precision != MC_PRECISION_MIXED || mixed_lone(run->line_mode, static_cast<int>(L)))
+    m->pool_cap = static_cast<uint32_t>(m->grid) * static_cast<uint32_t>(transport_block_size() / 32) * (kPoolLive - 1u);
   m->n_counter_words = kNCounterSlots + 2 + (static_cast<size_t>(m->pool_cap) + 1) / 2;
   // (a mixed-precision model's own is allocated by its first run by itself: batches
   // have one of theirs)
@@ -629,7 +630,7 @@ mc_status mc_run_iteration_range(mc_model *m, uint64_t seed, uint32_t iteration,
   if (!(t_inner > 0.0) || !std::isfinite(t_inner)) return fail(m, MC_ERR_INVALID_ARG, "t_inner must be positive");
   if (m->in_batch) return fail(m, MC_ERR_INVALID_ARG, "the model belongs to a batch; run it through the batch");
   m->spread = n_packets >= kSpreadPackets;
-  if (!m->pool) alloc_n(m, &m->pool, m->pool_cap);  // (without one walks stay in their warps)
+  if (!m->pool && m->pool_cap) alloc_n(m, &m->pool, m->pool_cap);  // (without one walks stay in their warps)
   mc_status st = model_prepare(m, m->stream, true);
   if (st != MC_OK) return st;
   TransportParams p{};

@@ -217,9 +217,10 @@ cudaError_t launch_transport(const TransportParams &p, int line_mode, int precis
                              bool record, int grid, int block, cudaStream_t st);
 int transport_block_size();
 // tables: the branching rows have bucket slots (a model's; not the caller-owned table's)
-cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, bool tables, int S,
+cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, bool tables, int S, int L,
                                 int *blocks_per_sm);
-const void *select_mixed_kernel(int line_mode, bool j_blue, bool record);
+bool mixed_lone(int line_mode, int L);  // a single mixed model's launches run lone walks
+const void *select_mixed_kernel(int line_mode, bool j_blue, bool record, int L);
 const void *select_virtual_kernel(int line_mode, bool j_blue, bool record);  // binary64, with v-packets
 // Batched launches: `block` threads per block (64, 128 or 256); lone: with 128,
 // the build with lone walks and the pool (batch_lone: worth it for such a batch).

@@ -215,7 +215,7 @@ extern "C" mc_status mc_transport_noalloc(const mc_noalloc_args *a, void *stream
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   e = transport_occupancy(a->line_mode, MC_PRECISION_FP64, a->j_blue != nullptr, false,
-                          false, static_cast<int>(S), &bps);
+                          false, static_cast<int>(S), static_cast<int>(L), &bps);
   if (e != cudaSuccess || bps <= 0) {
     set_create_error("mc_transport_noalloc: occupancy query failed");
     return MC_ERR_CUDA;

@@ -7,8 +7,8 @@ namespace mcgpu {
 namespace {
 
 // tables: the model's branching tables (bucket slots) are there
-const void *select_kernel(int line_mode, int precision, bool jb, bool rec, bool tables, bool virt) {
-  if (precision == 1) return select_mixed_kernel(line_mode, jb, rec);
+const void *select_kernel(int line_mode, int precision, bool jb, bool rec, bool tables, bool virt, int L) {
+  if (precision == 1) return select_mixed_kernel(line_mode, jb, rec, L);
   if (virt) return select_virtual_kernel(line_mode, jb, rec);
   if (line_mode == 0) return select_lines<0, false>(jb, rec);
   if (line_mode == 2) return select_lines<2, false>(jb, rec);
@@ -28,9 +28,9 @@ size_t smem_bytes(int S, int precision, bool virt) {
 
 int transport_block_size() { return kBlock; }
 
-cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, bool tables, int S,
+cudaError_t transport_occupancy(int line_mode, int precision, bool j_blue, bool record, bool tables, int S, int L,
                                 int *blocks_per_sm) {
-  const void *k = select_kernel(line_mode, precision, j_blue, record, tables, false);
+  const void *k = select_kernel(line_mode, precision, j_blue, record, tables, false, L);
   const size_t smem = smem_bytes(S, precision, false);
   if (smem > 48 * 1024) {  // the query, like the launch, needs the opt-in above 48 KB
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -45,7 +45,7 @@ cudaError_t launch_transport(const TransportParams &p, int line_mode, int precis
   // the shared-memory layout (one draw buffer per warp) is sized for kBlock
   if (block != kBlock) return cudaErrorInvalidValue;
   const bool virt = p.n_virtual > 0;
-  const void *k = select_kernel(line_mode, precision, j_blue, record, p.dbr_rec != nullptr, virt);
+  const void *k = select_kernel(line_mode, precision, j_blue, record, p.dbr_rec != nullptr, virt, p.L);
   const size_t smem = smem_bytes(p.S, precision, virt);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -273,8 +273,8 @@ __device__ __forceinline__ PoolWalk pack_walk(const PacketM &pk, uint32_t d, int
 // model's results do not depend on the company it is launched in.  It is
 // compiled twice: MINB = 1 (blocks of 128 threads, three per SM at up to 168
 // registers, with lone walks) for single models and for batches of 128
-// threads a block, and MINB = 2 for batches of 64 or 256 threads, of many models
-// or of short line lists (128 registers: 16 resident warps per SM, without lone walks).  A batch of 12
+// threads a block, and MINB = 2 for batches of 64 or 256 threads or of many models,
+// and for short line lists (128 registers: 16 resident warps per SM, without lone walks).  A batch of 12
 // uneven models (2.9e6 packets): 330 ms a launch with the second (26 ms until
 // the queue is empty, then the longest walks at 2.5 us a segment), 209 ms with
 // the first (34 ms, and 1.3 us), 185 since the lone loop takes fewer
@@ -1130,7 +1130,17 @@ const void *select_b(int line_mode, bool jb, bool rec) { return select_m<2>(line
 
 }  // namespace
 
-const void *select_mixed_kernel(int line_mode, bool jb, bool rec) { return select_m<1>(line_mode, jb, rec); }
+// A single model's launches take the build with lone walks, except through
+// downbranch or macro-atom lists below kLoneLinesSingle lines: 20 shells, 2000 lines,
+// ms with it and without: 2000 packets 0.65 and 0.47, 2e4 0.87 and 0.69, 1e6 5.24 and 4.49;
+// 5000 lines 1.31 and 1.13, 1.87 and 1.59, 8.43 and 7.44; 12 shells, 9000 lines 1.64 and
+// 1.95, 2.92 and 3.04, 11.1 and 10.4; 15,000 lines 5.7 and 9.0, 6.8 and 9.9, 20.7 and 21.6.
+// (Scattering lists: 2000 lines 1e6 packets 2.71 and 2.95, 12,347 lines 5.1 and 4.9.)
+constexpr int kLoneLinesSingle = 6'000;
+bool mixed_lone(int line_mode, int L) { return line_mode == 0 || L >= kLoneLinesSingle; }
+const void *select_mixed_kernel(int line_mode, bool jb, bool rec, int L) {
+  return mixed_lone(line_mode, L) ? select_m<1>(line_mode, jb, rec) : select_b(line_mode, jb, rec);
+}
 
 // single-model launches (128 threads): shell tables, then per warp a walk
 // handed to all lanes and the lone walk's draw buffer

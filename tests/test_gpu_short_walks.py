@@ -86,3 +86,38 @@ def test_same_bits_on_both_sides_of_the_model_count(n_models):
                                     n_packets=200 + 11 * k) for k in range(n_models)]
     for a, b in zip(*(_batch(mc, specs, block, 1)[1] for block in (128, 256))):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("line_mode,n_lines", [(1, 2000), (1, 5_999), (1, 6_000), (2, 5_999), (2, 6_000)])
+def test_single_models_of_short_lists_run_side_by_side(line_mode, n_lines):
+    """A model by itself against blocks of 256 threads: the same bits on both
+    sides of its own line count, and with a short list (0.87 and 0.69 ms in the
+    two builds) about the same time."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1401_5469_gb300 import mc
+    make = synth.downbranch_model if line_mode == 1 else synth.macroatom_model
+    spec = make(n_lines=n_lines, n_shells=20, n_packets=20_000)
+    m = mc.Model(spec, precision=mc.MC_PRECISION_MIXED, record_packets=True)
+    m.set_plasma()
+    times = []
+    for _ in range(10):
+        m.run_iteration(7, 0, spec.n_packets, spec.t_inner)
+        m.synchronize()
+        times.append(sum(m.phases()[:2]))
+    runs = [(*m.packets(0, spec.n_packets), *m.estimators()[:2])]
+    b = mc.Batch([m])
+    b.set_launch(block=256)
+    batch_times = []
+    for _ in range(10):
+        b.run_iteration([7], 0, [spec.n_packets], [spec.t_inner], update=False)
+        b.synchronize()
+        batch_times.append(b.transport_ms())
+    runs.append((*m.packets(0, spec.n_packets), *m.estimators()[:2]))
+    b.close()
+    m.close()
+    for x, y in zip(*runs):
+        assert np.array_equal(x, y)
+    if n_lines == 2000:
+        assert min(times) < 1.12 * min(batch_times), (min(times), min(batch_times))
